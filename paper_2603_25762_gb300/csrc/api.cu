@@ -123,7 +123,8 @@ struct SolveBufs {
 qh_status run_step(Ctx* ctx, const Graph& g, int precision, const TcPlan& plan, StepArgs a,
                    const float* x_cur_f32, float* x_next_f32, const __nv_bfloat16* xh_cur,
                    __nv_bfloat16* xh_next, const Fp8Operands* f8 = nullptr, int64_t ns = 0,
-                   float* zband = nullptr) {
+                   float* zband = nullptr, const F32Chunks& f32 = F32Chunks(),
+                   bool after_step = false) {
   if (precision == QH_PREC_FP8) {  // X_hat buffers hold the e4m3 hi part, then the lo part
     Fp8Operands op = *f8;
     op.xh_in = reinterpret_cast<const uint8_t*>(xh_cur);
@@ -138,7 +139,7 @@ qh_status run_step(Ctx* ctx, const Graph& g, int precision, const TcPlan& plan, 
     if (g.csr_mode)
       launch_step_csr(ctx->stream, g, a, g.pval, nullptr, plan.variant);
     else
-      launch_step_f32(ctx->stream, g, a);
+      return launch_step_f32(ctx, g, a, f32, after_step);
     return QH_OK;
   }
   a.xh_out = xh_next;
@@ -769,6 +770,11 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
   B.cut_z = tc_cut ? (float*)ctx->scratch(NS * 4, S_CUTS_Z) : nullptr;
   if (tc_cut && (!B.cut_s || !B.cut_z))
     return set_err(ctx, QH_ENOMEM, "allocation failed (tensor-core cuts)");
+  F32Chunks f32;
+  if (o->precision == QH_PREC_FP32 && !G.csr_mode) {
+    qh_status st = f32_prepare(ctx, G, W.tile_f32, o->sb_variant, &f32);
+    if (st != QH_OK) return st;
+  }
   // ---- the step loop, captured once per shape and replayed
   // The captured step loop bakes in pointers and sizes; it is replayed only when every
   // one of them is unchanged (a rebuilt graph at other addresses is captured anew).
@@ -803,7 +809,8 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
                           (const void*)B.running, (const void*)B.steps_b, (const void*)B.c0,
                           (const void*)B.seen, (const void*)B.stall, (const void*)B.steps_run,
                           (const void*)ctx->d_err, (const void*)B.deform, (const void*)B.trace,
-                          (const void*)B.cut_s, (const void*)B.cut_z})
+                          (const void*)B.cut_s, (const void*)B.cut_z,
+                          (const void*)f32.list, (const void*)f32.count})
       add(p);
   }
   StepArgs a{};
@@ -924,12 +931,16 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
     QH_STAGE_CHECK("solve: before step-loop capture");
     QH_CUDA_TRY(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     qh_status st = QH_OK;
+    bool after_step = false;  // the launch before is another step
     for (int32_t t = 0; t < max_steps && st == QH_OK; ++t) {
       a.t = t;
       const bool even = (t % 2) == 0;
       st = run_step(ctx, W, o->precision, tplan, a, even ? B.x : B.x1, even ? B.x1 : B.x,
-                    even ? B.xh0 : B.xh1, even ? B.xh1 : B.xh0, &f8, (int64_t)NS, B.zband);
+                    even ? B.xh0 : B.xh1, even ? B.xh1 : B.xh0, &f8, (int64_t)NS, B.zband,
+                    f32, after_step);
+      after_step = true;
       if (checking && (t + 1) % o->check_every == 0 && t + 1 < max_steps) {
+        after_step = false;
         const float* xc = (o->precision == QH_PREC_FP32 && even) ? B.x1 : B.x;
         if (st == QH_OK) st = replica_cuts(xc, B.running);
         launch_pick_best(s, nb, R, B.cuts, B.best_r, B.best_cut, B.running);
@@ -1628,7 +1639,10 @@ qh_status qh_debug_matvec(qh_ctx* h, const qh_graph* gh, int32_t precision, int3
   } else if (precision == QH_PREC_FP32) {
     a.xin = x;
     a.xout = nullptr;
-    launch_step_f32(ctx->stream, g, a);
+    F32Chunks ch;
+    st = f32_prepare(ctx, g, g.tile_f32, QH_SB_BALLISTIC, &ch);
+    if (st == QH_OK) st = launch_step_f32(ctx, g, a, ch, false);
+    if (st) return st;
   } else {
     __nv_bfloat16* xh = (__nv_bfloat16*)ctx->scratch((size_t)R * g.n_pad * 2, S_XH0);
     if (!xh) return set_err(ctx, QH_ENOMEM, "allocation failed (debug)");
@@ -1708,6 +1722,9 @@ qh_status qh_debug_steps_v(qh_ctx* h, const qh_graph* gh, int32_t precision, int
     float* x1 = (float*)ctx->scratch(NS * 4, S_X1);
     if (!x1) return set_err(ctx, QH_ENOMEM, "allocation failed (debug)");
     QH_CUDA_TRY(cudaMemcpyAsync(x1, x, NS * 4, cudaMemcpyDeviceToDevice, s));
+    F32Chunks ch;
+    if (!g.csr_mode) st = f32_prepare(ctx, g, g.tile_f32, sb_variant, &ch);
+    if (st) return st;
     for (int32_t k = 0; k < nsteps; ++k) {
       a.t = t0 + k;
       a.xin = (k % 2 == 0) ? x : x1;
@@ -1715,7 +1732,8 @@ qh_status qh_debug_steps_v(qh_ctx* h, const qh_graph* gh, int32_t precision, int
       if (g.csr_mode)
         launch_step_csr(s, g, a, g.pval, nullptr, csr_v);
       else
-        launch_step_f32(s, g, a);
+        st = launch_step_f32(ctx, g, a, ch, k > 0);
+      if (st) return st;
     }
     if (nsteps % 2 == 1) QH_CUDA_TRY(cudaMemcpyAsync(x, x1, NS * 4, cudaMemcpyDeviceToDevice, s));
   } else {

@@ -53,100 +53,314 @@ __global__ void k_x_to_sign_bf16(const float* __restrict__ x, __nv_bfloat16* xh,
 }
 
 // ------------------------------------------------------------------ FP32 step
-constexpr int F_RT = 64;   // replicas per CTA
-constexpr int F_KC = 32;   // K chunk staged in shared memory
+// The FP32 product walks only the 8-column chunks of J that hold a nonzero for a group of
+// 32 rows.  Row graphs are banded at a finer grain than the 128 x 128 tiles: on the
+// hifi-region graph a 32-row group meets about 19 of the 48 chunks of its three tiles.
+// Zero entries contribute fma(0, x, acc) = acc for a finite x, so leaving their chunks
+// out changes no bit; adiabatic SB has no walls, its x may overflow, and it walks every
+// chunk (F32Chunks::all).
+constexpr int F_ROWS = 32;             // rows of a group
+constexpr int F_COLS = 8;              // columns of a chunk: one 32-byte sector of x
+constexpr int F_TILE_CHUNKS = TILE / F_COLS;
+constexpr int F_GROUPS = TILE / F_ROWS;
+constexpr int F_STAGE_CHUNKS = 4;      // chunks per pipeline stage
+constexpr int F_KC = F_COLS * F_STAGE_CHUNKS;
+constexpr int F_STAGES = 3;
+constexpr int F_QUADS = F_KC / 4;      // 16-byte pieces of a staged row
+// Position of piece q of a staged row: row groups (J) and replicas (x) that a warp reads
+// at once fall into distinct banks.
+__device__ __forceinline__ int f32_jpos(int row, int q) { return (q ^ ((row >> 3) & 3)) * 4; }
+__device__ __forceinline__ int f32_xpos(int rep, int q) { return (q ^ (rep & 7)) * 4; }
 
-__global__ void __launch_bounds__(256) k_step_f32(StepArgs a) {
-  const int32_t t = a.t;
-  const double a0d = a.a0;
-  __shared__ __align__(16) float Js[F_KC][TILE + 4];
-  __shared__ __align__(16) float Xs[F_KC][F_RT + 4];
-  const RowTile rt = a.rt[blockIdx.x];
-  const int tid = threadIdx.x, lane = tid & 31, wg = tid >> 5;
-  const int32_t r0 = blockIdx.y * F_RT;
+// Chunk lists: CTA per row tile.  Group g's list starts at entry f32_begin * 64 +
+// g * 16 * n_hi, columns ascending: .x = offset of the chunk's first column in the FP32
+// tiles (in units of 8 floats), .y = its first padded column.
+__global__ void __launch_bounds__(256) k_f32_chunks(const RowTile* __restrict__ rts,
+                                                    const int32_t* __restrict__ tile_col,
+                                                    const float* __restrict__ tile_f32, int all,
+                                                    int2* __restrict__ list,
+                                                    int32_t* __restrict__ count) {
+  __shared__ uint32_t part[8];
+  const RowTile rt = rts[blockIdx.x];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int32_t n = 0;  // warps 0 .. 3: entries of group `warp` so far
+  int2* out = list + (int64_t)rt.f32_begin * (F_GROUPS * F_TILE_CHUNKS) +
+              (int64_t)(warp & 3) * F_TILE_CHUNKS * rt.n_hi;
+  for (int32_t e = 0; e < rt.n_hi; ++e) {
+    // warp w looks at rows 16 w .. 16 w + 15, lane l at columns 4 l .. 4 l + 3
+    const float4* src = reinterpret_cast<const float4*>(
+        tile_f32 + (int64_t)(rt.f32_begin + e) * (TILE * TILE) + warp * 16 * TILE) + lane;
+    bool nz = false;
+    if (!all) {
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        const float4 v = src[r * (TILE / 4)];
+        nz |= v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f;
+      }
+    }
+    const uint32_t m = all ? 0xffffffffu : __ballot_sync(0xffffffffu, nz);
+    if (lane == 0) part[warp] = m;
+    __syncthreads();
+    if (warp < F_GROUPS) {
+      const uint32_t both = part[2 * warp] | part[2 * warp + 1];
+      const bool on = lane < F_TILE_CHUNKS && ((both >> (2 * lane)) & 3u) != 0;
+      const uint32_t mask = __ballot_sync(0xffffffffu, on);
+      if (on)
+        out[n + __popc(mask & ((1u << lane) - 1u))] =
+            make_int2((rt.f32_begin + e) * (TILE * TILE / F_COLS) + lane,
+                      tile_col[rt.tile_begin + e] * TILE + lane * F_COLS);
+      n += __popc(mask);
+    }
+    __syncthreads();
+  }
+  if (warp < F_GROUPS && lane == 0) count[blockIdx.x * F_GROUPS + warp] = n;
+}
+
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(smem)),
+               "l"(gmem)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+// Programmatic dependent launch: wait until the kernel before this one in the stream has
+// completed (its writes are visible), and let the next one start its prologue.
+__device__ __forceinline__ void grid_dep_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dep_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// One FP32 step of a 32-row group for 8 RPT NW replicas.  A warp covers the 32 rows x
+// 8 RPT replicas, a thread 8 rows x RPT replicas: per 4 columns it reads 8 + RPT 16-byte
+// operands from shared memory for 32 RPT FMAs.  J and x chunks come through a three-stage
+// cp.async ring, both with their columns contiguous (no transpose); the XOR swizzles put
+// the 4 row groups (8 replicas) that a warp reads at once into distinct banks.  Every
+// output sums its columns in ascending order with one FMA each.  The rows' list and J do
+// not depend on the step before: they are fetched ahead of the grid dependency.
+// Bound by the latency of the operand copies at 12 warps per SM (ncu on hifi-region,
+// R = 1,024: issue slots 51 % busy, FMA pipe 34 %, DRAM under 25 %).  Stages of 2 chunks
+// (more CTAs per SM, twice the barriers) measured slower: 66 against 61 us per step there
+// with four of them, 85 against 69 on ont-like 3,000 SNPs at R = 512.  Microseconds per
+// step, the dense 128 x 64 tile product before -> now: 300 SNPs / 80 reads, R = 32:
+// 20.4 -> 2.9; 720 reads, R = 256: 49.7 -> 7.4; 7,200 reads, R = 256: 64.7 -> 17.9 and
+// R = 1,024: 192 -> 61; 12,000-SNP graph (468 neighbours), R = 128: 146 -> 63 and
+// R = 512: 349 -> 179.
+template <int RPT, int NW, bool DISC>
+__global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __restrict__ list,
+                                                      const int32_t* __restrict__ count,
+                                                      int vec4) {
+  constexpr int RC = 8 * RPT * NW, NT = 32 * NW;
+  extern __shared__ __align__(128) float f32_smem[];
+  float* const js = f32_smem;                               // [F_STAGES][32 rows][32]
+  float* const xs = f32_smem + F_STAGES * F_ROWS * F_KC;    // [F_STAGES][RC][32]
+  __shared__ float coef_s;
+  const int32_t rti = blockIdx.x / F_GROUPS, grp = blockIdx.x % F_GROUPS;
+  const RowTile rt = a.rt[rti];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rl = lane & 3, pl = lane >> 2;
+  const int32_t r0 = blockIdx.y * RC;
+  const int32_t vrows = rt.valid - grp * F_ROWS;  // real rows of this group
+  if (vrows <= 0) return;
   const int32_t sb = a.steps_b[rt.block];
-  const bool live = (a.active == nullptr || a.active[rt.block]) && t < sb;
+  if (tid == 0) {
+    const double at = a.a0 * (double)a.t / (double)sb;
+    coef_s = (float)(-(a.a0 - at));
+  }
+  const int32_t nc = count[blockIdx.x];
+  const int32_t ns = (nc + F_STAGE_CHUNKS - 1) / F_STAGE_CHUNKS;
+  const int2* lst = list + (int64_t)rt.f32_begin * (F_GROUPS * F_TILE_CHUNKS) +
+                    (int64_t)grp * F_TILE_CHUNKS * rt.n_hi;
+  // this thread copies quad q (4 of the stage's 32 columns) of some rows and replicas
+  const int q = tid % F_QUADS, qr = tid / F_QUADS, c_of = q >> 1, c_in = (q & 1) * 4;
+  auto entry = [&](int32_t st) -> int2 {
+    const int32_t c = st * F_STAGE_CHUNKS + c_of;
+    return c < nc ? lst[c] : make_int2(-1, 0);
+  };
+  auto load_j = [&](int32_t st, int2 en) {
+    if (en.x < 0) return;
+    float* dst = js + (st % F_STAGES) * (F_ROWS * F_KC);
+    const float* src = a.tile_f32 + (int64_t)en.x * F_COLS + (grp * F_ROWS) * TILE + c_in;
+#pragma unroll
+    for (int i = 0; i < F_ROWS * F_QUADS / NT; ++i) {
+      const int row = qr + i * (NT / F_QUADS);
+      cp_async16(dst + row * F_KC + f32_jpos(row, q), src + row * TILE);
+    }
+  };
+  auto load_x = [&](int32_t st, int2 en) {
+    if (en.x < 0) return;
+    float* dst = xs + (st % F_STAGES) * (RC * F_KC);
+    const float* src = a.xin + en.y + c_in;
+#pragma unroll
+    for (int i = 0; i < RC * F_QUADS / NT; ++i) {
+      const int rep = qr + i * (NT / F_QUADS);
+      const int32_t r = min(r0 + rep, a.R - 1);  // past the last replica: any valid row
+      cp_async16(dst + rep * F_KC + f32_xpos(rep, q), src + (int64_t)r * a.n_pad);
+    }
+  };
+  int2 en[F_STAGES];
+#pragma unroll
+  for (int i = 0; i < F_STAGES; ++i) en[i] = entry(i);
+#pragma unroll
+  for (int i = 0; i < F_STAGES - 1; ++i) load_j(i, en[i]);
+  grid_dep_wait();
+  grid_dep_launch();
+  const bool live = (a.active == nullptr || a.active[rt.block]) && a.t < sb;
+  const int32_t row0 = rt.row0 + grp * F_ROWS;
   if (!live) {
-    if (a.z_out == nullptr && a.xout != a.xin) {  // carry a frozen block to the next buffer
-      for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 8; ++j) {
-          int32_t row = lane + 32 * i, r = r0 + wg * 8 + j;
-          if (row < rt.valid && r < a.R) {
-            size_t idx = (size_t)r * a.n_pad + rt.row0 + row;
-            a.xout[idx] = a.xin[idx];
-          }
+    cp_async_wait<0>();
+    if (a.z_out == nullptr && a.xout != a.xin)  // carry a frozen block to the next buffer
+      for (int i = tid; i < RC * F_ROWS; i += NT) {
+        const int32_t r = r0 + i / F_ROWS, row = i % F_ROWS;
+        if (r < a.R && row < vrows)
+          a.xout[(size_t)r * a.n_pad + row0 + row] = a.xin[(size_t)r * a.n_pad + row0 + row];
+      }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < F_STAGES - 1; ++i) {
+    load_x(i, en[i]);
+    cp_async_commit();
+  }
+  int2 nxt = en[F_STAGES - 1];
+  float acc[RPT][8];
+#pragma unroll
+  for (int j = 0; j < RPT; ++j)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[j][i] = 0.f;
+  for (int32_t st = 0; st < ns; ++st) {
+    cp_async_wait<F_STAGES - 2>();
+    __syncthreads();  // stage st has landed; stage st - 1's buffers are free
+    load_j(st + F_STAGES - 1, nxt);
+    load_x(st + F_STAGES - 1, nxt);
+    cp_async_commit();
+    nxt = entry(st + F_STAGES);
+    const float* jb = js + (st % F_STAGES) * (F_ROWS * F_KC) + rl * 8 * F_KC;
+    const float* xb = xs + (st % F_STAGES) * (RC * F_KC) + (warp * 8 * RPT + pl) * F_KC;
+    const int nq = 2 * min(F_STAGE_CHUNKS, nc - st * F_STAGE_CHUNKS);
+#pragma unroll 2
+    for (int k = 0; k < nq; ++k) {
+      float4 jv[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        jv[i] = *reinterpret_cast<const float4*>(jb + i * F_KC + f32_jpos(rl * 8, k));
+#pragma unroll
+      for (int j = 0; j < RPT; ++j) {
+        float4 v = *reinterpret_cast<const float4*>(xb + j * 8 * F_KC + f32_xpos(pl, k));
+        if (DISC)  // J sgn(x); padding columns meet zero columns of J
+          v = make_float4(sb_operand(QH_SB_DISCRETE, v.x), sb_operand(QH_SB_DISCRETE, v.y),
+                          sb_operand(QH_SB_DISCRETE, v.z), sb_operand(QH_SB_DISCRETE, v.w));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[j][i] = fmaf(jv[i].x, v.x, acc[j][i]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[j][i] = fmaf(jv[i].y, v.y, acc[j][i]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[j][i] = fmaf(jv[i].z, v.z, acc[j][i]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[j][i] = fmaf(jv[i].w, v.w, acc[j][i]);
+      }
+    }
+  }
+  cp_async_wait<0>();
+  __syncthreads();  // coef_s (a list may be empty)
+  const float coef_x = coef_s;
+  const float c0 = a.c0[rt.block];
+  const float fe = deform_force(a.deform, rt.block, a.t, sb);
+  auto index = [&](int j) -> size_t {
+    return (size_t)(r0 + warp * 8 * RPT + pl + 8 * j) * a.n_pad + row0 + rl * 8;
+  };
+  if (vec4 && a.z_out == nullptr) {
+    // rows past the block keep what they hold (zeros); x and y of the next replica load
+    // while this one's are updated
+    float4 xn[2], yn[2];
+    auto fetch = [&](int j) {
+      if (r0 + warp * 8 * RPT + pl + 8 * j >= a.R) return;
+      const size_t idx = index(j);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        xn[h] = *reinterpret_cast<const float4*>(a.xin + idx + 4 * h);
+        yn[h] = *reinterpret_cast<const float4*>(a.y + idx + 4 * h);
+      }
+    };
+    fetch(0);
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) {
+      const float4 x4[2] = {xn[0], xn[1]}, y4[2] = {yn[0], yn[1]};
+      if (j + 1 < RPT) fetch(j + 1);
+      if (r0 + warp * 8 * RPT + pl + 8 * j >= a.R) continue;
+      const size_t idx = index(j);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float xv[4] = {x4[h].x, x4[h].y, x4[h].z, x4[h].w};
+        float yv[4] = {y4[h].x, y4[h].y, y4[h].z, y4[h].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float x = xv[i], y = yv[i];
+          sb_update(a.sb, acc[j][4 * h + i], x, y, a.dt, coef_x, a.dta0, c0, fe);
+          const bool real = rl * 8 + 4 * h + i < vrows;
+          xv[i] = real ? x : xv[i];
+          yv[i] = real ? y : yv[i];
         }
+        *reinterpret_cast<float4*>(a.xout + idx + 4 * h) = make_float4(xv[0], xv[1], xv[2], xv[3]);
+        *reinterpret_cast<float4*>(a.y + idx + 4 * h) = make_float4(yv[0], yv[1], yv[2], yv[3]);
+      }
     }
     return;
   }
-  float acc[4][8];
+#pragma unroll 1
+  for (int i = 0; i < 8 * RPT; ++i) {  // the product alone (z_out), or unaligned buffers
+    const int j = i >> 3;
+    float z = 0.f;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-  for (int32_t e = 0; e < rt.n_hi; ++e) {
-    const float* Jt = a.tile_f32 + (size_t)(rt.f32_begin + e) * (TILE * TILE);
-    const int32_t cbase = a.tile_col[rt.tile_begin + e] * TILE;
-    for (int kc = 0; kc < TILE; kc += F_KC) {
-      for (int idx = tid; idx < TILE * (F_KC / 4); idx += 256) {
-        int row = idx / (F_KC / 4), k4 = idx % (F_KC / 4);
-        float4 v = *reinterpret_cast<const float4*>(Jt + (size_t)row * TILE + kc + k4 * 4);
-        Js[k4 * 4 + 0][row] = v.x;
-        Js[k4 * 4 + 1][row] = v.y;
-        Js[k4 * 4 + 2][row] = v.z;
-        Js[k4 * 4 + 3][row] = v.w;
-      }
-      for (int idx = tid; idx < F_RT * (F_KC / 4); idx += 256) {
-        int rep = idx / (F_KC / 4), k4 = idx % (F_KC / 4);
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r0 + rep < a.R)
-          v = *reinterpret_cast<const float4*>(a.xin + (size_t)(r0 + rep) * a.n_pad + cbase + kc +
-                                               k4 * 4);
-        if (a.sb == QH_SB_DISCRETE)  // J sgn(x); padding columns meet zero columns of J
-          v = make_float4(sb_operand(a.sb, v.x), sb_operand(a.sb, v.y), sb_operand(a.sb, v.z),
-                          sb_operand(a.sb, v.w));
-        Xs[k4 * 4 + 0][rep] = v.x;
-        Xs[k4 * 4 + 1][rep] = v.y;
-        Xs[k4 * 4 + 2][rep] = v.z;
-        Xs[k4 * 4 + 3][rep] = v.w;
-      }
-      __syncthreads();
-#pragma unroll 8
-      for (int k = 0; k < F_KC; ++k) {
-        float av[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) av[i] = Js[k][lane + 32 * i];
-        float4 b0 = *reinterpret_cast<const float4*>(&Xs[k][wg * 8]);
-        float4 b1 = *reinterpret_cast<const float4*>(&Xs[k][wg * 8 + 4]);
-        float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-      }
-      __syncthreads();
+    for (int m = 0; m < 8 * RPT; ++m) z = m == i ? acc[m >> 3][m & 7] : z;
+    if (rl * 8 + (i & 7) >= vrows || r0 + warp * 8 * RPT + pl + 8 * j >= a.R) continue;
+    const size_t idx = index(j) + (i & 7);
+    if (a.z_out != nullptr) {
+      a.z_out[idx] = z;
+      continue;
     }
+    float x = a.xin[idx], y = a.y[idx];
+    sb_update(a.sb, z, x, y, a.dt, coef_x, a.dta0, c0, fe);
+    a.xout[idx] = x;
+    a.y[idx] = y;
   }
-  const double at = a0d * (double)t / (double)sb;
-  const float coef_x = (float)(-(a0d - at));
-  const float c0 = a.c0[rt.block];
-  const float fe = deform_force(a.deform, rt.block, a.t, a.steps_b[rt.block]);
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      int32_t row = lane + 32 * i, r = r0 + wg * 8 + j;
-      if (row >= rt.valid || r >= a.R) continue;
-      size_t idx = (size_t)r * a.n_pad + rt.row0 + row;
-      if (a.z_out != nullptr) {
-        a.z_out[idx] = acc[i][j];
-        continue;
-      }
-      float x = a.xin[idx], y = a.y[idx];
-      sb_update(a.sb, acc[i][j], x, y, a.dt, coef_x, a.dta0, c0, fe);
-      a.xout[idx] = x;
-      a.y[idx] = y;
-    }
+}
+
+template <int RPT, int NW, bool DISC>
+cudaError_t launch_f32_impl(cudaStream_t s, const Graph& g, const StepArgs& a,
+                            const F32Chunks& ch, int vec4, bool after_step) {
+  constexpr int RC = 8 * RPT * NW;
+  constexpr size_t SMEM = sizeof(float) * F_STAGES * F_KC * (F_ROWS + RC);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)g.n_row_tiles * F_GROUPS, (unsigned)((a.R + RC - 1) / RC));
+  cfg.blockDim = dim3(32 * NW);
+  cfg.dynamicSmemBytes = SMEM;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = after_step ? 1 : 0;
+  note_launch(1);
+  return cudaLaunchKernelEx(&cfg, k_step_f32<RPT, NW, DISC>, a, ch.list, ch.count, vec4);
+}
+
+template <int RPT, int NW>
+cudaError_t f32_attr() {
+  constexpr int SMEM = (int)sizeof(float) * F_STAGES * F_KC * (F_ROWS + 8 * RPT * NW);
+  cudaError_t e = cudaFuncSetAttribute(k_step_f32<RPT, NW, false>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_step_f32<RPT, NW, true>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+  return e;
 }
 
 // ------------------------------------------------------------------ CSR storage
@@ -1092,10 +1306,52 @@ void launch_f32_to_bf16(cudaStream_t s, const float* x, __nv_bfloat16* xh, int64
   if (n > 0) k_f32_to_bf16<<<::qh::counted(nblk(n)), 256, 0, s>>>(x, xh, n);
 }
 
-void launch_step_f32(cudaStream_t s, const Graph& g, const StepArgs& a) {
-  if (g.n_row_tiles == 0) return;
-  dim3 grid(g.n_row_tiles, (a.R + F_RT - 1) / F_RT);
-  k_step_f32<<<::qh::counted(grid), 256, 0, s>>>(a);
+qh_status f32_prepare(Ctx* ctx, const Graph& g, const float* tile_f32, int32_t sb,
+                      F32Chunks* ch) {
+  if (g.n_row_tiles == 0) return QH_OK;
+  const int64_t cap = std::max<int64_t>(g.n_tiles_hi, 1) * F_GROUPS * F_TILE_CHUNKS;
+  ch->list = (int2*)ctx->scratch((size_t)cap * sizeof(int2), S_F32_LIST);
+  ch->count = (int32_t*)ctx->scratch((size_t)g.n_row_tiles * F_GROUPS * 4, S_F32_COUNT);
+  if (!ch->list || !ch->count) return set_err(ctx, QH_ENOMEM, "allocation failed (FP32 chunks)");
+  k_f32_chunks<<<::qh::counted((unsigned)g.n_row_tiles), 256, 0, ctx->stream>>>(
+      g.rt, g.tile_col, tile_f32, sb == QH_SB_ADIABATIC ? 1 : 0, ch->list, ch->count);
+  return QH_OK;
+}
+
+cudaError_t f32_set_attrs() {
+  cudaError_t e = f32_attr<4, 2>();
+  if (e == cudaSuccess) e = f32_attr<2, 2>();
+  if (e == cudaSuccess) e = f32_attr<1, 2>();
+  return e;
+}
+
+qh_status launch_step_f32(Ctx* ctx, const Graph& g, const StepArgs& a, const F32Chunks& ch,
+                          bool after_step) {
+  if (g.n_row_tiles == 0) return QH_OK;
+  // 16-byte accesses of y, x_{t+1} and z (x_t is read in 16-byte pieces in any case)
+  const uintptr_t bits = (uintptr_t)a.y | (uintptr_t)a.xout | (uintptr_t)a.z_out;
+  const int vec4 = (bits & 15) == 0;
+  const bool disc = a.sb == QH_SB_DISCRETE;
+  // Replicas per thread: few warps hide no latency, so a small graph takes fewer replicas
+  // per thread (more warps), a large one more (fewer shared-memory reads per FMA).
+  // Measured, us per step at 1 / 2 / 4 replicas a thread: 720 reads, R = 64 (192 warps
+  // at 1): 5.4 / 6.6 / 8.8; 720 reads, R = 256 (768): 8.6 / 7.4 / 8.9; 1,800 reads,
+  // R = 256 (960 warps at 2): 15.7 / 9.9 / 11.8; 720 reads, R = 1,024 (1,536): 17 / 16 /
+  // 13.9; 7,200 reads, R = 256 (3,648): 32.9 / 25.2 / 17.9.  And no thread for replicas
+  // past R: 32 blocks, R = 16: 17.4 / 16.5 / 27.1.
+  auto warps = [&](int rpt) -> int64_t {
+    return (int64_t)g.n_row_tiles * F_GROUPS * ((a.R + 16 * rpt - 1) / (16 * rpt)) * 2;
+  };
+  const int rpt = a.R <= 16 || warps(1) <= 3 * ctx->n_sm     ? 1
+                  : a.R <= 32 || warps(2) <= 10 * ctx->n_sm ? 2
+                                                            : 4;
+  cudaError_t e;
+#define QH_F32(RPT)                                                               \
+  (disc ? launch_f32_impl<RPT, 2, true>(ctx->stream, g, a, ch, vec4, after_step)  \
+        : launch_f32_impl<RPT, 2, false>(ctx->stream, g, a, ch, vec4, after_step))
+  e = rpt == 1 ? QH_F32(1) : rpt == 2 ? QH_F32(2) : QH_F32(4);
+#undef QH_F32
+  return e == cudaSuccess ? QH_OK : cuda_fail(ctx, e, "k_step_f32 launch");
 }
 
 const char* csr_variant_name(int v, bool bf16) {

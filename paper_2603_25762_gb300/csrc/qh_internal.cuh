@@ -278,7 +278,20 @@ void launch_init_state(cudaStream_t s, const Graph& g, int32_t R, int32_t replic
 // X_hat of a state for the given SB variant: bf16(x), or sgn(x) at real vertices.
 void launch_x_operand(cudaStream_t s, const Graph& g, int32_t sb, const float* x,
                       __nv_bfloat16* xh, int64_t n);
-void launch_step_f32(cudaStream_t s, const Graph& g, const StepArgs& a);
+// FP32 step on tile storage.  f32_prepare lists, per 32-row group, the 8-column chunks of
+// the FP32 tiles that hold a nonzero (every chunk for adiabatic SB); the lists stay valid
+// while the tiles keep their pattern (a refinement's sign inversions do).
+struct F32Chunks {
+  int2* list = nullptr;
+  int32_t* count = nullptr;
+};
+constexpr int S_F32_LIST = 105, S_F32_COUNT = 106;  // scratch slots
+qh_status f32_prepare(Ctx* ctx, const Graph& g, const float* tile_f32, int32_t sb, F32Chunks* ch);
+// after_step: the launch before this one in the stream is another FP32 step (its prologue
+// may then overlap that step's end).
+qh_status launch_step_f32(Ctx* ctx, const Graph& g, const StepArgs& a, const F32Chunks& ch,
+                          bool after_step);
+cudaError_t f32_set_attrs();
 // CSR storage: warp per padded vertex, state [n_pad][R]; xh_in != nullptr selects the
 // BF16 X_hat operand, otherwise a.xin (FP32).  variant: CSR_LANE4 (4 replicas per lane,
 // any R that is a multiple of 4) or CSR_LANE8 (8 per lane, several neighbours per warp
