@@ -94,7 +94,7 @@ enum {
   S_SUMW, S_SUMJ2, S_NODETMP, S_SIGNS1, S_NODEVAL1, S_CUT1, S_DBG0, S_DBG1, S_DBG2, S_RUNNING,
   S_PVWORK, S_TR0, S_TR1, S_F8H, S_F8L, S_F8FLAG, S_X8, S_DEFORM, S_TRIES, S_DBGDEF,
   S_ZBAND, S_BANDWORK, S_RVWORK, S_TRACE, S_KCUT, S_KR, S_KFLAG, S_KSPINS, S_GAUGE, S_CTRACE,
-  S_CUTS_S, S_CUTS_Z
+  S_CUTS_S, S_CUTS_Z, S_TBASE
 };
 
 struct SolveBufs {
@@ -778,11 +778,25 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
   // ---- the step loop, captured once per shape and replayed
   // The captured step loop bakes in pointers and sizes; it is replayed only when every
   // one of them is unchanged (a rebuilt graph at other addresses is captured anew).
+  // A new graph usually sits at new addresses, and capturing costs 2 to 6 us a launch: as
+  // much as the steps of a small graph take.  So without checks only a chunk of steps is
+  // captured, replayed from a device-held step base; the steps past its last multiple are
+  // launched directly.  The chunk is even (the state's two buffers alternate) and, among
+  // 34 .. 64, leaves the fewest steps over.  With checks (their places and trace rows are
+  // baked in) the whole loop is one capture.
+  int32_t loop_steps = max_steps;
+  if (!checking) {
+    loop_steps = 0;  // up to 64 steps: direct launches only
+    for (int32_t c = 64; c >= 34 && max_steps > 64; c -= 2)
+      if (loop_steps == 0 || max_steps % c < max_steps % loop_steps) loop_steps = c;
+  }
+  int32_t* t_base = (int32_t*)ctx->scratch(16, S_TBASE);
+  if (!t_base) return set_err(ctx, QH_ENOMEM, "allocation failed (step base)");
   std::string skey;
   {
     auto add = [&skey](const void* p) { skey += std::to_string((uintptr_t)p) + "|"; };
     auto addi = [&skey](long long v) { skey += std::to_string(v) + "|"; };
-    addi(o->precision); addi(R); addi(max_steps); addi(checking ? o->check_every : 0);
+    addi(o->precision); addi(R); addi(loop_steps); addi(checking ? o->check_every : 0);
     addi(o->sb_variant);
     addi(o->patience);
     addi(track ? 1 : 0);
@@ -810,7 +824,7 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
                           (const void*)B.seen, (const void*)B.stall, (const void*)B.steps_run,
                           (const void*)ctx->d_err, (const void*)B.deform, (const void*)B.trace,
                           (const void*)B.cut_s, (const void*)B.cut_z,
-                          (const void*)f32.list, (const void*)f32.count})
+                          (const void*)f32.list, (const void*)f32.count, (const void*)t_base})
       add(p);
   }
   StepArgs a{};
@@ -913,6 +927,7 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
     StepArgs az = a;
     az.z_out = B.cut_z;
     az.t = 0;
+    az.t_base = nullptr;
     az.active = act;
     az.use_lo = W.has_lo ? 1 : 0;
     qh_status st = launch_step_tc(ctx, W, az, B.cut_s, pick_plan(R));
@@ -920,7 +935,16 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
     launch_cut_from_product(s, W, R, B.cut_z, B.cut_s, sum_w_work, B.node_val, B.cuts, act);
     return QH_OK;
   };
-  if (!multistep && (ctx->loop_key != skey || !ctx->loop_exec)) {
+  // one step t (relative to *base) of the per-step kernels
+  auto one_step = [&](int32_t t, const int32_t* base, bool after_step) -> qh_status {
+    a.t = t;
+    a.t_base = base;
+    const bool even = (t % 2) == 0;
+    return run_step(ctx, W, o->precision, tplan, a, even ? B.x : B.x1, even ? B.x1 : B.x,
+                    even ? B.xh0 : B.xh1, even ? B.xh1 : B.xh0, &f8, (int64_t)NS, B.zband, f32,
+                    after_step);
+  };
+  if (!multistep && loop_steps > 0 && (ctx->loop_key != skey || !ctx->loop_exec)) {
     if (ctx->loop_exec) {
       cudaGraphExecDestroy(ctx->loop_exec);
       ctx->loop_exec = nullptr;
@@ -932,16 +956,12 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
     QH_CUDA_TRY(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     qh_status st = QH_OK;
     bool after_step = false;  // the launch before is another step
-    for (int32_t t = 0; t < max_steps && st == QH_OK; ++t) {
-      a.t = t;
-      const bool even = (t % 2) == 0;
-      st = run_step(ctx, W, o->precision, tplan, a, even ? B.x : B.x1, even ? B.x1 : B.x,
-                    even ? B.xh0 : B.xh1, even ? B.xh1 : B.xh0, &f8, (int64_t)NS, B.zband,
-                    f32, after_step);
+    for (int32_t t = 0; t < loop_steps && st == QH_OK; ++t) {
+      st = one_step(t, checking ? nullptr : t_base, after_step);
       after_step = true;
       if (checking && (t + 1) % o->check_every == 0 && t + 1 < max_steps) {
         after_step = false;
-        const float* xc = (o->precision == QH_PREC_FP32 && even) ? B.x1 : B.x;
+        const float* xc = (o->precision == QH_PREC_FP32 && t % 2 == 0) ? B.x1 : B.x;
         if (st == QH_OK) st = replica_cuts(xc, B.running);
         launch_pick_best(s, nb, R, B.cuts, B.best_r, B.best_cut, B.running);
         launch_trace_check(s, nb, B.best_cut, B.running, t + 1, B.steps_b,
@@ -954,6 +974,7 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
                             o->patience, t + 1, B.steps_b);
       }
     }
+    if (!checking) launch_advance(s, t_base, loop_steps);
     cudaError_t ce = cudaStreamEndCapture(s, &graph);
     if (st != QH_OK) {
       if (ce == cudaSuccess) cudaGraphDestroy(graph);
@@ -1034,8 +1055,16 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
         }
       }
     } else {
-      QH_CUDA_TRY(cudaGraphLaunch(ctx->loop_exec, s));
-      note_launch(ctx->loop_kernels);
+      QH_CUDA_TRY(cudaMemsetAsync(t_base, 0, 4, s));
+      const int32_t n_rep = loop_steps > 0 ? max_steps / loop_steps : 0;
+      for (int32_t k = 0; k < n_rep; ++k) {
+        QH_CUDA_TRY(cudaGraphLaunch(ctx->loop_exec, s));
+        note_launch(ctx->loop_kernels);
+      }
+      for (int32_t t = n_rep * loop_steps; t < max_steps; ++t) {
+        qh_status st = one_step(t, nullptr, t > n_rep * loop_steps);
+        if (st != QH_OK) return st;
+      }
     }
     QH_CUDA_TRY(cudaEventRecord(ctx->ev[3], s));
     {

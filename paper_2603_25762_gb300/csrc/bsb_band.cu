@@ -71,8 +71,10 @@ __global__ void __launch_bounds__(192, 1) k_band_mma(const __grid_constant__ CUt
                                                        int32_t R,
                                                        const int32_t* __restrict__ active,
                                                        const int32_t* __restrict__ steps_b,
-                                                       int32_t t, float* __restrict__ z,
-                                                       int32_t* err) {
+                                                       int32_t t_rel,
+                                                       const int32_t* __restrict__ t_base,
+                                                       float* __restrict__ z, int32_t* err) {
+  const int32_t t = t_rel + (t_base != nullptr ? *t_base : 0);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -254,7 +256,7 @@ qh_status launch_band_mma(Ctx* ctx, const Graph& g, const StepArgs& a, const __n
   const unsigned grid = (unsigned)std::min<int64_t>(n_items, ctx->n_sm);
   k_band_mma<<<::qh::counted(grid), 192, P_SMEM, ctx->stream>>>(
       mA, mB, g.rt, g.n_row_tiles, nrep, a.R, a.active, a.z_out != nullptr ? nullptr : a.steps_b,
-      a.t, z, a.err);
+      a.t, a.t_base, z, a.err);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "k_band_mma launch");
   return QH_OK;

@@ -169,9 +169,9 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
   const int32_t r0 = blockIdx.y * RC;
   const int32_t vrows = rt.valid - grp * F_ROWS;  // real rows of this group
   if (vrows <= 0) return;
-  const int32_t sb = a.steps_b[rt.block];
+  const int32_t sb = a.steps_b[rt.block], t = step_of(a);
   if (tid == 0) {
-    const double at = a.a0 * (double)a.t / (double)sb;
+    const double at = a.a0 * (double)t / (double)sb;
     coef_s = (float)(-(a.a0 - at));
   }
   const int32_t nc = count[blockIdx.x];
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
   for (int i = 0; i < F_STAGES - 1; ++i) load_j(i, en[i]);
   grid_dep_wait();
   grid_dep_launch();
-  const bool live = (a.active == nullptr || a.active[rt.block]) && a.t < sb;
+  const bool live = (a.active == nullptr || a.active[rt.block]) && t < sb;
   const int32_t row0 = rt.row0 + grp * F_ROWS;
   if (!live) {
     cp_async_wait<0>();
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
   __syncthreads();  // coef_s (a list may be empty)
   const float coef_x = coef_s;
   const float c0 = a.c0[rt.block];
-  const float fe = deform_force(a.deform, rt.block, a.t, sb);
+  const float fe = deform_force(a.deform, rt.block, t, sb);
   auto index = [&](int j) -> size_t {
     return (size_t)(r0 + warp * 8 * RPT + pl + 8 * j) * a.n_pad + row0 + rl * 8;
   };
@@ -419,8 +419,8 @@ __global__ void __launch_bounds__(CSR_CTA, 1024 / CSR_CTA) k_step_csr(StepArgs a
   const int lane = threadIdx.x & 31;
   if (row >= a.n_pad) return;
   const RowTile rt = a.rt[row / TILE];
-  const int32_t sb = a.steps_b[rt.block];
-  const bool live = (a.active == nullptr || a.active[rt.block]) && a.t < sb;
+  const int32_t sb = a.steps_b[rt.block], t = step_of(a);
+  const bool live = (a.active == nullptr || a.active[rt.block]) && t < sb;
   if (row - rt.row0 >= rt.valid) return;  // padding vertex: state stays zero
   const size_t rbase = (size_t)row * a.R;
   if (!live) {
@@ -431,10 +431,10 @@ __global__ void __launch_bounds__(CSR_CTA, 1024 / CSR_CTA) k_step_csr(StepArgs a
     return;
   }
   const int64_t e0 = prow[row], e1 = prow[row + 1];
-  const double at = a.a0 * (double)a.t / (double)sb;
+  const double at = a.a0 * (double)t / (double)sb;
   const float coef_x = (float)(-(a.a0 - at));
   const float c0 = a.c0[rt.block];
-  const float fe = deform_force(a.deform, rt.block, a.t, a.steps_b[rt.block]);
+  const float fe = deform_force(a.deform, rt.block, t, sb);
   for (int32_t r0 = 0; r0 < a.R; r0 += 128) {
     const int32_t r = r0 + 4 * lane;
     const bool on = r < a.R;
@@ -553,8 +553,8 @@ __global__ void __launch_bounds__(CSR_CTA, 1024 / CSR_CTA) k_step_csr8(StepArgs 
   const int sub = lane / L, li = lane % L;
   if (row >= a.n_pad) return;
   const RowTile rt = a.rt[row / TILE];
-  const int32_t sb = a.steps_b[rt.block];
-  const bool live = (a.active == nullptr || a.active[rt.block]) && a.t < sb;
+  const int32_t sb = a.steps_b[rt.block], t = step_of(a);
+  const bool live = (a.active == nullptr || a.active[rt.block]) && t < sb;
   if (row - rt.row0 >= rt.valid) return;  // padding vertex: state stays zero
   const size_t rbase = (size_t)row * a.R;
   if (!live) {
@@ -650,10 +650,10 @@ __global__ void __launch_bounds__(CSR_CTA, 1024 / CSR_CTA) k_step_csr8(StepArgs 
       continue;
     }
     // the update's constants, taken after the gathers (fewer live registers there)
-    const double at = a.a0 * (double)a.t / (double)sb;
+    const double at = a.a0 * (double)t / (double)sb;
     const float coef_x = (float)(-(a.a0 - at));
     const float c0 = a.c0[rt.block];
-    const float fe = deform_force(a.deform, rt.block, a.t, sb);
+    const float fe = deform_force(a.deform, rt.block, t, sb);
     const float* xsrc = BF16 ? a.x : a.xin;
     float xs[8], ys[8];
 #pragma unroll
@@ -1476,6 +1476,12 @@ void launch_trace_check(cudaStream_t s, int32_t n_blocks, const double* best_cut
   if (n_blocks > 0)
     k_trace_check<<<::qh::counted(nblk(n_blocks)), 256, 0, s>>>(n_blocks, best_cut, running,
                                                                 t_done, steps_b, row);
+}
+
+__global__ void k_advance(int32_t* t_base, int32_t n) { *t_base += n; }
+
+void launch_advance(cudaStream_t s, int32_t* t_base, int32_t n) {
+  k_advance<<<::qh::counted(1), 1, 0, s>>>(t_base, n);
 }
 
 void launch_early_stop(cudaStream_t s, int32_t n_blocks, const double* best_cut, double* best_seen,

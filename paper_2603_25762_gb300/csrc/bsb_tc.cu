@@ -44,8 +44,8 @@ __global__ void __launch_bounds__(128) k_step_tc(const __grid_constant__ CUtenso
                  accb = smem_u32(bars + 2 * STAGES);
 
   const RowTile rt = a.rt[blockIdx.x];
-  const int32_t sb = a.steps_b[rt.block];
-  if ((a.active != nullptr && !a.active[rt.block]) || a.t >= sb) return;  // CTA-uniform
+  const int32_t sb = a.steps_b[rt.block], t = step_of(a);
+  if ((a.active != nullptr && !a.active[rt.block]) || t >= sb) return;  // CTA-uniform
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nk = (a.use_lo ? rt.n_all : rt.n_hi) * 2;  // 64-wide K slices
 
@@ -103,10 +103,10 @@ __global__ void __launch_bounds__(128) k_step_tc(const __grid_constant__ CUtenso
   tc_fence_after();
   const int row = warp * 32 + lane;
   const bool vrow = ok && row < rt.valid;
-  const double at = (double)a.a0 * (double)a.t / (double)sb;
+  const double at = (double)a.a0 * (double)t / (double)sb;
   const float coef_x = (float)(-((double)a.a0 - at));
   const float c0 = a.c0[rt.block];
-  const float fe = deform_force(a.deform, rt.block, a.t, a.steps_b[rt.block]);
+  const float fe = deform_force(a.deform, rt.block, t, a.steps_b[rt.block]);
   const size_t base = (size_t)blockIdx.y * BN * a.n_pad + rt.row0 + row;
 #pragma unroll
   for (int c = 0; c < BN / 32; ++c) {
@@ -168,8 +168,8 @@ __global__ void __launch_bounds__(128, MINB) k_step_tc_v(const __grid_constant__
                  accb = smem_u32(bars + 2 * STAGES);
 
   const RowTile rt = a.rt[blockIdx.x];
-  const int32_t sb = a.steps_b[rt.block];
-  if ((a.active != nullptr && !a.active[rt.block]) || a.t >= sb) return;  // CTA-uniform
+  const int32_t sb = a.steps_b[rt.block], t = step_of(a);
+  if ((a.active != nullptr && !a.active[rt.block]) || t >= sb) return;  // CTA-uniform
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nk = (a.use_lo ? rt.n_all : rt.n_hi) * 2;
   const int row = warp * 32 + lane;
@@ -234,10 +234,10 @@ __global__ void __launch_bounds__(128, MINB) k_step_tc_v(const __grid_constant__
 
   const bool ok = nk > 0 ? mbar_wait(accb, 0, a.err) : true;
   tc_fence_after();
-  const double at = a.a0 * (double)a.t / (double)sb;
+  const double at = a.a0 * (double)t / (double)sb;
   const float coef_x = (float)(-(a.a0 - at));
   const float c0 = a.c0[rt.block];
-  const float fe = deform_force(a.deform, rt.block, a.t, a.steps_b[rt.block]);
+  const float fe = deform_force(a.deform, rt.block, t, a.steps_b[rt.block]);
 #pragma unroll
   for (int c = 0; c < BN / CH; ++c) {
     uint32_t v[CH];
@@ -330,8 +330,8 @@ __global__ void __launch_bounds__(128, MINB)
                  accb = smem_u32(bars + 2 * STAGES);
 
   const RowTile rt = a.rt[blockIdx.x];
-  const int32_t sb = a.steps_b[rt.block];
-  if ((a.active != nullptr && !a.active[rt.block]) || a.t >= sb) return;  // CTA-uniform
+  const int32_t sb = a.steps_b[rt.block], t = step_of(a);
+  if ((a.active != nullptr && !a.active[rt.block]) || t >= sb) return;  // CTA-uniform
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nk = rt.n_hi * n_slices;
   const int row = warp * 32 + lane;
@@ -397,10 +397,10 @@ __global__ void __launch_bounds__(128, MINB)
 
   const bool ok = nk > 0 ? mbar_wait(accb, 0, a.err) : true;
   tc_fence_after();
-  const double at = a.a0 * (double)a.t / (double)sb;
+  const double at = a.a0 * (double)t / (double)sb;
   const float coef_x = (float)(-(a.a0 - at));
   const float c0 = a.c0[rt.block];
-  const float fe = deform_force(a.deform, rt.block, a.t, a.steps_b[rt.block]);
+  const float fe = deform_force(a.deform, rt.block, t, a.steps_b[rt.block]);
   const float inv_s = a.inv_scale;
 #pragma unroll
   for (int c = 0; c < BN / CH; ++c) {
@@ -523,8 +523,8 @@ struct PSmem {
   static constexpr uint32_t BYTES = BAR_OFF + 8 * N_BARS + 16 + 1024;
 };
 
-__device__ __forceinline__ bool item_live(const StepArgs& a, const RowTile& rt) {
-  return (a.active == nullptr || a.active[rt.block]) && a.t < a.steps_b[rt.block];
+__device__ __forceinline__ bool item_live(const StepArgs& a, int32_t t, const RowTile& rt) {
+  return (a.active == nullptr || a.active[rt.block]) && t < a.steps_b[rt.block];
 }
 
 template <int BN, int OSTAGES>
@@ -542,6 +542,7 @@ __global__ void __launch_bounds__(192, 1)
   const uint32_t sfull0 = smem_u32(bars + 2 * OSTAGES), sempty0 = sfull0 + 16;
   const uint32_t afull0 = sfull0 + 32, aempty0 = sfull0 + 48;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int32_t t = step_of(a);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < OSTAGES; ++s) {
@@ -570,7 +571,7 @@ __global__ void __launch_bounds__(192, 1)
       for (int32_t item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
         const int32_t rti = item / n_rep, rn = item % n_rep;
         const RowTile rt = a.rt[rti];
-        if (!item_live(a, rt)) continue;
+        if (!item_live(a, t, rt)) continue;
         const uint32_t sb = it & 1u, sph = (it >> 1) & 1u;
         if (!(ok = mbar_wait(sempty0 + 8 * sb, sph ^ 1u, a.err))) break;
         uint8_t* sx = smem + L::STATE_OFF + sb * 2 * L::STILE;
@@ -598,7 +599,7 @@ __global__ void __launch_bounds__(192, 1)
       bool ok = true;
       for (int32_t item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
         const RowTile rt = a.rt[item / n_rep];
-        if (!item_live(a, rt)) continue;
+        if (!item_live(a, t, rt)) continue;
         const uint32_t ab = it & 1u, aph = (it >> 1) & 1u;
         if (!(ok = mbar_wait(aempty0 + 8 * ab, aph ^ 1u, a.err))) break;
         tc_fence_after();
@@ -630,17 +631,17 @@ __global__ void __launch_bounds__(192, 1)
     for (int32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
       const int32_t rti = item / n_rep, rn = item % n_rep;
       const RowTile rt = a.rt[rti];
-      if (!item_live(a, rt)) continue;
+      if (!item_live(a, t, rt)) continue;
       const uint32_t b = it & 1u, ph = (it >> 1) & 1u;
       bool ok = mbar_wait(afull0 + 8 * b, ph, a.err);
       ok = mbar_wait(sfull0 + 8 * b, ph, a.err) && ok;
       tc_fence_after();
       float* sx = reinterpret_cast<float*>(smem + L::STATE_OFF + b * 2 * L::STILE);
       float* sy = sx + BN * TILE;
-      const double at = a.a0 * (double)a.t / (double)a.steps_b[rt.block];
+      const double at = a.a0 * (double)t / (double)a.steps_b[rt.block];
       const float coef_x = (float)(-(a.a0 - at));
       const float c0 = a.c0[rt.block];
-      const float fe = deform_force(a.deform, rt.block, a.t, a.steps_b[rt.block]);
+      const float fe = deform_force(a.deform, rt.block, t, a.steps_b[rt.block]);
       const bool vrow = ok && row < rt.valid;
       __nv_bfloat16* xh = a.xh_out + (size_t)rn * BN * a.n_pad + rt.row0 + row;
 #pragma unroll
@@ -732,6 +733,7 @@ __global__ void __launch_bounds__(384, 1)
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + P2_STAGES);
   const uint32_t afull0 = smem_u32(bars + 2 * P2_STAGES), aempty0 = afull0 + 16;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int32_t t = step_of(a);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < P2_STAGES; ++s) {
@@ -757,7 +759,7 @@ __global__ void __launch_bounds__(384, 1)
       // L2 while DRAM runs at full rate underneath
       for (int32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const RowTile rt = a.rt[item / n_rep];
-        if (!item_live(a, rt)) continue;
+        if (!item_live(a, t, rt)) continue;
         tma_prefetch_l2(&tmSx, rt.row0, (item % n_rep) * P2_BN);
         tma_prefetch_l2(&tmSy, rt.row0, (item % n_rep) * P2_BN);
       }
@@ -766,7 +768,7 @@ __global__ void __launch_bounds__(384, 1)
       for (int32_t item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
         const RowTile rt = a.rt[item / n_rep];
         const int32_t rn = item % n_rep;
-        if (!item_live(a, rt)) continue;
+        if (!item_live(a, t, rt)) continue;
         // stage this item's column tiles (independent loads, one latency)
         int32_t* cols = scol + (it & 1u) * P2_MAX_TILES;
         const int ne = a.use_lo ? rt.n_all : rt.n_hi;
@@ -792,7 +794,7 @@ __global__ void __launch_bounds__(384, 1)
       bool ok = true;
       for (int32_t item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
         const RowTile rt = a.rt[item / n_rep];
-        if (!item_live(a, rt)) continue;
+        if (!item_live(a, t, rt)) continue;
         const uint32_t ab = it & 1u, aph = (it >> 1) & 1u;
         if (!(ok = mbar_wait(aempty0 + 8 * ab, aph ^ 1u, a.err))) break;
         tc_fence_after();
@@ -823,7 +825,7 @@ __global__ void __launch_bounds__(384, 1)
     for (int32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
       const RowTile rt = a.rt[item / n_rep];
       const int32_t rn = item % n_rep;
-      if (!item_live(a, rt)) continue;
+      if (!item_live(a, t, rt)) continue;
       const uint32_t ab = it & 1u, aph = (it >> 1) & 1u;
       const bool vrow = row < rt.valid;
       const size_t base = ((size_t)rn * BN + hcol) * a.n_pad + rt.row0 + row;
@@ -838,10 +840,10 @@ __global__ void __launch_bounds__(384, 1)
       }
       const bool ok = mbar_wait(afull0 + 8 * ab, aph, a.err);
       tc_fence_after();
-      const double at = a.a0 * (double)a.t / (double)a.steps_b[rt.block];
+      const double at = a.a0 * (double)t / (double)a.steps_b[rt.block];
       const float coef_x = (float)(-(a.a0 - at));
       const float c0 = a.c0[rt.block];
-      const float fe = deform_force(a.deform, rt.block, a.t, a.steps_b[rt.block]);
+      const float fe = deform_force(a.deform, rt.block, t, a.steps_b[rt.block]);
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         uint32_t v[32];

@@ -208,7 +208,8 @@ struct StepArgs {
   const int32_t* active;  // [n_blocks] or nullptr
   const int32_t* steps_b;  // [n_blocks] schedule length per block (a(t) = a0 t / steps_b)
   int32_t n_pad, R;
-  int32_t t;              // step index
+  int32_t t;              // step index, relative to *t_base
+  const int32_t* t_base;  // device word a replayed chunk of steps counts from, or nullptr (0)
   int32_t use_lo;         // BF16 paths: also accumulate the lo (remainder) tiles
   uint8_t* x8h_out;       // FP8 path: e4m3 hi / lo parts of X_{t+1}
   uint8_t* x8l_out;
@@ -223,6 +224,10 @@ struct StepArgs {
                           // nullptr: y gains dt h_b (1 - t / steps_b) (uniform field
                           // along the incumbent, all +1 in the refinement's gauged frame)
 };
+
+__device__ __forceinline__ int32_t step_of(const StepArgs& a) {
+  return a.t + (a.t_base != nullptr ? *a.t_base : 0);
+}
 
 // The deformation field's force at step t of a block with schedule length sb.
 __device__ __forceinline__ float deform_force(const float* deform, int32_t block, int32_t t,
@@ -346,6 +351,8 @@ void launch_cut_from_product(cudaStream_t s, const Graph& g, int32_t R, const fl
 void launch_trace_check(cudaStream_t s, int32_t n_blocks, const double* best_cut,
                         const int32_t* running, int32_t t_done, const int32_t* steps_b,
                         double* row);
+// *t_base += n: the last node of a replayed chunk of n steps.
+void launch_advance(cudaStream_t s, int32_t* t_base, int32_t n);
 void launch_early_stop(cudaStream_t s, int32_t n_blocks, const double* best_cut, double* best_seen,
                        int32_t* stall, int32_t* active, int32_t* steps_run, int32_t patience,
                        int32_t t_done, const int32_t* steps_b);
