@@ -808,7 +808,8 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
     addi(G.max_tiles_per_row); addi(G.pnnz); addi(G.nnz);
     addi(f8.n_slices); add(f8_jh); add(f8_jl);
     skey += std::to_string(f8_s) + "|";
-    for (const void* p : {(const void*)G.rt, (const void*)G.tile_col, (const void*)W.tile_bf16,
+    for (const void* p : {(const void*)G.rt, (const void*)G.tile_col, (const void*)G.kslice,
+                          (const void*)W.tile_bf16,
                           (const void*)W.tile_f32, (const void*)G.prow_ptr, (const void*)G.pcol,
                           (const void*)W.pval, (const void*)W.band, (const void*)W.rval,
                           (const void*)G.rrow_ptr, (const void*)G.rcol, (const void*)B.zband,
@@ -830,6 +831,7 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
   StepArgs a{};
   a.rt = G.rt;
   a.tile_col = G.tile_col;
+  a.kslice = o->sb_variant == QH_SB_ADIABATIC ? nullptr : G.kslice;
   a.tile_f32 = W.tile_f32;
   a.x = B.x;
   a.y = B.y;
@@ -1585,6 +1587,7 @@ qh_status qh_debug_run_trace(qh_ctx* h, const qh_graph* gh, int32_t R, int32_t s
   a.a0 = 1.0;
   a.dta0 = 1.f;
   a.sb = QH_SB_BALLISTIC;
+  a.kslice = g.kslice;
   QH_CUDA_TRY(cudaMemsetAsync(xh1, 0, NS * 2, s));
   QH_CUDA_TRY(cudaMemsetAsync(tr, 0, n_stamps * 8, s));
   launch_init_state(s, g, R, 0, 1, 0, x, y, xh0, nullptr);
@@ -1704,6 +1707,7 @@ qh_status qh_debug_steps_v(qh_ctx* h, const qh_graph* gh, int32_t precision, int
   qh_status st = debug_common(ctx, g, precision, R, a, c0_per_block, steps, &c0h);
   if (st) return st;
   a.sb = sb_variant;
+  a.kslice = sb_variant == QH_SB_ADIABATIC ? nullptr : g.kslice;
   a.deform = nullptr;
   if (field_per_block != nullptr && g.n_blocks > 0) {
     std::vector<float> hf(g.n_blocks);

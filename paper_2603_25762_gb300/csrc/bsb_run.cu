@@ -69,7 +69,10 @@ constexpr uint32_t SLICE = TILE * 64 * 2;  // a 128 x 64 BF16 K-slice (16 KB)
 constexpr int JRES_TILES = 4;              // resident J tiles (hi + lo entries) per CTA
 
 struct ItemInfo {
-  int32_t row0, valid, tile_begin, nk;  // nk = K-slices (2 per J tile entry)
+  int32_t row0, valid, tile_begin, nk;  // nk = K-slices walked
+  int32_t ks_begin;                     // their first record (Graph::kslice)
+  const KSlice* ks;                     // the records: shared memory, or global if too many,
+                                        // or nullptr (every slice, too many to stage)
   int32_t block, k, last_t, steps_b;    // last_t < t0: nothing to do this launch
   int32_t rt;                           // row tile index (= its column tile index)
   uint32_t rows_b;                      // row tiles of the block
@@ -88,13 +91,19 @@ struct RunSmem {
   // sfull, sfree
   static constexpr int N_BARS = 3 * ST + 3 * MAX_ITEMS + 4;
   static constexpr uint32_t INFO_OFF = BAR_OFF + 8 * N_BARS;
+  static_assert(INFO_OFF % 8 == 0 && sizeof(ItemInfo) % 8 == 0, "records are 8-byte aligned");
   static constexpr uint32_t STOP_OFF = INFO_OFF + sizeof(ItemInfo) * MAX_ITEMS;
-  static constexpr uint32_t BYTES = STOP_OFF + 4 * MAX_ITEMS + 16 + 1024;
+  static constexpr uint32_t KS_OFF = STOP_OFF + 4 * MAX_ITEMS;  // staged K-slice records
+  // (JRES: at most JRES_TILES tiles, 2 slices each, for each of MAX_ITEMS items)
+  static constexpr int KS_CAP = JRES ? 2 * JRES_TILES * MAX_ITEMS : 1024;
+  static constexpr uint32_t BYTES = KS_OFF + 8 * KS_CAP + 16 + 1024;
+  static_assert(BYTES <= 227 * 1024, "shared memory of one CTA");
 };
 
 struct RunArgs {
   const RowTile* rt;
   const int32_t* tile_col;
+  const KSlice* kslice;     // nonzero K-slices per row tile, or nullptr: every K-slice
   float* x;                 // [R][n_pad]: read before the first step, written after the last
   float* y;                 // [R][n_pad]: likewise
   float4* xq;               // [R/4][n_pad] working copy of x between the first and the last
@@ -497,6 +506,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
   const int n_steps = a.t1 - a.t0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
+  KSlice* const sks = reinterpret_cast<KSlice*>(smem + L::KS_OFF);
   if (warp == 2 && lane < n_items) {
     const int item = a.items[wk.x + lane * a.item_stride];
     const RowTile rt = a.rt[item / a.n_kt];
@@ -504,7 +514,8 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
     it.row0 = rt.row0;
     it.valid = rt.valid;
     it.tile_begin = rt.tile_begin;
-    it.nk = 2 * (a.use_lo ? rt.n_all : rt.n_hi);
+    it.nk = row_slices(a.kslice, rt, a.use_lo);
+    it.ks_begin = rt.ks_begin;
     it.block = rt.block;
     it.k = item % a.n_kt;
     it.steps_b = a.steps_b[rt.block];
@@ -544,6 +555,30 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
+  // The items' K-slice records go into shared memory: the producers look one up per slice
+  // and step on the chain from release to product, where a global load misses L1 (the
+  // state sweeps it).
+  {
+    int total = 0;
+    for (int i = 0; i < n_items; ++i) total += info[i].nk;
+    const bool fits = total <= L::KS_CAP;
+    int at = 0;
+    for (int i = 0; i < n_items; ++i) {
+      const int nk = info[i].nk;
+      if (fits)
+        for (int kb = threadIdx.x; kb < nk; kb += RUN_THREADS)
+          sks[at + kb] =
+              slice_at(a.kslice, a.tile_col, info[i].ks_begin, info[i].tile_begin, kb);
+      if (threadIdx.x == 0)
+        info[i].ks = fits ? sks + at : a.kslice != nullptr ? a.kslice + info[i].ks_begin : nullptr;
+      at += nk;
+    }
+  }
+  __syncthreads();
+  auto slice = [&](const ItemInfo& it, int kb) -> KSlice {
+    return it.ks != nullptr ? it.ks[kb]
+                            : slice_at(nullptr, a.tile_col, it.ks_begin, it.tile_begin, kb);
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -558,9 +593,10 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
       if (JRES && lead) {  // all items of the CTA share one row tile
         const ItemInfo& it = info[0];
         mbar_expect_tx(jbar, (uint32_t)it.nk * SLICE);
-        for (int kb = 0; kb < it.nk; ++kb)
-          tma_load_2d(smem_u32(smem + kb * SLICE), &tmJ, jbar, (kb & 1) * 64,
-                      (it.tile_begin + (kb >> 1)) * TILE);
+        for (int kb = 0; kb < it.nk; ++kb) {
+          const KSlice ks = slice(it, kb);
+          tma_load_2d(smem_u32(smem + kb * SLICE), &tmJ, jbar, ks.half() * 64, ks.jrow());
+        }
         jissued = true;
       }
       bool ok = true;
@@ -614,8 +650,9 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
             for (int kb0 = 0; ok && kb0 < it.nk; kb0 += ST) {
               const int kb = kb0 + lane;
               const bool mine = lane < ST && kb < it.nk;
-              const int e = kb >> 1, half = kb & 1;
-              const int32_t ct = mine ? a.tile_col[it.tile_begin + e] : 0;
+              const KSlice ks = slice(it, mine ? kb : 0);
+              const int half = ks.half();
+              const int32_t ct = ks.ct();
               bool lok = true;
               if (pass == 0) {
                 if (u > 0 && kb0 == 0 && lead && !a.group_sync) {
@@ -651,8 +688,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
                   const uint32_t xdst = JRES ? smem_u32(slot) : smem_u32(slot + SLICE);
                   tma_load_2d(xdst, mp, full0 + 8 * s, ct * TILE + half * 64, it.k * RB);
                   if (!JRES && !jsplit)
-                    tma_load_2d(smem_u32(slot), &tmJ, full0 + 8 * s, half * 64,
-                                (it.tile_begin + e) * TILE);
+                    tma_load_2d(smem_u32(slot), &tmJ, full0 + 8 * s, half * 64, ks.jrow());
                 }
               }
               if (!__all_sync(0xffffffffu, lok)) ok = false;
@@ -678,7 +714,8 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
       constexpr uint32_t idesc = idesc_bf16<RB>();
       bool ok = true;
       if (JRES) ok = rwait(jbar, 0, a.err, abort_flag);
-      uint32_t q = 0, dead = 0, n_chk = 0;
+      uint32_t dead = 0, n_chk = 0;
+      uint32_t s = 0, ph = 0;  // next ring slot and its phase
       for (int u = 0; ok && u < n_steps; ++u) {
         const int t = a.t0 + u;
         for (int i = 0; ok && i < n_items; ++i) {
@@ -707,8 +744,6 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
             }
             const uint32_t d = pass == 0 ? tmem + (uint32_t)(i * RB) : tmem + SPARE_COL;
             for (int kb = 0; kb < it.nk; ++kb) {
-              const int s = (int)(q % ST);
-              const uint32_t ph = (q / ST) & 1u;
               if (!(ok = rwait(full0 + 8 * s, ph, a.err, abort_flag))) break;
               if (jsplit && !(ok = rwait(fullj0 + 8 * s, ph, a.err, abort_flag))) break;
               tc_fence_after();
@@ -722,7 +757,10 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
                 mma_bf16(d, jd + (uint64_t)(2 * k), xd + (uint64_t)(2 * k), idesc,
                          (pass == 0 || kb > 0 || k > 0) ? 1u : 0u);
               mma_commit(empty0 + 8 * s);
-              ++q;
+              if (++s == (uint32_t)ST) {
+                s = 0;
+                ph ^= 1u;
+              }
             }
             if (!ok) break;
             if (pass == 0) {
@@ -1009,9 +1047,10 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
               const uint32_t ph = ((q + kb) / ST) & 1u;
               lok = rwait(empty0 + 8 * s, ph ^ 1u, a.err, abort_flag);
               if (lok) {
+                const KSlice ks = slice(it, kb);
                 mbar_expect_tx(fullj0 + 8 * s, SLICE);
                 tma_load_2d(smem_u32(smem + L::RING_OFF + s * L::SLOT), &tmJ, fullj0 + 8 * s,
-                            (kb & 1) * 64, (it.tile_begin + (kb >> 1)) * TILE);
+                            ks.half() * 64, ks.jrow());
               }
             }
             const uint32_t issued = __ballot_sync(0xffffffffu, mine && lok);
@@ -1219,13 +1258,13 @@ qh_status run_prepare(Ctx* ctx, const Graph& g, int R, int variant, bool use_lo,
   const int n_kt = R / RB;
   rb->jres = run_jres(variant);
   rb->group_sync = run_group(variant);
-  // J copies run ahead in their own ring when most row tiles span more K-slices (2 per
-  // stored tile entry) than the operand ring holds: the copies of their later K-slices
+  // J copies run ahead in their own ring when most row tiles span more nonzero K-slices
+  // than the operand ring holds: the copies of their later K-slices
   // wait for ring slots, and without the split the J copies wait with them.  Rows that
   // fit the ring measured slower with the split (one more wait per K-slice).
   int64_t wide = 0;
   for (const RowTile& rt : g.h_rt)
-    if (2 * (use_lo ? rt.n_all : rt.n_hi) > RunSmem<false>::ST) ++wide;
+    if ((use_lo ? rt.nk_all : rt.nk_hi) > RunSmem<false>::ST) ++wide;
   rb->jsplit = 2 * wide > (int64_t)g.h_rt.size();
   rb->waves = plan.waves;
   std::vector<int32_t> rows(std::max(g.n_blocks, 1), 0);
@@ -1266,6 +1305,7 @@ qh_status launch_run_impl(Ctx* ctx, const Graph& g, const StepArgs& s, const Run
   RunArgs a{};
   a.rt = s.rt;
   a.tile_col = s.tile_col;
+  a.kslice = s.kslice;
   a.x = s.x;
   a.y = s.y;
   a.xq = rb.xq;

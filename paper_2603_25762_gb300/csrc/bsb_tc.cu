@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(128, MINB) k_step_tc_v(const __grid_constant__
   const int32_t sb = a.steps_b[rt.block], t = step_of(a);
   if ((a.active != nullptr && !a.active[rt.block]) || t >= sb) return;  // CTA-uniform
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nk = (a.use_lo ? rt.n_all : rt.n_hi) * 2;
+  const int nk = row_slices(a.kslice, rt, a.use_lo);
   const int row = warp * 32 + lane;
   const bool vrow = row < rt.valid;
   const size_t base = (size_t)blockIdx.y * BN * a.n_pad + rt.row0 + row;
@@ -207,10 +207,10 @@ __global__ void __launch_bounds__(128, MINB) k_step_tc_v(const __grid_constant__
       if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, a.err)) break;
       uint8_t* sa = smem + s * L::STAGE;
       mbar_expect_tx(full0 + 8 * s, L::STAGE);
-      const int e = kb >> 1, half = kb & 1;
-      tma_load_2d(smem_u32(sa), &tmJ, full0 + 8 * s, half * 64, (rt.tile_begin + e) * TILE);
-      tma_load_2d(smem_u32(sa + A_BYTES), &tmX, full0 + 8 * s,
-                  a.tile_col[rt.tile_begin + e] * TILE + half * 64, (int32_t)blockIdx.y * BN);
+      const KSlice ks = slice_at(a.kslice, a.tile_col, rt.ks_begin, rt.tile_begin, kb);
+      tma_load_2d(smem_u32(sa), &tmJ, full0 + 8 * s, ks.half() * 64, ks.jrow());
+      tma_load_2d(smem_u32(sa + A_BYTES), &tmX, full0 + 8 * s, ks.ct() * TILE + ks.half() * 64,
+                  (int32_t)blockIdx.y * BN);
     }
   } else if (warp == 1 && lane == 0 && nk > 0) {
     constexpr uint32_t idesc = idesc_bf16<BN>();
@@ -578,16 +578,16 @@ __global__ void __launch_bounds__(192, 1)
         mbar_expect_tx(sfull0 + 8 * sb, 2 * L::STILE);
         tma_load_2d(smem_u32(sx), &tmSx, sfull0 + 8 * sb, rt.row0, rn * BN);
         tma_load_2d(smem_u32(sx + L::STILE), &tmSy, sfull0 + 8 * sb, rt.row0, rn * BN);
-        const int nk = (a.use_lo ? rt.n_all : rt.n_hi) * 2;
+        const int nk = row_slices(a.kslice, rt, a.use_lo);
         for (int kb = 0; kb < nk; ++kb, ++kg) {
           const uint32_t st = kg % OSTAGES, ph = (kg / OSTAGES) & 1u;
           if (!(ok = mbar_wait(empty0 + 8 * st, ph ^ 1u, a.err))) break;
           uint8_t* sa = smem + st * L::OSTAGE;
           mbar_expect_tx(full0 + 8 * st, L::OSTAGE);
-          const int e = kb >> 1, half = kb & 1;
-          tma_load_2d(smem_u32(sa), &tmJ, full0 + 8 * st, half * 64, (rt.tile_begin + e) * TILE);
+          const KSlice ks = slice_at(a.kslice, a.tile_col, rt.ks_begin, rt.tile_begin, kb);
+          tma_load_2d(smem_u32(sa), &tmJ, full0 + 8 * st, ks.half() * 64, ks.jrow());
           tma_load_2d(smem_u32(sa + A_BYTES), &tmX, full0 + 8 * st,
-                      a.tile_col[rt.tile_begin + e] * TILE + half * 64, rn * BN);
+                      ks.ct() * TILE + ks.half() * 64, rn * BN);
         }
         ++it;
       }
@@ -604,7 +604,7 @@ __global__ void __launch_bounds__(192, 1)
         if (!(ok = mbar_wait(aempty0 + 8 * ab, aph ^ 1u, a.err))) break;
         tc_fence_after();
         const uint32_t dcol = tmem + ab * BN;
-        const int nk = (a.use_lo ? rt.n_all : rt.n_hi) * 2;
+        const int nk = row_slices(a.kslice, rt, a.use_lo);
         for (int kb = 0; kb < nk; ++kb, ++kg) {
           const uint32_t st = kg % OSTAGES, ph = (kg / OSTAGES) & 1u;
           if (!(ok = mbar_wait(full0 + 8 * st, ph, a.err))) break;
@@ -705,8 +705,8 @@ constexpr int P2_MAX_TILES = 64;  // per row tile (hi + lo entries); more falls 
 struct P2Smem {
   static constexpr uint32_t B_BYTES = P2_BN * 64 * 2;
   static constexpr uint32_t OSTAGE = A_BYTES + B_BYTES;
-  static constexpr uint32_t COL_OFF = P2_STAGES * OSTAGE;       // staged tile columns
-  static constexpr uint32_t BAR_OFF = COL_OFF + 2 * P2_MAX_TILES * 4;
+  static constexpr uint32_t KS_OFF = P2_STAGES * OSTAGE;        // staged K-slice records
+  static constexpr uint32_t BAR_OFF = KS_OFF + 4 * P2_MAX_TILES * 8;
   static constexpr uint32_t N_BARS = 2 * P2_STAGES + 4;
   static constexpr uint32_t BYTES = BAR_OFF + 8 * N_BARS + 16 + 1024;
 };
@@ -729,7 +729,7 @@ __global__ void __launch_bounds__(384, 1)
                                              ~static_cast<uintptr_t>(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::BAR_OFF);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::N_BARS);
-  int32_t* scol = reinterpret_cast<int32_t*>(smem + L::COL_OFF);  // [2][P2_MAX_TILES]
+  KSlice* sks = reinterpret_cast<KSlice*>(smem + L::KS_OFF);  // [2][2 P2_MAX_TILES]
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + P2_STAGES);
   const uint32_t afull0 = smem_u32(bars + 2 * P2_STAGES), aempty0 = afull0 + 16;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -769,20 +769,20 @@ __global__ void __launch_bounds__(384, 1)
         const RowTile rt = a.rt[item / n_rep];
         const int32_t rn = item % n_rep;
         if (!item_live(a, t, rt)) continue;
-        // stage this item's column tiles (independent loads, one latency)
-        int32_t* cols = scol + (it & 1u) * P2_MAX_TILES;
-        const int ne = a.use_lo ? rt.n_all : rt.n_hi;
-        for (int e = 0; e < ne; ++e) cols[e] = a.tile_col[rt.tile_begin + e];
-        const int nk = ne * 2;
+        // stage this item's K-slices (independent loads, one latency)
+        KSlice* slices = sks + (it & 1u) * 2 * P2_MAX_TILES;
+        const int nk = row_slices(a.kslice, rt, a.use_lo);
+        for (int kb = 0; kb < nk; ++kb)
+          slices[kb] = slice_at(a.kslice, a.tile_col, rt.ks_begin, rt.tile_begin, kb);
         for (int kb = 0; kb < nk; ++kb, ++kg) {
           const uint32_t st = kg % P2_STAGES, ph = (kg / P2_STAGES) & 1u;
           if (!(ok = mbar_wait(empty0 + 8 * st, ph ^ 1u, a.err))) break;
           uint8_t* sa = smem + st * L::OSTAGE;
           mbar_expect_tx(full0 + 8 * st, L::OSTAGE);
-          const int e = kb >> 1, half = kb & 1;
-          tma_load_2d(smem_u32(sa), &tmJ, full0 + 8 * st, half * 64, (rt.tile_begin + e) * TILE);
-          tma_load_2d(smem_u32(sa + A_BYTES), &tmX, full0 + 8 * st, cols[e] * TILE + half * 64,
-                      rn * BN);
+          const KSlice ks = slices[kb];
+          tma_load_2d(smem_u32(sa), &tmJ, full0 + 8 * st, ks.half() * 64, ks.jrow());
+          tma_load_2d(smem_u32(sa + A_BYTES), &tmX, full0 + 8 * st,
+                      ks.ct() * TILE + ks.half() * 64, rn * BN);
         }
         ++it;
       }
@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(384, 1)
         if (!(ok = mbar_wait(aempty0 + 8 * ab, aph ^ 1u, a.err))) break;
         tc_fence_after();
         const uint32_t dcol = tmem + ab * BN;
-        const int nk = (a.use_lo ? rt.n_all : rt.n_hi) * 2;
+        const int nk = row_slices(a.kslice, rt, a.use_lo);
         for (int kb = 0; kb < nk; ++kb, ++kg) {
           const uint32_t st = kg % P2_STAGES, ph = (kg / P2_STAGES) & 1u;
           if (!(ok = mbar_wait(full0 + 8 * st, ph, a.err))) break;

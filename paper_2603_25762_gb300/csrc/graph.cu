@@ -688,20 +688,29 @@ __global__ void k_perm_local(int64_t total, const uint64_t* __restrict__ keys,
 }
 
 // ------------------------------------------------------------------ tiles
+// Warp per vertex, the lanes striding over its row: flags[slot] = 1 for a 128 x 128 tile
+// with an edge, halves[slot] = its 64-column halves that hold one (bit per half).  Most
+// entries of a row fall into halves that are marked already: the mark is read first.
 __global__ void k_tile_flags(int32_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                              const double* __restrict__ w, const int32_t* __restrict__ block_of,
                              const int32_t* __restrict__ local, const int64_t* __restrict__ slot_off,
-                             const int32_t* __restrict__ tiles_per_block, int32_t* flags) {
-  int32_t a = blockIdx.x * blockDim.x + threadIdx.x;
+                             const int32_t* __restrict__ tiles_per_block, int32_t* flags,
+                             uint32_t* halves) {
+  const int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (a >= n) return;
-  int32_t b = block_of[a];
+  const int32_t b = block_of[a];
   if (b < 0) return;
-  int32_t T = tiles_per_block[b];
-  int32_t ra = local[a] / TILE;
-  for (int64_t e = rp[a]; e < rp[a + 1]; ++e) {
+  const int64_t s0 = slot_off[b] + (int64_t)(local[a] / TILE) * tiles_per_block[b];
+  for (int64_t e = rp[a] + lane; e < rp[a + 1]; e += 32) {
     if (w[e] == 0.0) continue;
-    int32_t cb = local[col[e]] / TILE;
-    flags[slot_off[b] + (int64_t)ra * T + cb] = 1;
+    const int32_t l = local[col[e]];
+    const int64_t slot = s0 + l / TILE;
+    const uint32_t bit = 1u << (l % TILE / 64);
+    if ((halves[slot] & bit) == 0) {
+      flags[slot] = 1;
+      atomicOr(halves + slot, bit);
+    }
   }
 }
 
@@ -1142,8 +1151,9 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
   int32_t* d_T = (int32_t*)ctx->scratch(sizeof(int32_t) * std::max(nb, 1), 18);
   int32_t* flags = (int32_t*)ctx->scratch(sizeof(int32_t) * std::max<int64_t>(n_slots, 1), 19);
   int64_t* slot_tile = (int64_t*)ctx->scratch(sizeof(int64_t) * (n_slots + 1), 20);
+  uint32_t* halves = (uint32_t*)ctx->scratch(4 * (size_t)std::max<int64_t>(n_slots, 1), 25);
   if (!g->block_ptr || !g->pad_off || !g->perm || !g->pad_node || !d_slot_off || !d_T || !flags ||
-      !slot_tile)
+      !slot_tile || !halves)
     return set_err(ctx, QH_ENOMEM, "allocation failed (layout)");
   QH_CUDA_TRY(cudaMemcpyAsync(g->block_ptr, h_block_ptr.data(), sizeof(int64_t) * (nb + 1),
                               cudaMemcpyHostToDevice, s));
@@ -1167,12 +1177,23 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
     QH_CUDA_TRY(cudaStreamSynchronize(s));
   } else {
     QH_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int32_t) * std::max<int64_t>(n_slots, 1), s));
+    QH_CUDA_TRY(cudaMemsetAsync(halves, 0, 4 * (size_t)std::max<int64_t>(n_slots, 1), s));
     if (N > 0)
-      k_tile_flags<<<::qh::counted(nblk(N)), 256, 0, s>>>(N, g->row_ptr, g->col, g->w, g->block_of, g->local,
-                                          d_slot_off, d_T, flags);
+      k_tile_flags<<<::qh::counted(nblk((int64_t)N * 32)), 256, 0, s>>>(N, g->row_ptr, g->col, g->w, g->block_of, g->local,
+                                          d_slot_off, d_T, flags, halves);
   }
   if (!scan_i32_to_i64(ctx, s, flags, slot_tile, n_slots)) return set_err(ctx, QH_ENOMEM, "allocation failed (scan)");
   std::vector<int64_t> h_slot_tile(n_slots + 1);
+  // the tiles' halves come with the slots, unless there are so many slots that the
+  // storage (CSR needs no halves) is better known first
+  std::vector<uint32_t> h_halves;
+  auto fetch_halves = [&]() -> cudaError_t {
+    h_halves.assign((size_t)n_slots, 3u);  // dense mode: both
+    if (o->dense || n_slots == 0) return cudaSuccess;
+    return cudaMemcpyAsync(h_halves.data(), halves, 4 * (size_t)n_slots, cudaMemcpyDeviceToHost, s);
+  };
+  const bool halves_later = n_slots > 65536;
+  if (!halves_later) QH_CUDA_TRY(fetch_halves());
   QH_CUDA_TRY(cudaMemcpyAsync(h_slot_tile.data(), slot_tile, sizeof(int64_t) * (n_slots + 1),
                               cudaMemcpyDeviceToHost, s));
   QH_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1185,11 +1206,15 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
     g->n_tiles_hi = 0;
     g->has_lo = false;
     std::fill(h_slot_tile.begin(), h_slot_tile.end(), 0);
+  } else if (halves_later) {
+    QH_CUDA_TRY(fetch_halves());
+    QH_CUDA_TRY(cudaStreamSynchronize(s));
   }
   // row tiles: hi entries then (if needed) lo entries, contiguous per row tile
   g->h_rt.clear();
   std::vector<int32_t> h_rt_of_block(std::max(nb, 1), 0);
   std::vector<int32_t> h_tile_col;
+  std::vector<KSlice> h_kslice;
   int64_t entry = 0;
   for (int32_t b = 0; b < nb; ++b) {
     h_rt_of_block[b] = (int32_t)g->h_rt.size();
@@ -1208,6 +1233,19 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
       std::vector<int32_t> cols;
       for (int32_t c = 0; c < T; ++c)
         if (h_slot_tile[s0 + c + 1] > h_slot_tile[s0 + c]) cols.push_back(ct0 + c);
+      // its K-slices with a nonzero (a remainder is nonzero only where J is)
+      rt.ks_begin = (int32_t)h_kslice.size();
+      for (int rep = 0; rep < (g->has_lo ? 2 : 1); ++rep) {
+        for (size_t j = 0; j < cols.size(); ++j) {
+          const uint32_t e = (uint32_t)(entry + rep * (int64_t)cols.size() + (int64_t)j);
+          const uint32_t m = h_halves[s0 + (cols[j] - ct0)];
+          for (uint32_t half = 0; half < 2; ++half)
+            if ((m >> half) & 1u)
+              h_kslice.push_back(KSlice{2 * e + half, 2 * (uint32_t)cols[j] + half});
+        }
+        if (rep == 0) rt.nk_hi = (int32_t)h_kslice.size() - rt.ks_begin;
+      }
+      rt.nk_all = (int32_t)h_kslice.size() - rt.ks_begin;
       for (int rep = 0; rep < (g->has_lo ? 2 : 1); ++rep)
         h_tile_col.insert(h_tile_col.end(), cols.begin(), cols.end());
       entry += rt.n_all;
@@ -1219,13 +1257,14 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
   g->n_row_tiles = (int32_t)g->h_rt.size();
   g->rt = (RowTile*)dalloc(*g, sizeof(RowTile) * std::max(g->n_row_tiles, 1));
   g->tile_col = (int32_t*)dalloc(*g, sizeof(int32_t) * std::max<int64_t>(g->n_tiles, 1));
+  g->kslice = (KSlice*)dalloc(*g, sizeof(KSlice) * std::max<size_t>(h_kslice.size(), 1));
   g->tile_bf16 = (__nv_bfloat16*)dalloc(*g, sizeof(__nv_bfloat16) * TILE * TILE * std::max<int64_t>(g->n_tiles, 1));
   g->tile_f32 = (float*)dalloc(*g, sizeof(float) * TILE * TILE * std::max<int64_t>(g->n_tiles_hi, 1));
   g->rt_of_block = (int32_t*)dalloc(*g, sizeof(int32_t) * std::max(nb, 1));
   g->slot_off = (int64_t*)dalloc(*g, sizeof(int64_t) * (nb + 1));
   g->tiles_per_block = (int32_t*)dalloc(*g, sizeof(int32_t) * std::max(nb, 1));
   g->slot_tile = (int64_t*)dalloc(*g, sizeof(int64_t) * (n_slots + 1));
-  if (!g->rt || !g->tile_col || !g->tile_bf16 || !g->tile_f32 || !g->rt_of_block || !g->slot_off ||
+  if (!g->rt || !g->tile_col || !g->kslice || !g->tile_bf16 || !g->tile_f32 || !g->rt_of_block || !g->slot_off ||
       !g->tiles_per_block || !g->slot_tile)
     return set_err(ctx, QH_ENOMEM, "allocation failed (tiles)");
   if (g->n_row_tiles > 0)
@@ -1233,6 +1272,9 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
                                 cudaMemcpyHostToDevice, s));
   if (g->n_tiles > 0)
     QH_CUDA_TRY(cudaMemcpyAsync(g->tile_col, h_tile_col.data(), sizeof(int32_t) * g->n_tiles,
+                                cudaMemcpyHostToDevice, s));
+  if (!h_kslice.empty())
+    QH_CUDA_TRY(cudaMemcpyAsync(g->kslice, h_kslice.data(), sizeof(KSlice) * h_kslice.size(),
                                 cudaMemcpyHostToDevice, s));
   QH_CUDA_TRY(cudaMemcpyAsync(g->rt_of_block, h_rt_of_block.data(), sizeof(int32_t) * std::max(nb, 1),
                               cudaMemcpyHostToDevice, s));

@@ -46,7 +46,18 @@ struct RowTile {           // one 128-row slab of a block in the padded layout
   int32_t n_hi;            // entries carrying J (FP32 path uses these only)
   int32_t n_all;           // hi entries followed by lo (BF16 remainder) entries
   int32_t f32_begin;       // first FP32 tile of this row tile
-  int32_t pad_;
+  int32_t ks_begin;        // first K-slice record (Graph::kslice)
+  int32_t nk_hi;           // nonzero K-slices of the hi entries
+  int32_t nk_all;          // and of the hi and lo entries
+};
+
+// One 64-column K-slice of a row tile's BF16 tile entries.
+struct KSlice {
+  uint32_t j;  // tile entry * 2 + half
+  uint32_t x;  // column tile * 2 + half
+  __host__ __device__ int32_t jrow() const { return (int32_t)(j >> 1) * TILE; }
+  __host__ __device__ int32_t half() const { return (int32_t)(j & 1u); }
+  __host__ __device__ int32_t ct() const { return (int32_t)(x >> 1); }
 };
 
 // Device memory of graphs and solutions comes from the owning context's stream-ordered
@@ -108,6 +119,7 @@ struct Graph {
   RowTile* rt = nullptr;          // [n_row_tiles]
   int32_t* rt_of_block = nullptr; // [n_blocks] first row tile of the block
   int32_t* tile_col = nullptr;    // [n_tiles] column tile (padded col / 128)
+  KSlice* kslice = nullptr;       // per row tile: its K-slices that hold a nonzero
   int64_t* slot_off = nullptr;    // [n_blocks+1] tile-slot offsets (T_b^2 slots per block)
   int32_t* tiles_per_block = nullptr;  // [n_blocks] T_b
   int64_t* slot_tile = nullptr;   // [slots+1] exclusive scan of nonzero slots
@@ -197,6 +209,7 @@ struct Ctx {
 struct StepArgs {
   const RowTile* rt;
   const int32_t* tile_col;
+  const KSlice* kslice;   // the nonzero K-slices, or nullptr: every K-slice
   const float* tile_f32;
   float* x;               // [R][n_pad]  (BF16 path: in place)
   float* y;               // [R][n_pad]
@@ -227,6 +240,19 @@ struct StepArgs {
 
 __device__ __forceinline__ int32_t step_of(const StepArgs& a) {
   return a.t + (a.t_base != nullptr ? *a.t_base : 0);
+}
+
+// The K-slices a tensor-core step walks.  A slice of zeros adds exact zeros for a finite
+// X_hat, so the steps whose x the walls keep in [-1, 1] leave it out; adiabatic SB has no
+// walls and the product entry points take any x: they walk every slice (kslice null).
+__device__ __forceinline__ int row_slices(const KSlice* ks, const RowTile& rt, int use_lo) {
+  return ks != nullptr ? (use_lo ? rt.nk_all : rt.nk_hi) : 2 * (use_lo ? rt.n_all : rt.n_hi);
+}
+__device__ __forceinline__ KSlice slice_at(const KSlice* ks, const int32_t* tile_col,
+                                           int32_t ks_begin, int32_t tile_begin, int kb) {
+  if (ks != nullptr) return ks[ks_begin + kb];
+  const uint32_t e = (uint32_t)(tile_begin + (kb >> 1)), half = kb & 1;
+  return KSlice{2 * e + half, 2 * (uint32_t)tile_col[e] + half};
 }
 
 // The deformation field's force at step t of a block with schedule length sb.
