@@ -42,7 +42,7 @@
 // separate instantiation (CHECK = true): the kernel without them carries none of their
 // code.
 //
-// Roles (384 threads): warp 0 = TMA producer (six lanes), warp 1 = MMA issuer (one
+// Roles (384 threads): warp 0 = TMA producer (six lanes for X_hat, six for J), warp 1 = MMA issuer (one
 // thread), warps 2-9 = epilogue (TMEM lane quarter = warp % 4 = 32 vertices, two warps
 // per quarter split the 128 replicas), warp 10 = signal, warp 11 = J producer.  With JRES
 // the J tiles of the CTA's single row tile stay in shared memory for the whole launch and
@@ -156,7 +156,7 @@ enum : int {
   TR_EPI_END = 6,   // epilogue (warp 2): its share of the update is stored (before it arrives)
   TR_RELEASE = 7,   // signal warp: X_hat of the next step is released to the other CTAs
   TR_PROD_START = 8,  // producer: reaches the item (before any of its waits)
-  TR_OWN = 9,       // producer: the item's own previous step is released (tile mode)
+  TR_OWN = 9,       // producer: lane 0's first K-slice is released
   TR_SLOT = 10,     // producer: the first ring slot for the item is free
   TR_SLOT1 = 11,    // producer: the ring slots of K-slices 1 .. 5 are free (5 events)
   TRACE_EVENTS = 16
@@ -582,10 +582,16 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    // Lanes 0 .. ST-1 fill up to ST ring slots at once, one K-slice (X_hat and J
-    // copies) per lane: the bulk copies of one thread complete one after the other, so
+    // Lanes 0 .. ST-1 (X_hat) and 8 .. 8 + ST-1 (J) fill up to ST ring slots at once, one
+    // copy per lane: the bulk copies of one thread complete one after the other, so
     // parallel lanes multiply the bytes in flight.  The MMA issuer consumes the slots
-    // in order.
+    // in order.  Only the K-slices that hold a nonzero are copied and multiplied (on
+    // hifi-region mostly 4 of a row tile's 6).  us per
+    // step, every slice and one lane per slice -> now: hifi-region (7,200 reads,
+    // R = 1,024) 9.37 -> 9.03; 1,800 reads, R = 1,024: 6.73 -> 6.0; 900 reads, R = 128:
+    // 5.88 -> 5.30; 12,000-SNP graph, R = 512: 16.65 -> 15.8; with early-stop checks
+    // (hifi-region) 12.98 -> 12.07.  Skipping single zero 16-column MMAs of a slice too
+    // measured slower: its lookup sits in the issuing thread (12,000 SNPs: 18.0).
     if (n_items > 0) {
       const bool lead = lane == 0;
       uint32_t q = 0;
@@ -635,11 +641,13 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
             }
           }
           // Dependencies, waited in parallel by the lanes (acquire loads of one thread
-          // would serialise, a round trip each).  Tile mode: lane 0 waits for the item's
-          // own previous step, every loading lane for the column tile of its K-slice
-          // (both halves of a column check its counter).  Group mode: lane 0 waits until
+          // would serialise, a round trip each).  Tile mode: every X_hat lane waits for the
+          // column tile of its K-slice (both halves of a column check its counter); the
+          // item's own step t-1 needs no wait of its own: its X_hat is read only through
+          // such a slice, and the MMA issuer waits for its accumulator.  Group mode: until
           // every row tile of the block has finished step t-1.  Then the lanes fill up to
-          // ST ring slots, one K-slice each.
+          // ST ring slots: lane l the X_hat copy and lane 8 + l the J copy of K-slice l (the
+          // copies one thread issues complete one after the other, 0.45 us each).
           if (lead) trace_at(a, u, i, TR_PROD_START);
           // pass 0: X_hat_t and J; pass 1 (check steps): S_t and J for the check product.
           // S_t is released together with X_hat_t, so pass 1 needs no waits of its own:
@@ -648,27 +656,23 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
             const CUtensorMap* mp =
                 pass == 0 ? mx : (((t / a.check_every) & 1) ? &tmS1 : &tmS0);
             for (int kb0 = 0; ok && kb0 < it.nk; kb0 += ST) {
-              const int kb = kb0 + lane;
-              const bool mine = lane < ST && kb < it.nk;
-              const KSlice ks = slice(it, mine ? kb : 0);
+              const int kb = kb0 + (lane & 7);
+              const bool in = (lane & 7) < ST && kb < it.nk;
+              const bool mine = in && lane < 8;                       // X_hat of slice kb
+              const bool minej = in && (lane >> 3) == 1 && !JRES && !jsplit;  // its J
+              const KSlice ks = slice(it, in ? kb : 0);
               const int half = ks.half();
               const int32_t ct = ks.ct();
               bool lok = true;
               if (pass == 0) {
-                if (u > 0 && kb0 == 0 && lead && !a.group_sync) {
-                  lok = wait_count(a.done + (size_t)it.rt * a.n_kt + it.k, (uint32_t)u, a.err,
-                                   abort_flag);
-                  if (lok) trace_at(a, u, i, TR_OWN);
-                }
-                // every loading lane acquires the release its own copies depend on
-                if (lok && mine && u > 0)
+                // every X_hat lane acquires the release its own copy depends on
+                if (mine && u > 0)
                   lok = a.group_sync
                             ? wait_count(a.done + (size_t)it.block * a.n_kt + it.k,
                                          (uint32_t)u * it.rows_b, a.err, abort_flag)
                             : wait_count(a.done + (size_t)ct * a.n_kt + it.k, (uint32_t)u,
                                          a.err, abort_flag);
-                if (lok && lead && (u == 0 || a.group_sync) && kb0 == 0)
-                  trace_at(a, u, i, TR_OWN);
+                if (lok && lead && kb0 == 0) trace_at(a, u, i, TR_OWN);
                 if (!__all_sync(0xffffffffu, lok)) {
                   ok = false;
                   break;
@@ -676,19 +680,18 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
                 if (u > 0 && mine) fence_proxy_async_global();
                 if (kb0 + ST >= it.nk && lead) trace_at(a, u, i, TR_DEPS);
               }
-              if (mine) {
+              if (mine || minej) {
                 const int s = (int)((q + kb) % ST);
                 const uint32_t ph = ((q + kb) / ST) & 1u;
                 lok = rwait(empty0 + 8 * s, ph ^ 1u, a.err, abort_flag);
                 if (lok) {
-                  if (pass == 0 && kb == 0) trace_at(a, u, i, TR_SLOT);
-                  if (pass == 0 && kb >= 1 && kb <= 5) trace_at(a, u, i, TR_SLOT1 + kb - 1);
+                  if (mine && pass == 0 && kb == 0) trace_at(a, u, i, TR_SLOT);
+                  if (mine && pass == 0 && kb >= 1 && kb <= 5) trace_at(a, u, i, TR_SLOT1 + kb - 1);
                   uint8_t* slot = smem + L::RING_OFF + s * L::SLOT;
-                  mbar_expect_tx(full0 + 8 * s, jsplit ? SLICE : L::SLOT);
-                  const uint32_t xdst = JRES ? smem_u32(slot) : smem_u32(slot + SLICE);
-                  tma_load_2d(xdst, mp, full0 + 8 * s, ct * TILE + half * 64, it.k * RB);
-                  if (!JRES && !jsplit)
-                    tma_load_2d(smem_u32(slot), &tmJ, full0 + 8 * s, half * 64, ks.jrow());
+                  if (mine) mbar_expect_tx(full0 + 8 * s, jsplit ? SLICE : L::SLOT);
+                  tma_load_2d(smem_u32(mine && !JRES ? slot + SLICE : slot), mine ? mp : &tmJ,
+                              full0 + 8 * s, mine ? ct * TILE + half * 64 : half * 64,
+                              mine ? it.k * RB : ks.jrow());
                 }
               }
               if (!__all_sync(0xffffffffu, lok)) ok = false;
@@ -1165,6 +1168,12 @@ static bool run_group(int v) { return v == RUN_VARIANT_FIRST || v == RUN_VARIANT
 // tiles of ONE row tile (its J tiles stay resident), the same k ranges in every row.
 // Stream: CTA c of the wave's G CTAs takes the wave's items c, c + G, c + 2G, ...
 // False when some block does not fit one wave.
+static bool rows_wide(const Graph& g, bool use_lo) {
+  int64_t wide = 0;
+  for (const RowTile& rt : g.h_rt)
+    if ((use_lo ? rt.nk_all : rt.nk_hi) > RunSmem<false>::ST) ++wide;
+  return 2 * wide > (int64_t)g.h_rt.size();
+}
 bool run_plan(const Graph& g, int R, int n_sm, int variant, bool use_lo, RunPlan* plan,
               const std::vector<int32_t>* mask, int max_items) {
   if (!run_variant(variant) || max_items < 1 || max_items > MAX_ITEMS) return false;
@@ -1262,10 +1271,7 @@ qh_status run_prepare(Ctx* ctx, const Graph& g, int R, int variant, bool use_lo,
   // than the operand ring holds: the copies of their later K-slices
   // wait for ring slots, and without the split the J copies wait with them.  Rows that
   // fit the ring measured slower with the split (one more wait per K-slice).
-  int64_t wide = 0;
-  for (const RowTile& rt : g.h_rt)
-    if ((use_lo ? rt.nk_all : rt.nk_hi) > RunSmem<false>::ST) ++wide;
-  rb->jsplit = 2 * wide > (int64_t)g.h_rt.size();
+  rb->jsplit = rows_wide(g, use_lo);
   rb->waves = plan.waves;
   std::vector<int32_t> rows(std::max(g.n_blocks, 1), 0);
   for (const RowTile& rt : g.h_rt) rows[rt.block] += 1;
