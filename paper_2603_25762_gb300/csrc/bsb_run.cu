@@ -66,6 +66,7 @@ constexpr int RUN_THREADS = 32 * (4 + EPI_WARPS);
 constexpr int SIGNAL_WARP = 2 + EPI_WARPS;
 constexpr int JPROD_WARP = SIGNAL_WARP + 1;  // J K-slices into their own ring (stream mode)
 constexpr uint32_t SLICE = TILE * 64 * 2;  // a 128 x 64 BF16 K-slice (16 KB)
+constexpr int JSPLIT_SLICES = 6;           // J copies by their own warp above this many
 constexpr int JRES_TILES = 4;              // resident J tiles (hi + lo entries) per CTA
 
 struct ItemInfo {
@@ -81,9 +82,13 @@ struct ItemInfo {
   double inv_steps;                     // 1 / steps_b
 };
 
-template <bool JRES>
+template <bool JRES, int SB>
 struct RunSmem {
-  static constexpr int ST = 6;                                  // operand ring slots
+  // Operand ring slots.  Stream mode: four hold the K-slices of most read-graph row tiles;
+  // measured us per step at 4 / 5 / 6: hifi-region 8.81 / 8.85 / 9.02, 12,000 SNPs 15.79 /
+  // 15.57 / 15.82, 96 blocks (R = 256) 50.3 / 51.6 / 51.4.  Adiabatic SB walks all six
+  // (hifi-region 9.68 / - / 9.06).
+  static constexpr int ST = JRES || SB == QH_SB_ADIABATIC ? 6 : 4;
   static constexpr uint32_t SLOT = JRES ? SLICE : 2 * SLICE;    // X_hat (+ J) per slot
   static constexpr uint32_t RING_OFF = JRES ? JRES_TILES * 2 * SLICE : 0;
   static constexpr uint32_t BAR_OFF = RING_OFF + ST * SLOT;
@@ -473,7 +478,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
     k_bsb_run(const __grid_constant__ CUtensorMap tmJ, const __grid_constant__ CUtensorMap tmX0,
               const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ CUtensorMap tmS0,
               const __grid_constant__ CUtensorMap tmS1, RunArgs a) {
-  using L = RunSmem<JRES>;
+  using L = RunSmem<JRES, SB>;
   constexpr int ST = L::ST;
   // J K-slices in a ring of their own, filled by the J producer warp (stream mode without
   // checks, chosen by the host when row tiles span more K-slices than the ring holds);
@@ -1171,7 +1176,7 @@ static bool run_group(int v) { return v == RUN_VARIANT_FIRST || v == RUN_VARIANT
 static bool rows_wide(const Graph& g, bool use_lo) {
   int64_t wide = 0;
   for (const RowTile& rt : g.h_rt)
-    if ((use_lo ? rt.nk_all : rt.nk_hi) > RunSmem<false>::ST) ++wide;
+    if ((use_lo ? rt.nk_all : rt.nk_hi) > JSPLIT_SLICES) ++wide;
   return 2 * wide > (int64_t)g.h_rt.size();
 }
 bool run_plan(const Graph& g, int R, int n_sm, int variant, bool use_lo, RunPlan* plan,
@@ -1268,7 +1273,7 @@ qh_status run_prepare(Ctx* ctx, const Graph& g, int R, int variant, bool use_lo,
   rb->jres = run_jres(variant);
   rb->group_sync = run_group(variant);
   // J copies run ahead in their own ring when most row tiles span more nonzero K-slices
-  // than the operand ring holds: the copies of their later K-slices
+  // than six (JSPLIT_SLICES): the copies of their later K-slices
   // wait for ring slots, and without the split the J copies wait with them.  Rows that
   // fit the ring measured slower with the split (one more wait per K-slice).
   rb->jsplit = rows_wide(g, use_lo);
@@ -1297,7 +1302,7 @@ qh_status launch_run_impl(Ctx* ctx, const Graph& g, const StepArgs& s, const Run
                           __nv_bfloat16* xh0, __nv_bfloat16* xh1, int t0, int t1,
                           unsigned long long* trace, int trace_u0, int trace_nu,
                           const RunCheck* chk) {
-  using L = RunSmem<JRES>;
+  using L = RunSmem<JRES, SB>;
   CUtensorMap mJ, mX0, mX1, mS0, mS1;
   // without checks the S maps repeat the X_hat ones (never loaded)
   __nv_bfloat16* s0 = chk ? chk->s : xh0;
@@ -1411,13 +1416,13 @@ template <bool JRES, int SB>
 static cudaError_t run_attr() {
   cudaError_t e = cudaFuncSetAttribute(k_bsb_run<JRES, SB, false, false>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)RunSmem<JRES>::BYTES);
+                                       (int)RunSmem<JRES, SB>::BYTES);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_bsb_run<JRES, SB, false, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RunSmem<JRES>::BYTES);
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RunSmem<JRES, SB>::BYTES);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_bsb_run<JRES, SB, true, false>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RunSmem<JRES>::BYTES);
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RunSmem<JRES, SB>::BYTES);
   return e;
 }
 
