@@ -56,10 +56,13 @@ __global__ void k_cov_count(int64_t nnz, const int32_t* __restrict__ snp, int32_
 }
 
 // Warp per fragment, the lanes taking its entries in parallel: the order within a SNP's
-// list is set afterwards by k_cov_sort.
+// list is set afterwards by k_cov_sort.  cov_pos (SNP mode, else nullptr): the SNP's
+// position inside the fragment, so that its rows need no search for it; the alleles are
+// for the voting (READ mode).
 __global__ void k_cov_fill(int32_t m, const int64_t* __restrict__ fp, const int32_t* __restrict__ snp,
                            const int8_t* __restrict__ allele, const int64_t* __restrict__ cov_ptr,
-                           int32_t* cursor, int32_t* cov_frag, int8_t* cov_allele) {
+                           int32_t* cursor, int32_t* cov_frag, int8_t* cov_allele,
+                           int32_t* cov_pos) {
   const int64_t i64 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   if (i64 >= m) return;
   const int32_t i = (int32_t)i64;
@@ -67,17 +70,22 @@ __global__ void k_cov_fill(int32_t m, const int64_t* __restrict__ fp, const int3
     int32_t s = snp[k];
     int64_t slot = cov_ptr[s] + atomicAdd(&cursor[s], 1);
     cov_frag[slot] = i;
-    cov_allele[slot] = allele[k];
+    if (cov_pos != nullptr)
+      cov_pos[slot] = (int32_t)(k - fp[i]);
+    else
+      cov_allele[slot] = allele[k];
   }
 }
 
-// Sort each SNP's covering list by fragment index.  Warp per SNP: lists of up to
-// 256 entries are sorted in the warp's shared-memory slice (bitonic, keys
-// fragment << 8 | allele); longer ones (rare) by lane 0 in place.
+// Sort each SNP's covering list by fragment index, each entry with its allele or (cov_pos
+// != nullptr) its position.  Warp per SNP: lists of up to 256 entries are sorted in the
+// warp's shared-memory slice (bitonic, keys fragment << 32 | payload); longer ones (rare)
+// by lane 0 in place.
 constexpr int COV_SORT_MAX = 256;
 
 __global__ void __launch_bounds__(256) k_cov_sort(int32_t n, const int64_t* __restrict__ cov_ptr,
-                                                  int32_t* cov_frag, int8_t* cov_allele) {
+                                                  int32_t* cov_frag, int8_t* cov_allele,
+                                                  int32_t* cov_pos) {
   __shared__ int64_t keys[8][COV_SORT_MAX];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int32_t s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -90,7 +98,9 @@ __global__ void __launch_bounds__(256) k_cov_sort(int32_t n, const int64_t* __re
     while (N < len) N <<= 1;
     int64_t* k = keys[w];
     for (int i = lane; i < N; i += 32)
-      k[i] = i < len ? (((int64_t)cov_frag[b + i] << 8) | (int64_t)(uint8_t)(cov_allele[b + i] + 1))
+      k[i] = i < len ? (((int64_t)cov_frag[b + i] << 32) |
+                        (cov_pos != nullptr ? (int64_t)cov_pos[b + i]
+                                            : (int64_t)(uint8_t)(cov_allele[b + i] + 1)))
                      : INT64_MAX;
     __syncwarp();
     for (int kk = 2; kk <= N; kk <<= 1) {
@@ -110,23 +120,32 @@ __global__ void __launch_bounds__(256) k_cov_sort(int32_t n, const int64_t* __re
       }
     }
     for (int i = lane; i < len; i += 32) {
-      cov_frag[b + i] = (int32_t)(k[i] >> 8);
-      cov_allele[b + i] = (int8_t)((int32_t)(k[i] & 0xff) - 1);
+      cov_frag[b + i] = (int32_t)(k[i] >> 32);
+      if (cov_pos != nullptr)
+        cov_pos[b + i] = (int32_t)(k[i] & 0xffffffff);
+      else
+        cov_allele[b + i] = (int8_t)((int32_t)(k[i] & 0xff) - 1);
     }
     return;
   }
   if (lane != 0) return;
   for (int64_t i = b + 1; i < e; ++i) {
-    int32_t f = cov_frag[i];
-    int8_t a = cov_allele[i];
+    const int32_t f = cov_frag[i];
+    const int32_t v = cov_pos != nullptr ? cov_pos[i] : cov_allele[i];
     int64_t j = i - 1;
     while (j >= b && cov_frag[j] > f) {
       cov_frag[j + 1] = cov_frag[j];
-      cov_allele[j + 1] = cov_allele[j];
+      if (cov_pos != nullptr)
+        cov_pos[j + 1] = cov_pos[j];
+      else
+        cov_allele[j + 1] = cov_allele[j];
       --j;
     }
     cov_frag[j + 1] = f;
-    cov_allele[j + 1] = a;
+    if (cov_pos != nullptr)
+      cov_pos[j + 1] = v;
+    else
+      cov_allele[j + 1] = (int8_t)v;
   }
 }
 
@@ -284,30 +303,226 @@ struct SnpRowSmem {
   double val[SNP_ROW_CAP];
 };
 
-// The small kernel's capacities: a dense window of this many SNPs, else this many
-// fragment terms on the sorted path (both fit its 32 KB of shared memory).
-constexpr int SNP_SMALL_CAP = 2048;
-constexpr int SNP_SMALL_TERMS = 2048;
-constexpr size_t SNP_SMALL_SMEM = (size_t)SNP_SMALL_TERMS * 16;
+// Warp per SNP row u.  PASS 0: count distinct partners; PASS 1: write (v, w_uv).  The terms
+// of a partner are summed in fragment order from 0, as in the CTA kernel below.
+//  * The covering fragments come 32 at a time, a lane each (extent, u's position in it from
+//    the coverage list, reciprocal of |S| - 1), and are then taken one after the other, the
+//    lanes striding over a fragment's partners, which are distinct.
+//  * Partners within SNP_NEAR / 2 of u sum into a dense window in shared memory.  The
+//    others (long-range contacts) go into a list of SNP_FAR terms, sorted by (partner,
+//    fragment) at the end; a partner is always on one side of that line.
+//  * A row with more far terms, or with more terms than the CTA kernel's sort path takes
+//    (which alone says whether its window is small enough), is deferred to the CTA kernel.
+// Bound by FP64 and by the latency of the terms' loads.  GB300's FP64 rate makes a division
+// per term the largest cost of the fill: the divisor is a fragment's, so the quotient is
+// taken from its correctly rounded reciprocal (snp_quotient, the same bits).  Measured,
+// both passes, against a CTA per row with a search for u and a barrier per fragment, and a
+// 2,048-element sort for rows with contacts: 12,000 SNPs (468 neighbours)
+// 2.00 -> 0.88 ms; 50,000 SNPs with 500,000 Pore-C contacts 15.0 -> 2.96 ms (and 0.23 ms for
+// the rows with more contacts).
+constexpr int SNP_NEAR = 1024;
+constexpr int SNP_FAR = 256;
+constexpr int SNP_WARPS = 4;
 
-// CTA per SNP row u.  PASS 0: count distinct partners; PASS 1: write (v, w_uv).
-// A row with a narrow window of covered SNPs sums into a dense window; otherwise its
-// fragment terms are gathered and sorted by (partner, fragment).  SMALL: capacities
-// SNP_SMALL_CAP / SNP_SMALL_TERMS in a small shared-memory footprint (many CTAs per
-// SM); a row over them is appended to `defer` in PASS 0 and left to the large kernel
-// (SNP_DENSE_CAP / SNP_ROW_CAP), which walks the deferred rows (`rows`, `n_list` of
-// them).  Every path sums a partner's terms in fragment order: the same weights.
-template <int PASS, bool SMALL>
-__global__ void __launch_bounds__(SMALL ? 256 : 512) k_snp_rows(
+struct SnpWarpSmem {
+  double acc[SNP_NEAR];
+  uint64_t key[SNP_FAR];  // (partner SNP << 32) | fragment
+  double val[SNP_FAR];
+  uint8_t touched[SNP_NEAR];
+};
+
+// x / d for a divisor d with correctly rounded reciprocal y = RN(1 / d): q = RN(x y), the
+// remainder r = x - q d is exact in an FMA, and RN(q + r y) is the correctly rounded
+// quotient (P. Markstein, "Computation of elementary functions on the IBM RISC System/6000
+// processor", IBM J. Res. Dev. 34, 1990; "one multiplication and two fused MACs" in
+// Brisebarre, Muller & Raina, IEEE Trans. Comput. 53, 2004), as long as nothing over- or
+// underflows: `plain` takes the division.
+__device__ __forceinline__ double snp_quotient(double x, double d, double y, bool plain) {
+  if (plain) return x / d;
+  const double q = __dmul_rn(x, y);
+  return __fma_rn(__fma_rn(-q, d, x), y, q);
+}
+
+template <int PASS>
+__global__ void __launch_bounds__(32 * SNP_WARPS) k_snp_rows_warp(
     int32_t n, const int64_t* __restrict__ fp, const int32_t* __restrict__ snp,
+    const int8_t* __restrict__ allele, const uint8_t* __restrict__ qual,
+    const uint8_t* __restrict__ is_porec, const int64_t* __restrict__ cov_ptr,
+    const int32_t* __restrict__ cov_frag, const int32_t* __restrict__ cov_pos,
+    const double* __restrict__ L, double alpha, int linkage_k, int64_t* cnt,
+    const int64_t* __restrict__ row_ptr, int32_t* col, double* w, int32_t* defer,
+    int32_t* n_defer) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SnpWarpSmem& sm = reinterpret_cast<SnpWarpSmem*>(smem_raw)[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const int64_t u64 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (u64 >= n) return;
+  const int32_t u = (int32_t)u64;
+  const bool plain = !(alpha == 0.0 || (alpha >= 1e-200 && alpha <= 1e200));
+  for (int t = lane; t < SNP_NEAR; t += 32) {
+    if (PASS == 1) sm.acc[t] = 0.0;
+    sm.touched[t] = 0;
+  }
+  __syncwarp();
+  const int64_t cb = cov_ptr[u], ce = cov_ptr[u + 1];
+  const int32_t near0 = u - SNP_NEAR / 2;
+  int32_t n_far = 0;
+  int64_t terms = 0;
+  for (int64_t c0 = cb; c0 < ce; c0 += 32) {
+    const int cn = (int)(ce - c0 < 32 ? ce - c0 : 32);
+    // lane c: covering fragment c0 + c
+    int64_t fb = 0;
+    int32_t frag = 0, p = 0, lo = 0, hi = -1;
+    double d = 1.0, y = 1.0, a = 1.0;
+    int qu = 0, au = 1;
+    if (lane < cn) {
+      frag = cov_frag[c0 + lane];
+      p = cov_pos[c0 + lane];
+      fb = fp[frag];
+      const int32_t S = (int32_t)(fp[frag + 1] - fb);
+      const int32_t depth = (int32_t)(((int64_t)linkage_k * (S - 1)) / 10);
+      lo = max(0, p - depth);
+      hi = min(S - 1, p + depth);
+      terms += hi - lo;
+      if (PASS == 1) {
+        d = (double)(S - 1);
+        y = S > 1 ? 1.0 / d : 0.0;
+        a = is_porec[frag] ? alpha : 1.0;
+        qu = qual[fb + p];
+        au = allele[fb + p];
+      }
+    }
+    for (int c = 0; c < cn; ++c) {
+      const int64_t fbc = __shfl_sync(0xffffffffu, fb, c);
+      const int32_t pc = __shfl_sync(0xffffffffu, p, c), loc = __shfl_sync(0xffffffffu, lo, c),
+                    hic = __shfl_sync(0xffffffffu, hi, c),
+                    fragc = __shfl_sync(0xffffffffu, frag, c);
+      double dc = 1.0, yc = 1.0, ac = 1.0;
+      int quc = 0, auc = 1;
+      if (PASS == 1) {
+        dc = __shfl_sync(0xffffffffu, d, c);
+        yc = __shfl_sync(0xffffffffu, y, c);
+        ac = __shfl_sync(0xffffffffu, a, c);
+        quc = __shfl_sync(0xffffffffu, qu, c);
+        auc = __shfl_sync(0xffffffffu, au, c);
+      }
+      for (int32_t pp0 = loc; pp0 <= hic; pp0 += 32) {
+        const int32_t pp = pp0 + lane;
+        const bool on = pp <= hic && pp != pc;
+        int32_t v = u;
+        double term = 0.0;
+        if (on) {
+          const int64_t ev = fbc + pp;
+          v = snp[ev];
+          if (PASS == 1) {
+            const double lv = L[quc * 94 + (int)qual[ev]];
+            const double q = snp_quotient(ac == 1.0 ? lv : __dmul_rn(ac, lv), dc, yc, plain);
+            term = auc * (int)allele[ev] > 0 ? -q : q;
+          }
+        }
+        const int32_t k = v - near0;
+        const bool near = (uint32_t)k < (uint32_t)SNP_NEAR;
+        if (on && near) {
+          sm.touched[k] = 1;
+          if (PASS == 1) sm.acc[k] = __dadd_rn(sm.acc[k], term);
+        }
+        const uint32_t far = __ballot_sync(0xffffffffu, on && !near);
+        if (far != 0) {
+          const int32_t at = n_far + __popc(far & ((1u << lane) - 1u));
+          if (on && !near && at < SNP_FAR) {
+            sm.key[at] = ((uint64_t)(uint32_t)v << 32) | (uint32_t)fragc;
+            sm.val[at] = term;
+          }
+          n_far += __popc(far);
+        }
+      }
+      __syncwarp();  // the next fragment's terms go on top of this one's
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) terms += __shfl_xor_sync(0xffffffffu, terms, off);
+  if (n_far > SNP_FAR || terms > SNP_ROW_CAP) {  // the CTA kernel's row
+    if (PASS == 0 && lane == 0) defer[atomicAdd(n_defer, 1)] = u;
+    return;
+  }
+  // sort the far terms by (partner, fragment)
+  int32_t N = 1;
+  while (N < n_far) N <<= 1;
+  for (int32_t t = n_far + lane; t < N; t += 32) sm.key[t] = ~0ull;
+  __syncwarp();
+  for (int32_t k = 2; k <= N; k <<= 1)
+    for (int32_t j = k >> 1; j > 0; j >>= 1) {
+      for (int32_t t = lane; t < N; t += 32) {
+        const int32_t l = t ^ j;
+        if (l > t) {
+          const uint64_t ka = sm.key[t], kb = sm.key[l];
+          if ((ka > kb) == ((t & k) == 0)) {
+            sm.key[t] = kb;
+            sm.key[l] = ka;
+            if (PASS == 1) {
+              const double va = sm.val[t];
+              sm.val[t] = sm.val[l];
+              sm.val[l] = va;
+            }
+          }
+        }
+      }
+      __syncwarp();
+    }
+  // partners in ascending order: far below u, near, far above u
+  int64_t out = PASS == 1 ? row_ptr[u] : 0;
+  int32_t total = 0;
+  auto far_runs = [&](int32_t f0, int32_t f1) {
+    for (int32_t t0 = f0; t0 < f1; t0 += 32) {
+      const int32_t t = t0 + lane;
+      const bool start = t < f1 && (t == f0 || (sm.key[t] >> 32) != (sm.key[t - 1] >> 32));
+      const uint32_t m = __ballot_sync(0xffffffffu, start);
+      if (PASS == 1 && start) {
+        const uint32_t v = (uint32_t)(sm.key[t] >> 32);
+        double sum = 0.0;
+        for (int32_t q = t; q < f1 && (uint32_t)(sm.key[q] >> 32) == v; ++q)
+          sum = __dadd_rn(sum, sm.val[q]);
+        const int64_t o = out + total + __popc(m & ((1u << lane) - 1u));
+        col[o] = (int32_t)v;
+        w[o] = sum;
+      }
+      total += __popc(m);
+    }
+  };
+  int32_t below = 0;
+  for (int32_t t0 = 0; t0 < n_far; t0 += 32)
+    below += __popc(__ballot_sync(0xffffffffu,
+                                  t0 + lane < n_far && (sm.key[t0 + lane] >> 32) < (uint32_t)u));
+  far_runs(0, below);
+  for (int t0 = 0; t0 < SNP_NEAR; t0 += 32) {
+    const bool on = sm.touched[t0 + lane] != 0;
+    const uint32_t m = __ballot_sync(0xffffffffu, on);
+    if (PASS == 1 && on) {
+      const int64_t o = out + total + __popc(m & ((1u << lane) - 1u));
+      col[o] = near0 + t0 + lane;
+      w[o] = sm.acc[t0 + lane];
+    }
+    total += __popc(m);
+  }
+  far_runs(below, n_far);
+  if (PASS == 0 && lane == 0) cnt[u] = total;
+}
+
+// The rows k_snp_rows_warp deferred (`rows`, *n_list of them), a CTA each.  PASS 0: count
+// distinct partners; PASS 1: write (v, w_uv).  A row whose covered window is at most
+// SNP_DENSE_CAP sums into a dense window; otherwise its fragment terms are gathered and
+// sorted by (partner, fragment), at most SNP_ROW_CAP of them.  Both sum a partner's terms
+// in fragment order.
+template <int PASS>
+__global__ void __launch_bounds__(512) k_snp_rows(
+    const int64_t* __restrict__ fp, const int32_t* __restrict__ snp,
     const int8_t* __restrict__ allele, const uint8_t* __restrict__ qual,
     const uint8_t* __restrict__ is_porec, const int64_t* __restrict__ cov_ptr,
     const int32_t* __restrict__ cov_frag, const double* __restrict__ L, double alpha,
     int linkage_k, int64_t* cnt, const int64_t* __restrict__ row_ptr, int32_t* col, double* w,
-    int32_t* err, const int32_t* __restrict__ rows, const int32_t* __restrict__ n_list,
-    int32_t* defer, int32_t* n_defer) {
-  constexpr int DCAP = SMALL ? SNP_SMALL_CAP : SNP_DENSE_CAP;
-  constexpr int TCAP = SMALL ? SNP_SMALL_TERMS : SNP_ROW_CAP;
+    int32_t* err, const int32_t* __restrict__ rows, const int32_t* __restrict__ n_list) {
+  constexpr int DCAP = SNP_DENSE_CAP;
+  constexpr int TCAP = SNP_ROW_CAP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int32_t s_total;
   __shared__ int32_t s_runs[32];
@@ -315,9 +530,9 @@ __global__ void __launch_bounds__(SMALL ? 256 : 512) k_snp_rows(
   __shared__ int32_t s_off[1025];
   uint64_t* skey = reinterpret_cast<uint64_t*>(smem_raw);       // sorted path: TCAP keys
   double* sval = reinterpret_cast<double*>(smem_raw) + TCAP;    // and their terms
-  const int32_t count = rows != nullptr ? *n_list : n;
+  const int32_t count = *n_list;
   for (int32_t ri = blockIdx.x; ri < count; ri += gridDim.x) {
-    const int32_t u = rows != nullptr ? rows[ri] : ri;
+    const int32_t u = rows[ri];
     int64_t cb = cov_ptr[u], ce = cov_ptr[u + 1];
     int32_t ncov = (int32_t)(ce - cb);
     // SNP window spanned by the covering fragments
@@ -437,8 +652,8 @@ __global__ void __launch_bounds__(SMALL ? 256 : 512) k_snp_rows(
       }
       __syncthreads();
       int32_t tot = s_off[cn];
-      if (base + tot > TCAP) {  // small kernel: the large kernel's row; large: error
-        if (threadIdx.x == 0 && !SMALL) atomicOr(err, ERR_ROWCAP);
+      if (base + tot > TCAP) {
+        if (threadIdx.x == 0) atomicOr(err, ERR_ROWCAP);
         base = TCAP + 1;
         __syncthreads();
         break;
@@ -477,11 +692,7 @@ __global__ void __launch_bounds__(SMALL ? 256 : 512) k_snp_rows(
       __syncthreads();
     }
     if (base > TCAP) {
-      if (SMALL) {
-        if (PASS == 0 && threadIdx.x == 0) defer[atomicAdd(n_defer, 1)] = u;
-      } else if (PASS == 0 && threadIdx.x == 0) {
-        cnt[u] = 0;
-      }
+      if (PASS == 0 && threadIdx.x == 0) cnt[u] = 0;
       __syncthreads();
       continue;
     }
@@ -689,13 +900,13 @@ __global__ void k_perm_local(int64_t total, const uint64_t* __restrict__ keys,
 
 // ------------------------------------------------------------------ tiles
 // Warp per vertex, the lanes striding over its row: flags[slot] = 1 for a 128 x 128 tile
-// with an edge, halves[slot] = its 64-column halves that hold one (bit per half).  Most
-// entries of a row fall into halves that are marked already: the mark is read first.
+// with an edge, halves[2 slot + h] = 1 for its 64-column half h with one.  Most entries of
+// a row fall into halves that are marked already: the mark is read first.
 __global__ void k_tile_flags(int32_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                              const double* __restrict__ w, const int32_t* __restrict__ block_of,
                              const int32_t* __restrict__ local, const int64_t* __restrict__ slot_off,
                              const int32_t* __restrict__ tiles_per_block, int32_t* flags,
-                             uint32_t* halves) {
+                             uint8_t* halves) {
   const int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (a >= n) return;
@@ -706,10 +917,10 @@ __global__ void k_tile_flags(int32_t n, const int64_t* __restrict__ rp, const in
     if (w[e] == 0.0) continue;
     const int32_t l = local[col[e]];
     const int64_t slot = s0 + l / TILE;
-    const uint32_t bit = 1u << (l % TILE / 64);
-    if ((halves[slot] & bit) == 0) {
+    uint8_t* half = halves + 2 * slot + l % TILE / 64;
+    if (*half == 0) {  // every writer stores the same value
       flags[slot] = 1;
-      atomicOr(halves + slot, bit);
+      *half = 1;
     }
   }
 }
@@ -956,6 +1167,7 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
   if (herr & ERR_QUAL) return set_err(ctx, QH_EINVAL, "Phred quality outside [4, 93]");
   QH_STAGE_CHECK("graph build: validate");
   // ---- SNP -> fragment coverage lists (used by SNP rows and by voting)
+  int32_t* cov_pos = nullptr;  // SNP mode: the SNP's position in the fragment
   {
     int32_t* cnt = (int32_t*)ctx->scratch(sizeof(int32_t) * (n + 1), 0);
     if (!cnt) return set_err(ctx, QH_ENOMEM, "allocation failed (coverage)");
@@ -964,13 +1176,18 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
     g->cov_ptr = (int64_t*)dalloc(*g, sizeof(int64_t) * (n + 1));
     g->cov_frag = (int32_t*)dalloc(*g, sizeof(int32_t) * std::max<int64_t>(nnz_f, 1));
     g->cov_allele = (int8_t*)dalloc(*g, std::max<int64_t>(nnz_f, 1));
+    if (o->mode == QH_MODE_SNP) {
+      cov_pos = (int32_t*)ctx->scratch(sizeof(int32_t) * (size_t)std::max<int64_t>(nnz_f, 1), 26);
+      if (!cov_pos) return set_err(ctx, QH_ENOMEM, "allocation failed (coverage)");
+    }
     if (!g->cov_ptr || !g->cov_frag || !g->cov_allele) return set_err(ctx, QH_ENOMEM, "allocation failed (coverage)");
     if (!scan_i32_to_i64(ctx, s, cnt, g->cov_ptr, n)) return set_err(ctx, QH_ENOMEM, "allocation failed (scan)");
     QH_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (n + 1), s));
     if (m > 0)
       k_cov_fill<<<::qh::counted(nblk((int64_t)m * 32)), 256, 0, s>>>(m, g->frag_ptr, g->snp, g->allele, g->cov_ptr, cnt,
-                                         g->cov_frag, g->cov_allele);
-    if (n > 0) k_cov_sort<<<::qh::counted(nblk((int64_t)n * 32)), 256, 0, s>>>(n, g->cov_ptr, g->cov_frag, g->cov_allele);
+                                         g->cov_frag, g->cov_allele, cov_pos);
+    if (n > 0) k_cov_sort<<<::qh::counted(nblk((int64_t)n * 32)), 256, 0, s>>>(n, g->cov_ptr, g->cov_frag, g->cov_allele,
+                                                                           cov_pos);
   }
   QH_STAGE_CHECK("graph build: coverage lists");
   // ---- edges
@@ -1015,30 +1232,28 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
     if (!L || !cnt) return set_err(ctx, QH_ENOMEM, "allocation failed (SNP graph scratch)");
     k_llr_table<<<::qh::counted(94), 94, 0, s>>>(L);
     QH_CUDA_TRY(cudaMemsetAsync(ctx->d_err, 0, sizeof(int32_t), s));
-    // rows whose covered window is narrow go to the small-footprint kernel (many CTAs
-    // per SM); the others are deferred to the large kernel
     const size_t smem = sizeof(SnpRowSmem);
-    const size_t smem_s = SNP_SMALL_SMEM;
-    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_s));
-    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_s));
-    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const unsigned grid = (unsigned)std::max(1, std::min(n, ctx->n_sm * 4));
-    const unsigned grid_s = (unsigned)std::max(1, std::min(n, ctx->n_sm * 16));
+    const size_t smem_w = sizeof(SnpWarpSmem) * SNP_WARPS;
+    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows_warp<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w));
+    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows_warp<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w));
+    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const unsigned grid = (unsigned)std::max(1, std::min(n, ctx->n_sm));
+    const unsigned grid_w = (unsigned)((n + SNP_WARPS - 1) / SNP_WARPS);
     int32_t* defer = (int32_t*)ctx->scratch(sizeof(int32_t) * (n + 1), 23);
     g->row_ptr = (int64_t*)dalloc(*g, sizeof(int64_t) * (n + 1));
     if (!g->row_ptr || !defer) return set_err(ctx, QH_ENOMEM, "allocation failed (edges)");
     int32_t* n_defer = defer + n;
     QH_CUDA_TRY(cudaMemsetAsync(n_defer, 0, sizeof(int32_t), s));
     if (n > 0) {
-      k_snp_rows<0, true><<<::qh::counted(grid_s), 256, smem_s, s>>>(
-          n, g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, L,
-          o->porec_alpha, o->linkage_k, cnt, nullptr, nullptr, nullptr, ctx->d_err, nullptr,
-          nullptr, defer, n_defer);
-      k_snp_rows<0, false><<<::qh::counted(grid), 512, smem, s>>>(
-          n, g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, L,
+      k_snp_rows_warp<0><<<::qh::counted(grid_w), 32 * SNP_WARPS, smem_w, s>>>(
+          n, g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag,
+          cov_pos, L, o->porec_alpha, o->linkage_k, cnt, nullptr, nullptr, nullptr, defer,
+          n_defer);
+      k_snp_rows<0><<<::qh::counted(grid), 512, smem, s>>>(
+          g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, L,
           o->porec_alpha, o->linkage_k, cnt, nullptr, nullptr, nullptr, ctx->d_err, defer,
-          n_defer, nullptr, nullptr);
+          n_defer);
     }
     if (!scan_i64(ctx, s, cnt, g->row_ptr, n)) return set_err(ctx, QH_ENOMEM, "allocation failed (scan)");
     QH_CUDA_TRY(cudaMemcpyAsync(&g->nnz, g->row_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
@@ -1050,14 +1265,14 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
     g->w = (double*)dalloc(*g, sizeof(double) * std::max<int64_t>(g->nnz, 1));
     if (!g->col || !g->w) return set_err(ctx, QH_ENOMEM, "allocation failed (edges)");
     if (n > 0 && g->nnz > 0) {
-      k_snp_rows<1, true><<<::qh::counted(grid_s), 256, smem_s, s>>>(
-          n, g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, L,
-          o->porec_alpha, o->linkage_k, nullptr, g->row_ptr, g->col, g->w, ctx->d_err, nullptr,
-          nullptr, nullptr, nullptr);
-      k_snp_rows<1, false><<<::qh::counted(grid), 512, smem, s>>>(
-          n, g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, L,
+      k_snp_rows_warp<1><<<::qh::counted(grid_w), 32 * SNP_WARPS, smem_w, s>>>(
+          n, g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag,
+          cov_pos, L, o->porec_alpha, o->linkage_k, nullptr, g->row_ptr, g->col, g->w, nullptr,
+          nullptr);
+      k_snp_rows<1><<<::qh::counted(grid), 512, smem, s>>>(
+          g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, L,
           o->porec_alpha, o->linkage_k, nullptr, g->row_ptr, g->col, g->w, ctx->d_err, defer,
-          n_defer, nullptr, nullptr);
+          n_defer);
     }
   }
   const int32_t N = g->n_nodes;
@@ -1151,7 +1366,7 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
   int32_t* d_T = (int32_t*)ctx->scratch(sizeof(int32_t) * std::max(nb, 1), 18);
   int32_t* flags = (int32_t*)ctx->scratch(sizeof(int32_t) * std::max<int64_t>(n_slots, 1), 19);
   int64_t* slot_tile = (int64_t*)ctx->scratch(sizeof(int64_t) * (n_slots + 1), 20);
-  uint32_t* halves = (uint32_t*)ctx->scratch(4 * (size_t)std::max<int64_t>(n_slots, 1), 25);
+  uint8_t* halves = (uint8_t*)ctx->scratch(2 * (size_t)std::max<int64_t>(n_slots, 1), 25);
   if (!g->block_ptr || !g->pad_off || !g->perm || !g->pad_node || !d_slot_off || !d_T || !flags ||
       !slot_tile || !halves)
     return set_err(ctx, QH_ENOMEM, "allocation failed (layout)");
@@ -1177,7 +1392,7 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
     QH_CUDA_TRY(cudaStreamSynchronize(s));
   } else {
     QH_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int32_t) * std::max<int64_t>(n_slots, 1), s));
-    QH_CUDA_TRY(cudaMemsetAsync(halves, 0, 4 * (size_t)std::max<int64_t>(n_slots, 1), s));
+    QH_CUDA_TRY(cudaMemsetAsync(halves, 0, 2 * (size_t)std::max<int64_t>(n_slots, 1), s));
     if (N > 0)
       k_tile_flags<<<::qh::counted(nblk((int64_t)N * 32)), 256, 0, s>>>(N, g->row_ptr, g->col, g->w, g->block_of, g->local,
                                           d_slot_off, d_T, flags, halves);
@@ -1186,11 +1401,11 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
   std::vector<int64_t> h_slot_tile(n_slots + 1);
   // the tiles' halves come with the slots, unless there are so many slots that the
   // storage (CSR needs no halves) is better known first
-  std::vector<uint32_t> h_halves;
+  std::vector<uint8_t> h_halves;
   auto fetch_halves = [&]() -> cudaError_t {
-    h_halves.assign((size_t)n_slots, 3u);  // dense mode: both
+    h_halves.assign(2 * (size_t)n_slots, 1);  // dense mode: both
     if (o->dense || n_slots == 0) return cudaSuccess;
-    return cudaMemcpyAsync(h_halves.data(), halves, 4 * (size_t)n_slots, cudaMemcpyDeviceToHost, s);
+    return cudaMemcpyAsync(h_halves.data(), halves, 2 * (size_t)n_slots, cudaMemcpyDeviceToHost, s);
   };
   const bool halves_later = n_slots > 65536;
   if (!halves_later) QH_CUDA_TRY(fetch_halves());
@@ -1238,9 +1453,9 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
       for (int rep = 0; rep < (g->has_lo ? 2 : 1); ++rep) {
         for (size_t j = 0; j < cols.size(); ++j) {
           const uint32_t e = (uint32_t)(entry + rep * (int64_t)cols.size() + (int64_t)j);
-          const uint32_t m = h_halves[s0 + (cols[j] - ct0)];
+          const uint8_t* m = &h_halves[2 * (size_t)(s0 + (cols[j] - ct0))];
           for (uint32_t half = 0; half < 2; ++half)
-            if ((m >> half) & 1u)
+            if (m[half])
               h_kslice.push_back(KSlice{2 * e + half, 2 * (uint32_t)cols[j] + half});
         }
         if (rep == 0) rt.nk_hi = (int32_t)h_kslice.size() - rt.ks_begin;
