@@ -3,6 +3,7 @@
 //    GPU bSB), exact cut evaluation, replica selection, early stop,
 //  - SNP refinement (flip counter, sign inversion), read voting, parity swap.
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "qh_internal.cuh"
@@ -783,9 +784,10 @@ __global__ void k_cut_nodes(int32_t n, const int64_t* __restrict__ rp, const int
   }
 }
 
-// Real weights, at most 4 replicas (the final parity cut): FP64, the lanes of the
-// vertex's warp stride over its edges and the partial sums are combined in a fixed
-// shuffle order, so the result does not depend on scheduling.
+// Real weights, at most 4 replicas (the final parity cut), or a weight range that fixed
+// point cannot scale (grid.y = groups of four replicas): FP64, the lanes of the vertex's
+// warp stride over its edges and the partial sums are combined in a fixed shuffle order,
+// so the result does not depend on scheduling.
 __global__ void k_cut_nodes_few(int32_t n, const int64_t* __restrict__ rp,
                                 const int32_t* __restrict__ col, const double* __restrict__ w,
                                 const int32_t* __restrict__ block_of,
@@ -797,132 +799,215 @@ __global__ void k_cut_nodes_few(int32_t n, const int64_t* __restrict__ rp,
   if (a >= n) return;
   int32_t b = block_of[a];
   if (b < 0 || (active != nullptr && !active[b])) return;
-  const int32_t pa = pad_index[a];
+  const int32_t pa = pad_index[a], r0 = 4 * (int32_t)blockIdx.y;
   const int64_t e0 = rp[a], e1 = rp[a + 1];
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
   for (int64_t e = e0 + lane; e < e1; e += 32) {
     const double we = w[e];
     if (we == 0.0) continue;  // zero edges may reach vertices outside every block
-    const int8_t* sb = st + (size_t)pad_index[col[e]] * R;
+    const int8_t* sb = st + (size_t)pad_index[col[e]] * R + r0;
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      if (k < R) acc[k] += sb[k] > 0 ? we : -we;
+      if (r0 + k < R) acc[k] += sb[k] > 0 ? we : -we;
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k)
     for (int off = 16; off > 0; off >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], off);
-  if (lane < R) {
+  if (lane < 4 && r0 + lane < R) {
     double v = acc[0];
 #pragma unroll
     for (int k = 1; k < 4; ++k)
       if (lane == k) v = acc[k];
-    node_val[(size_t)pa * R + lane] = (double)st[(size_t)pa * R + lane] * v;
+    node_val[(size_t)pa * R + r0 + lane] = (double)st[(size_t)pa * R + r0 + lane] * v;
   }
 }
 
-// Real weights over many replicas: the same per-vertex sums, accumulated in FP32 with
-// compensation.  Each weight is split into FP32 hi + lo parts, and each running sum
-// is kept as an unevaluated pair (hi, lo) updated with the exact rounding error of the
-// hi addition (Knuth's TwoSum), which carries about 48 bits: within ~1e-11 of the FP64
-// sum even over thousands of edges, at FP32 speed (this part's FP64 rate is a small
-// fraction of its FP32 rate).  Signs are +-1, so the terms are exact negations.
-template <int PER>
-__global__ void k_cut_nodes_df(int32_t n, const int64_t* __restrict__ rp,
-                               const int32_t* __restrict__ col, const double* __restrict__ w,
-                               const int32_t* __restrict__ block_of,
-                               const int32_t* __restrict__ pad_index, const int8_t* __restrict__ st,
-                               int32_t R, int32_t per, double* node_val,
-                               const int32_t* __restrict__ active) {
-  int32_t a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
+// Real weights over many replicas: the same per-vertex sums in fixed point.  A weight is
+// the integer W = rn(w scale), |W| <= 2^CUT_BITS (scale a power of two from the largest
+// |w|), as three signed base-2^16 digits held as FP32 values.  One FMA per digit adds a
+// sign's term; up to CUT_FOLD edges the digit sums stay below 2^24, where FP32 holds every
+// integer, and are then folded into a 64-bit integer: the vertex's sum is exact, and the
+// only rounding is that of the weights, 2^-47 of the largest.  Relative error of the cuts
+// against FP64 (exact summation), largest over 8 solves: 12,000 SNPs 3.8e-16, 3,000 SNPs
+// 3.8e-16 (compensated FP32 sums, which this replaces: 4.8e-15 and 9.6e-15).
+// Warp per vertex, 32 edges at a time: each lane turns one weight into digits (shared
+// memory) and holds its column; a lane owns PER replicas, their signs one byte each.  us
+// per call, compensated FP32 -> now: 12,000 SNPs (5.6M entries), R = 512: 2,163 -> 815;
+// 50,000 SNPs (7.6M entries), R = 128: 1,190 -> 558.  Six base-256 digits with a DP4A
+// per four edges measured 1,127 and 624: this part's DP4A rate is low.
+constexpr int CUT_DIGITS = 3;
+constexpr int CUT_BITS = 46;
+constexpr int CUT_FOLD = 256;
+
+template <int PER, bool VEC>
+__global__ void __launch_bounds__(256) k_cut_nodes_fx(
+    int32_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
+    const double* __restrict__ w, const int32_t* __restrict__ block_of,
+    const int32_t* __restrict__ pad_index, const int8_t* __restrict__ st, int32_t R, double scale,
+    double inv_scale, double* node_val, const int32_t* __restrict__ active) {
+  static_assert(PER == 4 || PER == 8, "one or two sign words per lane");
+  constexpr int Q = PER / 4;
+  __shared__ __align__(16) float dig_all[256 / 32][CUT_DIGITS][32];
+  const int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (a >= n) return;
-  int32_t b = block_of[a];
+  const int32_t b = block_of[a];
   if (b < 0 || (active != nullptr && !active[b])) return;
+  float(*dig)[32] = dig_all[threadIdx.x >> 5];
   const int32_t pa = pad_index[a];
   const int64_t e0 = rp[a], e1 = rp[a + 1];
-  const bool vec = (R & 3) == 0;
-  for (int32_t r0 = 0; r0 < R; r0 += 32 * per) {
-    const int32_t r = r0 + per * lane;
-    const int nr = max(0, min(per, R - r));
-    float hi[PER], lo[PER];
+  for (int32_t r0 = 0; r0 < R; r0 += 32 * PER) {
+    const int32_t r = r0 + PER * lane;
+    // the signs of PER replicas of one vertex, as Q words (bytes past R: +1, unused)
+    auto signs = [&](int32_t p, uint32_t (&x)[Q]) {
+      const int8_t* sb = st + (size_t)p * R + r;
+      if (VEC && Q == 2) {
+        const uint2 v = r < R ? *reinterpret_cast<const uint2*>(sb) : make_uint2(0u, 0u);
+        x[0] = v.x;
+        x[Q - 1] = v.y;
+      } else if (VEC) {
+        x[0] = r < R ? *reinterpret_cast<const uint32_t*>(sb) : 0u;
+      } else {
 #pragma unroll
-    for (int k = 0; k < PER; ++k) hi[k] = lo[k] = 0.f;
-    auto add = [&](int k, int sg, float wh, float wl) {
-      const float th = sg > 0 ? wh : -wh, tl = sg > 0 ? wl : -wl;
-      const float s = __fadd_rn(hi[k], th);
-      const float bp = __fsub_rn(s, hi[k]);
-      const float err = __fadd_rn(__fsub_rn(hi[k], __fsub_rn(s, bp)), __fsub_rn(th, bp));
-      hi[k] = s;
-      lo[k] = __fadd_rn(lo[k], __fadd_rn(err, tl));
+        for (int q = 0; q < Q; ++q) {
+          x[q] = 0;
+          for (int k = 0; k < 4; ++k)
+            if (r + 4 * q + k < R) x[q] |= (uint32_t)(uint8_t)sb[4 * q + k] << (8 * k);
+        }
+      }
     };
-    // edges in groups of 32, as in k_cut_nodes; the terms still go in edge order
+    float2 acc[PER / 2][CUT_DIGITS];
+    long long tot[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) tot[k] = 0;
+    // the next 32 edges' weights and columns load while this group is summed; zero edges
+    // (which may reach vertices outside every block) and the row's end: W = 0, vertex 0
     double wv_n = e0 + lane < e1 ? w[e0 + lane] : 0.0;
     int32_t pv_n = wv_n != 0.0 ? pad_index[col[e0 + lane]] : 0;
-    for (int64_t eg = e0; eg < e1; eg += 32) {
-      const int ne = e1 - eg < 32 ? (int)(e1 - eg) : 32;
-      const float whv = (float)wv_n, wlv = (float)(wv_n - (double)(float)wv_n);
-      const bool nzv = wv_n != 0.0;
-      const int32_t pv = pv_n;
-      const int64_t en = eg + 32 + lane;
-      wv_n = en < e1 ? w[en] : 0.0;
-      pv_n = wv_n != 0.0 ? pad_index[col[en]] : 0;
-#pragma unroll 4
-      for (int k = 0; k < ne; ++k) {
-        const float wh = __shfl_sync(0xffffffffu, whv, k);
-        const float wl = __shfl_sync(0xffffffffu, wlv, k);
-        const int32_t p = __shfl_sync(0xffffffffu, pv, k);
-        const bool nz = __shfl_sync(0xffffffffu, (int)nzv, k) != 0;
-        // zero edges may reach vertices outside every block: skipped before any load
-        if (!nz || nr <= 0) continue;
-        const int8_t* sb = st + (size_t)p * R + r;
-        if (vec && nr == per) {
+    for (int64_t ef = e0; ef < e1; ef += CUT_FOLD) {
 #pragma unroll
-          for (int q = 0; q < PER / 4; ++q) {
-            if (4 * q >= per) break;
-            const char4 c = *reinterpret_cast<const char4*>(sb + 4 * q);
-            add(4 * q + 0, c.x, wh, wl);
-            add(4 * q + 1, c.y, wh, wl);
-            add(4 * q + 2, c.z, wh, wl);
-            add(4 * q + 3, c.w, wh, wl);
-          }
-        } else {
+      for (int k = 0; k < PER / 2; ++k)
 #pragma unroll
-          for (int k2 = 0; k2 < PER; ++k2)
-            if (k2 < nr) add(k2, sb[k2], wh, wl);
+        for (int d = 0; d < CUT_DIGITS; ++d) acc[k][d] = make_float2(0.f, 0.f);
+      const int64_t el = e1 < ef + CUT_FOLD ? e1 : ef + CUT_FOLD;
+      for (int64_t eg = ef; eg < el; eg += 32) {
+        long long W = __double2ll_rn(wv_n * scale);
+        const int32_t pv = pv_n;
+        const int64_t en = eg + 32 + lane;
+        wv_n = en < e1 ? w[en] : 0.0;
+        pv_n = wv_n != 0.0 ? pad_index[col[en]] : 0;
+        __syncwarp();  // the group before has been read
+#pragma unroll
+        for (int d = 0; d < CUT_DIGITS; ++d) {
+          const int16_t v = (int16_t)(W & 0xffff);
+          dig[d][lane] = (float)v;
+          W = (W - v) >> 16;
         }
+        __syncwarp();
+        const int ng = (int)(e1 - eg < 32 ? (e1 - eg + 3) / 4 : 8);  // groups of four edges
+#pragma unroll 2
+        for (int g = 0; g < ng; ++g) {
+          uint32_t x[4][Q];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) signs(__shfl_sync(0xffffffffu, pv, 4 * g + j), x[j]);
+          float dv[CUT_DIGITS][4];
+#pragma unroll
+          for (int d = 0; d < CUT_DIGITS; ++d) {
+            const float4 v = *reinterpret_cast<const float4*>(&dig[d][4 * g]);
+            dv[d][0] = v.x;
+            dv[d][1] = v.y;
+            dv[d][2] = v.z;
+            dv[d][3] = v.w;
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+              // +-1.0 from the byte's sign bit: its top byte 0x3f or 0xbf over 0x800000
+              const uint32_t t = (x[j][q] & 0x80808080u) | 0x3f3f3f3fu;
+              float sg[4];
+#pragma unroll
+              for (int k = 0; k < 4; ++k)
+                sg[k] = __uint_as_float(__byte_perm(t, 0x00800000u, 0x0654 | (k << 12)));
+#pragma unroll
+              for (int k = 0; k < 4; k += 2)
+#pragma unroll
+                for (int d = 0; d < CUT_DIGITS; ++d)
+                  acc[2 * q + k / 2][d] =
+                      __ffma2_rn(make_float2(dv[d][j], dv[d][j]), make_float2(sg[k], sg[k + 1]),
+                                 acc[2 * q + k / 2][d]);
+            }
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < PER; ++k) {
+        long long v = 0;
+#pragma unroll
+        for (int d = CUT_DIGITS - 1; d >= 0; --d)
+          v = v * 65536 + __float2int_rn(k & 1 ? acc[k / 2][d].y : acc[k / 2][d].x);
+        tot[k] += v;
       }
     }
     const int8_t* sa = st + (size_t)pa * R + r;
 #pragma unroll
     for (int k = 0; k < PER; ++k)
-      if (k < nr) node_val[(size_t)pa * R + r + k] = (double)sa[k] * ((double)hi[k] + (double)lo[k]);
+      if (r + k < R)
+        node_val[(size_t)pa * R + r + k] = (double)(sa[k] > 0 ? tot[k] : -tot[k]) * inv_scale;
   }
 }
 
-// CTA per (block, 32 replicas): 32 vertex slices per replica summed in a fixed
-// order, then the 32 slice sums in order: cut = (sum_w - s^T W s) / 4.
-__global__ void __launch_bounds__(1024) k_cut_reduce(int32_t nb, const int32_t* __restrict__ pad_off,
+// CTA per (32 replicas, CUT_ROWS vertices, block): 32 vertex slices per replica summed in
+// a fixed order, then the 32 slice sums in order.  A block of one chunk gets its cuts =
+// (sum_w - s^T W s) / 4 here; a larger one leaves the chunk's sum in the chunk's first row
+// of node_val (read by this CTA alone, before the barrier) for k_cut_chunks.  One CTA per
+// 32 replicas walked all vertices before: 469 us for 50,000 vertices at R = 128, 44 us
+// now with k_cut_chunks.
+constexpr int CUT_ROWS = 512;
+
+__global__ void __launch_bounds__(1024) k_cut_reduce(const int32_t* __restrict__ pad_off,
                                                      const int64_t* __restrict__ block_ptr, int32_t R,
-                                                     const double* __restrict__ node_val,
+                                                     double* node_val,
                                                      const double* __restrict__ sum_w, double* cuts,
                                                      const int32_t* __restrict__ active) {
   __shared__ double part[32][33];
-  const int32_t b = blockIdx.y;
+  const int32_t b = blockIdx.z;
   if (active != nullptr && !active[b]) return;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int32_t r = blockIdx.x * 32 + tx;
-  const int32_t p0 = pad_off[b];
   const int32_t sz = (int32_t)(block_ptr[b + 1] - block_ptr[b]);
+  const int32_t c0 = blockIdx.y * CUT_ROWS, c1 = min(sz, c0 + CUT_ROWS);
+  if (c0 >= sz) return;
+  double* nv = node_val + (size_t)pad_off[b] * R;
   double s = 0.0;
   if (r < R)
-    for (int32_t p = ty; p < sz; p += 32) s += node_val[(size_t)(p0 + p) * R + r];
+    for (int32_t p = c0 + ty; p < c1; p += 32) s += nv[(size_t)p * R + r];
   part[ty][tx] = s;
   __syncthreads();
   if (ty == 0 && r < R) {
     double t = 0.0;
     for (int k = 0; k < 32; ++k) t += part[k][tx];
-    cuts[(size_t)b * R + r] = 0.25 * (sum_w[b] - t);
+    if (sz <= CUT_ROWS)
+      cuts[(size_t)b * R + r] = 0.25 * (sum_w[b] - t);
+    else
+      nv[(size_t)c0 * R + r] = t;
   }
+}
+
+// The chunk sums of the blocks of several chunks, in order.
+__global__ void k_cut_chunks(int32_t nb, const int32_t* __restrict__ pad_off,
+                             const int64_t* __restrict__ block_ptr, int32_t R,
+                             const double* __restrict__ node_val, const double* __restrict__ sum_w,
+                             double* cuts, const int32_t* __restrict__ active) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= (int64_t)nb * R) return;
+  const int32_t b = (int32_t)(i / R), r = (int32_t)(i % R);
+  if (active != nullptr && !active[b]) return;
+  const int32_t sz = (int32_t)(block_ptr[b + 1] - block_ptr[b]);
+  if (sz <= CUT_ROWS) return;
+  double t = 0.0;
+  for (int32_t c0 = 0; c0 < sz; c0 += CUT_ROWS)
+    t += node_val[((size_t)pad_off[b] + c0) * R + r];
+  cuts[i] = 0.25 * (sum_w[b] - t);
 }
 
 // Cuts from the product z = J S of the replicas' signs (tensor cores, exact for integer
@@ -1424,20 +1509,45 @@ void launch_cut(cudaStream_t s, const Graph& g, int32_t R, const int8_t* signs_t
   int32_t per = (((R + 31) / 32) + 3) / 4 * 4;
   per = per < 4 ? 4 : (per > 32 ? 32 : per);
   // integer weights: exact int32; real weights: FP64 for a few replicas (the final
-  // parity cut), compensated FP32 for the many-replica pick
-  if (g.integer_weights)
-    k_cut_nodes<<<::qh::counted(nblk((int64_t)g.n_nodes * 32)), 256, 0, s>>>(
+  // parity cut), fixed point for the many-replica pick
+  int32_t max_n = 1;
+  for (int32_t b = 0; b < g.n_blocks; ++b) max_n = std::max(max_n, g.h_block_size[b]);
+  const unsigned warps = nblk((int64_t)g.n_nodes * 32);
+  const double m = g.max_abs_w;
+  if (g.integer_weights) {
+    k_cut_nodes<<<::qh::counted(warps), 256, 0, s>>>(
         g.n_nodes, g.row_ptr, g.col, w, g.block_of, g.pad_index, signs_t, R, per, node_val, active);
-  else if (R <= 4)
-    k_cut_nodes_few<<<::qh::counted(nblk((int64_t)g.n_nodes * 32)), 256, 0, s>>>(
+  } else if (R <= 4 || !(m > 1e-250 && m < 1e250)) {
+    const dim3 grid(warps, (unsigned)((R + 3) / 4));
+    k_cut_nodes_few<<<::qh::counted(grid), 256, 0, s>>>(
         g.n_nodes, g.row_ptr, g.col, w, g.block_of, g.pad_index, signs_t, R, node_val, active);
-  else  // at most 8 replicas per lane: 16 accumulators, more warps in flight
-    k_cut_nodes_df<8><<<::qh::counted(nblk((int64_t)g.n_nodes * 32)), 256, 0, s>>>(
-        g.n_nodes, g.row_ptr, g.col, w, g.block_of, g.pad_index, signs_t, R, per < 8 ? per : 8,
-        node_val, active);
-  dim3 grid((R + 31) / 32, g.n_blocks);
-  k_cut_reduce<<<::qh::counted(grid), 1024, 0, s>>>(g.n_blocks, g.pad_off, g.block_ptr, R, node_val, sum_w, cuts,
-                                     active);
+  } else {
+    // |w| scale < 2^bits, and a row of the largest block stays below 2^62
+    int bits = CUT_BITS, lg = 0;
+    while ((1 << lg) < max_n && lg < 30) ++lg;
+    bits = std::min(bits, 62 - lg);
+    const int ex = bits - 1 - std::ilogb(m);
+    const double sc = std::ldexp(1.0, ex), inv = std::ldexp(1.0, -ex);
+#define QH_CUT_FX(PER, VEC)                                                                    \
+  k_cut_nodes_fx<PER, VEC><<<::qh::counted(warps), 256, 0, s>>>(g.n_nodes, g.row_ptr, g.col, w, \
+                                                                g.block_of, g.pad_index,       \
+                                                                signs_t, R, sc, inv, node_val, \
+                                                                active)
+    // eight replicas a lane when they fill the warp
+    if (R % 8 == 0 && R >= 256)
+      QH_CUT_FX(8, true);
+    else if (R % 4 == 0)
+      QH_CUT_FX(4, true);
+    else
+      QH_CUT_FX(4, false);
+#undef QH_CUT_FX
+  }
+  const dim3 grid((R + 31) / 32, (max_n + CUT_ROWS - 1) / CUT_ROWS, g.n_blocks);
+  k_cut_reduce<<<::qh::counted(grid), 1024, 0, s>>>(g.pad_off, g.block_ptr, R, node_val, sum_w,
+                                                    cuts, active);
+  if (max_n > CUT_ROWS)
+    k_cut_chunks<<<::qh::counted(nblk((int64_t)g.n_blocks * R)), 256, 0, s>>>(
+        g.n_blocks, g.pad_off, g.block_ptr, R, node_val, sum_w, cuts, active);
 }
 
 void launch_cut_from_product(cudaStream_t s, const Graph& g, int32_t R, const float* z,
