@@ -123,8 +123,7 @@ struct SolveBufs {
 qh_status run_step(Ctx* ctx, const Graph& g, int precision, const TcPlan& plan, StepArgs a,
                    const float* x_cur_f32, float* x_next_f32, const __nv_bfloat16* xh_cur,
                    __nv_bfloat16* xh_next, const Fp8Operands* f8 = nullptr, int64_t ns = 0,
-                   float* zband = nullptr, const F32Chunks& f32 = F32Chunks(),
-                   bool after_step = false) {
+                   float* zband = nullptr, const F32Chunks& f32 = F32Chunks()) {
   if (precision == QH_PREC_FP8) {  // X_hat buffers hold the e4m3 hi part, then the lo part
     Fp8Operands op = *f8;
     op.xh_in = reinterpret_cast<const uint8_t*>(xh_cur);
@@ -139,7 +138,7 @@ qh_status run_step(Ctx* ctx, const Graph& g, int precision, const TcPlan& plan, 
     if (g.csr_mode)
       launch_step_csr(ctx->stream, g, a, g.pval, nullptr, plan.variant);
     else
-      return launch_step_f32(ctx, g, a, f32, after_step);
+      return launch_step_f32(ctx, g, a, f32);
     return QH_OK;
   }
   a.xh_out = xh_next;
@@ -846,6 +845,13 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
   a.dta0 = (float)(o->dt * o->a0);
   a.err = ctx->d_err;
   a.sb = o->sb_variant;
+  {  // the schedule lengths: one, or the AUTO schedule's two
+    int32_t len0 = h_steps[0], len1 = 0;
+    for (int32_t v : h_steps)
+      if (v != len0) len1 = v;
+    qh_status st = coef_prepare(ctx, len0, len1, &a);
+    if (st != QH_OK) return st;
+  }
   const float* x_final = B.x;
   if (o->precision == QH_PREC_FP32 && (max_steps % 2 == 1)) x_final = B.x1;
   TcPlan tplan = plan;
@@ -868,9 +874,10 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
   }
   if (G.csr_mode) tplan.variant = csr_v;
   sol.kernel = G.csr_mode ? csr_variant_name(tplan.variant, is_tc_precision(o->precision))
-              : fp8 ? (R % 128 == 0 ? "e4m3-bn128-s2-x3" : "e4m3-bn64-s2-x4")
+              : fp8 ? (f8_bn(G, R, ctx->n_sm) == 128 ? "e4m3-bn128-s2-x3" : "e4m3-bn64-s2-x4")
               : is_tc_precision(o->precision) ? tc_variant_name(tplan.variant) : "k_step_f32";
-  skey += "|v" + std::to_string(tplan.variant);
+  skey += "|v" + std::to_string(tplan.variant) + "|c" + std::to_string((uintptr_t)a.coef) + "|" +
+          std::to_string(a.coef_len);
   // the multi-step kernel runs whole step ranges: a few direct launches, no capture
   const bool multistep = is_tc_precision(o->precision) && !G.csr_mode && run_variant(tplan.variant);
   RunBufs rb;
@@ -930,6 +937,7 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
     az.z_out = B.cut_z;
     az.t = 0;
     az.t_base = nullptr;
+    az.after_step = 0;
     az.active = act;
     az.use_lo = W.has_lo ? 1 : 0;
     qh_status st = launch_step_tc(ctx, W, az, B.cut_s, pick_plan(R));
@@ -941,10 +949,10 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
   auto one_step = [&](int32_t t, const int32_t* base, bool after_step) -> qh_status {
     a.t = t;
     a.t_base = base;
+    a.after_step = after_step ? 1 : 0;
     const bool even = (t % 2) == 0;
     return run_step(ctx, W, o->precision, tplan, a, even ? B.x : B.x1, even ? B.x1 : B.x,
-                    even ? B.xh0 : B.xh1, even ? B.xh1 : B.xh0, &f8, (int64_t)NS, B.zband, f32,
-                    after_step);
+                    even ? B.xh0 : B.xh1, even ? B.xh1 : B.xh0, &f8, (int64_t)NS, B.zband, f32);
   };
   if (!multistep && loop_steps > 0 && (ctx->loop_key != skey || !ctx->loop_exec)) {
     if (ctx->loop_exec) {
@@ -1586,6 +1594,8 @@ qh_status qh_debug_run_trace(qh_ctx* h, const qh_graph* gh, int32_t R, int32_t s
   a.dt = 1.f;
   a.a0 = 1.0;
   a.dta0 = 1.f;
+  st = coef_prepare(ctx, steps, 0, &a);
+  if (st) return st;
   a.sb = QH_SB_BALLISTIC;
   a.kslice = g.kslice;
   QH_CUDA_TRY(cudaMemsetAsync(xh1, 0, NS * 2, s));
@@ -1673,7 +1683,7 @@ qh_status qh_debug_matvec(qh_ctx* h, const qh_graph* gh, int32_t precision, int3
     a.xout = nullptr;
     F32Chunks ch;
     st = f32_prepare(ctx, g, g.tile_f32, QH_SB_BALLISTIC, &ch);
-    if (st == QH_OK) st = launch_step_f32(ctx, g, a, ch, false);
+    if (st == QH_OK) st = launch_step_f32(ctx, g, a, ch);
     if (st) return st;
   } else {
     __nv_bfloat16* xh = (__nv_bfloat16*)ctx->scratch((size_t)R * g.n_pad * 2, S_XH0);
@@ -1736,6 +1746,8 @@ qh_status qh_debug_steps_v(qh_ctx* h, const qh_graph* gh, int32_t precision, int
   a.dt = (float)dt;
   a.a0 = a0;
   a.dta0 = (float)(dt * a0);
+  st = coef_prepare(ctx, steps, 0, &a);
+  if (st) return st;
   const size_t NS = (size_t)R * g.n_pad;
   cudaStream_t s = ctx->stream;
   float* xu = x;  // user buffers in [R][n_pad]
@@ -1762,10 +1774,11 @@ qh_status qh_debug_steps_v(qh_ctx* h, const qh_graph* gh, int32_t precision, int
       a.t = t0 + k;
       a.xin = (k % 2 == 0) ? x : x1;
       a.xout = (k % 2 == 0) ? x1 : x;
+      a.after_step = k > 0 ? 1 : 0;
       if (g.csr_mode)
         launch_step_csr(s, g, a, g.pval, nullptr, csr_v);
       else
-        st = launch_step_f32(ctx, g, a, ch, k > 0);
+        st = launch_step_f32(ctx, g, a, ch);
       if (st) return st;
     }
     if (nsteps % 2 == 1) QH_CUDA_TRY(cudaMemcpyAsync(x, x1, NS * 4, cudaMemcpyDeviceToDevice, s));
@@ -1791,6 +1804,7 @@ qh_status qh_debug_steps_v(qh_ctx* h, const qh_graph* gh, int32_t precision, int
         f8.xl_in = cur + NS;
         a.x8h_out = nxt;
         a.x8l_out = nxt + NS;
+        a.after_step = k > 0 ? 1 : 0;
         st = launch_step_f8(ctx, g, a, f8);
         if (st) return st;
       }
@@ -1818,6 +1832,7 @@ qh_status qh_debug_steps_v(qh_ctx* h, const qh_graph* gh, int32_t precision, int
     for (int32_t k = 0; k < nsteps; ++k) {
       a.t = t0 + k;
       a.xh_out = (k % 2 == 0) ? xh1 : xh0;
+      a.after_step = k > 0 ? 1 : 0;
       if (g.csr_mode) {
         const __nv_bfloat16* xc = (k % 2 == 0) ? xh0 : xh1;
         if (csr_v == CSR_BAND8) {

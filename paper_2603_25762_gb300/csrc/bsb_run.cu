@@ -80,6 +80,8 @@ struct ItemInfo {
   float dtc0, inv_dtc0;                 // dt * c0 and its reciprocal
   float dth;                            // dt * deformation field strength (0: none)
   double inv_steps;                     // 1 / steps_b
+  const float* ctab;                    // schedule table of this length: steps_b
+                                        // coefficients, then steps_b ramp values; or nullptr
 };
 
 template <bool JRES, int SB>
@@ -131,6 +133,8 @@ struct RunArgs {
   double a0;
   int32_t* err;
   const float* deform;      // [n_blocks] deformation field strength, or nullptr
+  const float* coef;        // schedule table (StepArgs::coef)
+  int32_t coef_len;
   // early-stop checks inside the launch (check_every = 0: none)
   int32_t check_every, patience;
   __nv_bfloat16* s0;        // [R][n_pad] S_t = sgn(x_t) for even t / check_every
@@ -531,6 +535,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
     it.dtc0 = a.dt * a.c0[rt.block];
     it.inv_dtc0 = 1.0f / it.dtc0;
     it.inv_steps = 1.0 / (double)it.steps_b;
+    it.ctab = a.coef ? a.coef + coef_offset(a.coef_len, it.steps_b) + it.steps_b : nullptr;
     it.dth = a.deform ? a.dt * a.deform[rt.block] : 0.f;
     info[lane] = it;
   }
@@ -864,13 +869,22 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
         dst[4 * m + 3] = q.w;
       }
     };
-    bool fresh = true;  // xb holds nothing for the cursor's item yet
+    // {-(a0 - a(t)), 1 - t / steps_b} of an item's step, from the schedule table: FP64 in the
+    // epilogue warps held up the item after it (hifi-region 8.80 us per step against 8.47)
+    auto load_sched = [&](const ItemInfo& it, int t) -> float2 {
+      if (it.ctab == nullptr)
+        return make_float2(run_coef(a.a0, t, it.inv_steps), run_ramp(t, it.inv_steps));
+      return make_float2(it.ctab[t], it.dth != 0.f ? it.ctab[it.steps_b + t] : 0.f);
+    };
+    float2 sched = make_float2(0.f, 0.f);
+    bool fresh = true;  // xb and sched hold nothing for the cursor's item yet
     while (cur.u < n_steps) {
       if (fresh) {
         const bool gx = !xt(cur.i);
         load_x(xb[0], nit, gx, 0);
         load_x(xb[1], nit, gx, 1);
         load_x(xb[2], nit, gx, 2);
+        sched = load_sched(nit, a.t0 + cur.u);
         fresh = false;
       }
       if (decision_step<CHECK>(a, a.t0 + cur.u, nit.steps_b)) {
@@ -898,16 +912,11 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
       nit = info[non ? nxt.i : cur.i];
       const bool vr = r < it.valid, last = t == it.last_t;
       __nv_bfloat16* __restrict__ xh_out = (t & 1) ? a.xh0 : a.xh1;  // X_hat_{t+1}
-      // -(a0 - a(t)) in FP64 as in the other step kernels (a(t) = a0 t / steps_b, with
-      // the reciprocal taken once per item), by one lane, shared with the warp
-      // and the deformation force dt h (1 - t / steps_b) (0 without deformation)
-      float coef = 0.f, dtfe = 0.f;
-      if (lane == 0) {
-        coef = (float)(-(a.a0 - a.a0 * (double)t * it.inv_steps));
-        dtfe = it.dth * (float)(1.0 - (double)t * it.inv_steps);
-      }
-      const float dtcx = a.dt * __shfl_sync(0xffffffffu, coef, 0);
-      const float dtfe_s = __shfl_sync(0xffffffffu, dtfe, 0);
+      // -(a0 - a(t)) (a(t) = a0 t / steps_b, with the reciprocal taken once per item) and
+      // the deformation force dt h (1 - t / steps_b) (0 without deformation); the next
+      // item's values load while this one is updated
+      const float dtcx = a.dt * sched.x, dtfe_s = it.dth * sched.y;
+      if (non) sched = load_sched(nit, a.t0 + nxt.u);
       const float dtc0 = it.dtc0, inv = it.inv_dtc0, dta0 = a.dta0;
       const bool ok = __all_sync(0xffffffffu, rwait(accf0 + 8 * cur.i, (uint32_t)cur.u & 1u,
                                                     a.err, abort_flag));
@@ -1341,6 +1350,8 @@ qh_status launch_run_impl(Ctx* ctx, const Graph& g, const StepArgs& s, const Run
   a.a0 = s.a0;
   a.err = s.err;
   a.deform = s.deform;
+  a.coef = s.coef;
+  a.coef_len = s.coef_len;
   a.trace = trace;
   a.trace_u0 = trace_u0;
   a.trace_nu = trace_nu;

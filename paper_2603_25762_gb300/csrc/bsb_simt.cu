@@ -130,15 +130,6 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
-// Programmatic dependent launch: wait until the kernel before this one in the stream has
-// completed (its writes are visible), and let the next one start its prologue.
-__device__ __forceinline__ void grid_dep_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-__device__ __forceinline__ void grid_dep_launch() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // One FP32 step of a 32-row group for 8 RPT NW replicas.  A warp covers the 32 rows x
 // 8 RPT replicas, a thread 8 rows x RPT replicas: per 4 columns it reads 8 + RPT 16-byte
 // operands from shared memory for 32 RPT FMAs.  J and x chunks come through a three-stage
@@ -172,8 +163,7 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
   if (vrows <= 0) return;
   const int32_t sb = a.steps_b[rt.block], t = step_of(a);
   if (tid == 0) {
-    const double at = a.a0 * (double)t / (double)sb;
-    coef_s = (float)(-(a.a0 - at));
+    coef_s = step_coef(a, min(t, sb - 1), sb);  // (a step past the schedule is not live)
   }
   const int32_t nc = count[blockIdx.x];
   const int32_t ns = (nc + F_STAGE_CHUNKS - 1) / F_STAGE_CHUNKS;
@@ -336,21 +326,12 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
 
 template <int RPT, int NW, bool DISC>
 cudaError_t launch_f32_impl(cudaStream_t s, const Graph& g, const StepArgs& a,
-                            const F32Chunks& ch, int vec4, bool after_step) {
+                            const F32Chunks& ch, int vec4) {
   constexpr int RC = 8 * RPT * NW;
   constexpr size_t SMEM = sizeof(float) * F_STAGES * F_KC * (F_ROWS + RC);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)g.n_row_tiles * F_GROUPS, (unsigned)((a.R + RC - 1) / RC));
-  cfg.blockDim = dim3(32 * NW);
-  cfg.dynamicSmemBytes = SMEM;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = after_step ? 1 : 0;
-  note_launch(1);
-  return cudaLaunchKernelEx(&cfg, k_step_f32<RPT, NW, DISC>, a, ch.list, ch.count, vec4);
+  StepLaunch l(dim3((unsigned)g.n_row_tiles * F_GROUPS, (unsigned)((a.R + RC - 1) / RC)), 32 * NW,
+               SMEM, s, a.after_step != 0);
+  return cudaLaunchKernelEx(&l.cfg, k_step_f32<RPT, NW, DISC>, a, ch.list, ch.count, vec4);
 }
 
 template <int RPT, int NW>
@@ -432,8 +413,7 @@ __global__ void __launch_bounds__(CSR_CTA, 1024 / CSR_CTA) k_step_csr(StepArgs a
     return;
   }
   const int64_t e0 = prow[row], e1 = prow[row + 1];
-  const double at = a.a0 * (double)t / (double)sb;
-  const float coef_x = (float)(-(a.a0 - at));
+  const float coef_x = step_coef(a, t, sb);
   const float c0 = a.c0[rt.block];
   const float fe = deform_force(a.deform, rt.block, t, sb);
   for (int32_t r0 = 0; r0 < a.R; r0 += 128) {
@@ -651,8 +631,7 @@ __global__ void __launch_bounds__(CSR_CTA, 1024 / CSR_CTA) k_step_csr8(StepArgs 
       continue;
     }
     // the update's constants, taken after the gathers (fewer live registers there)
-    const double at = a.a0 * (double)t / (double)sb;
-    const float coef_x = (float)(-(a.a0 - at));
+    const float coef_x = step_coef(a, t, sb);
     const float c0 = a.c0[rt.block];
     const float fe = deform_force(a.deform, rt.block, t, sb);
     const float* xsrc = BF16 ? a.x : a.xin;
@@ -1410,8 +1389,7 @@ cudaError_t f32_set_attrs() {
   return e;
 }
 
-qh_status launch_step_f32(Ctx* ctx, const Graph& g, const StepArgs& a, const F32Chunks& ch,
-                          bool after_step) {
+qh_status launch_step_f32(Ctx* ctx, const Graph& g, const StepArgs& a, const F32Chunks& ch) {
   if (g.n_row_tiles == 0) return QH_OK;
   // 16-byte accesses of y, x_{t+1} and z (x_t is read in 16-byte pieces in any case)
   const uintptr_t bits = (uintptr_t)a.y | (uintptr_t)a.xout | (uintptr_t)a.z_out;
@@ -1432,8 +1410,8 @@ qh_status launch_step_f32(Ctx* ctx, const Graph& g, const StepArgs& a, const F32
                                                             : 4;
   cudaError_t e;
 #define QH_F32(RPT)                                                               \
-  (disc ? launch_f32_impl<RPT, 2, true>(ctx->stream, g, a, ch, vec4, after_step)  \
-        : launch_f32_impl<RPT, 2, false>(ctx->stream, g, a, ch, vec4, after_step))
+  (disc ? launch_f32_impl<RPT, 2, true>(ctx->stream, g, a, ch, vec4)  \
+        : launch_f32_impl<RPT, 2, false>(ctx->stream, g, a, ch, vec4))
   e = rpt == 1 ? QH_F32(1) : rpt == 2 ? QH_F32(2) : QH_F32(4);
 #undef QH_F32
   return e == cudaSuccess ? QH_OK : cuda_fail(ctx, e, "k_step_f32 launch");
@@ -1586,6 +1564,29 @@ void launch_trace_check(cudaStream_t s, int32_t n_blocks, const double* best_cut
   if (n_blocks > 0)
     k_trace_check<<<::qh::counted(nblk(n_blocks)), 256, 0, s>>>(n_blocks, best_cut, running,
                                                                 t_done, steps_b, row);
+}
+
+__global__ void k_coef_table(int32_t len0, int32_t len1, double a0, float* out) {
+  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= len0 + len1) return;
+  const int32_t sb = i < len0 ? len0 : len1, t = i < len0 ? i : i - len0;
+  float* p = out + (i < len0 ? 0 : 3 * (int64_t)len0);
+  const double inv_steps = 1.0 / (double)sb;
+  p[t] = (float)(-(a0 - step_at(a0, t, sb)));
+  p[sb + t] = run_coef(a0, t, inv_steps);
+  p[2 * (int64_t)sb + t] = run_ramp(t, inv_steps);
+}
+
+qh_status coef_prepare(Ctx* ctx, int32_t len0, int32_t len1, StepArgs* a) {
+  a->coef = nullptr;
+  if (len0 < 1 || len1 < 0 || len0 > COEF_MAX_STEPS || len1 > COEF_MAX_STEPS) return QH_OK;
+  float* p = (float*)ctx->scratch(sizeof(float) * 3 * ((size_t)len0 + len1), S_COEF);
+  if (!p) return set_err(ctx, QH_ENOMEM, "allocation failed (schedule table)");
+  k_coef_table<<<::qh::counted(nblk((int64_t)len0 + len1)), 256, 0, ctx->stream>>>(len0, len1,
+                                                                                a->a0, p);
+  a->coef = p;
+  a->coef_len = len0;
+  return QH_OK;
 }
 
 __global__ void k_advance(int32_t* t_base, int32_t n) { *t_base += n; }

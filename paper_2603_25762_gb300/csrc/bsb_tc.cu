@@ -22,6 +22,17 @@ namespace qh {
 
 namespace {
 
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void tmem_ld_n(uint32_t addr, uint32_t (&v)[N]) {
+  if constexpr (N == 32)
+    tmem_ld32(addr, v);
+  else
+    tmem_ld16(addr, v);
+}
+
 template <int BN, int STAGES>
 struct TcSmem {
   static constexpr uint32_t B_BYTES = BN * 64 * 2;
@@ -103,8 +114,7 @@ __global__ void __launch_bounds__(128) k_step_tc(const __grid_constant__ CUtenso
   tc_fence_after();
   const int row = warp * 32 + lane;
   const bool vrow = ok && row < rt.valid;
-  const double at = (double)a.a0 * (double)t / (double)sb;
-  const float coef_x = (float)(-((double)a.a0 - at));
+  const float coef_x = a.z_out != nullptr ? 0.f : step_coef(a, t, sb);
   const float c0 = a.c0[rt.block];
   const float fe = deform_force(a.deform, rt.block, t, a.steps_b[rt.block]);
   const size_t base = (size_t)blockIdx.y * BN * a.n_pad + rt.row0 + row;
@@ -154,7 +164,13 @@ __global__ void __launch_bounds__(128) k_step_tc(const __grid_constant__ CUtenso
 // the SM (one CTA's epilogue overlaps another's TMA / MMA phase).  The first 32
 // replica columns of the state are loaded before the accumulator is ready and the
 // next 32 are in flight while the current 32 are updated.
-template <int BN, int STAGES, int MINB>
+// A step's launch overlaps the end of the step before it (grid_dep_wait): barriers, TMEM,
+// and the first J copies come before the wait.  us per step, BF16, before -> with that,
+// a ring as deep as the grid allows and the coefficient table: 80 reads R = 64 6.8 -> 4.5;
+// 1,800 reads R = 192 8.05 -> 6.15; 7,200 reads R = 576 14.9 -> 12.5.  FP8: 720 reads
+// R = 128 14.2 -> 7.6; 7,200 reads R = 256 15.5 -> 9.8, R = 512 19.7 -> 17.0, R = 1,024
+// 31.8 -> 29.9.
+template <int BN, int STAGES, int MINB, int CH>
 __global__ void __launch_bounds__(128, MINB) k_step_tc_v(const __grid_constant__ CUtensorMap tmJ,
                                                          const __grid_constant__ CUtensorMap tmX,
                                                          StepArgs a) {
@@ -169,22 +185,17 @@ __global__ void __launch_bounds__(128, MINB) k_step_tc_v(const __grid_constant__
 
   const RowTile rt = a.rt[blockIdx.x];
   const int32_t sb = a.steps_b[rt.block], t = step_of(a);
-  if ((a.active != nullptr && !a.active[rt.block]) || t >= sb) return;  // CTA-uniform
+  if ((a.active != nullptr && !a.active[rt.block]) || t >= sb) {  // CTA-uniform
+    grid_dep_wait();
+    return;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nk = row_slices(a.kslice, rt, a.use_lo);
   const int row = warp * 32 + lane;
   const bool vrow = row < rt.valid;
   const size_t base = (size_t)blockIdx.y * BN * a.n_pad + rt.row0 + row;
-  constexpr int CH = 16;  // replica columns per epilogue chunk
+  static_assert(CH == 16 || CH == 32, "replica columns per epilogue chunk");
   float xs[CH], ys[CH];
-  if (vrow) {  // chunk 0 of the state: independent of the product, start it now
-#pragma unroll
-    for (int j = 0; j < CH; ++j) {
-      xs[j] = a.x[base + (size_t)j * a.n_pad];
-      ys[j] = a.y[base + (size_t)j * a.n_pad];
-    }
-  }
-
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(full0 + 8 * s, 1);
@@ -195,20 +206,41 @@ __global__ void __launch_bounds__(128, MINB) k_step_tc_v(const __grid_constant__
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), (uint32_t)BN);
+  // J does not depend on the step before: its first stages load ahead of the wait
+  if (threadIdx.x == 0) {
+    prefetch_map(&tmX);
+    for (int kb = 0; kb < min(nk, STAGES); ++kb) {
+      mbar_expect_tx(full0 + 8 * kb, L::STAGE);
+      const KSlice ks = slice_at(a.kslice, a.tile_col, rt.ks_begin, rt.tile_begin, kb);
+      tma_load_2d(smem_u32(smem + kb * L::STAGE), &tmJ, full0 + 8 * kb, ks.half() * 64, ks.jrow());
+    }
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_dep_wait();
+  grid_dep_launch();
+  if (vrow) {  // chunk 0 of the state: independent of the product, start it now
+#pragma unroll
+    for (int j = 0; j < CH; ++j) {
+      xs[j] = a.x[base + (size_t)j * a.n_pad];
+      ys[j] = a.y[base + (size_t)j * a.n_pad];
+    }
+  }
 
   if (warp == 0 && lane == 0 && nk > 0) {
     for (int kb = 0; kb < nk; ++kb) {
       const int s = kb % STAGES;
       const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
-      if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, a.err)) break;
       uint8_t* sa = smem + s * L::STAGE;
-      mbar_expect_tx(full0 + 8 * s, L::STAGE);
+      if (kb >= STAGES) {
+        if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, a.err)) break;
+        mbar_expect_tx(full0 + 8 * s, L::STAGE);
+      }
       const KSlice ks = slice_at(a.kslice, a.tile_col, rt.ks_begin, rt.tile_begin, kb);
-      tma_load_2d(smem_u32(sa), &tmJ, full0 + 8 * s, ks.half() * 64, ks.jrow());
+      if (kb >= STAGES)
+        tma_load_2d(smem_u32(sa), &tmJ, full0 + 8 * s, ks.half() * 64, ks.jrow());
       tma_load_2d(smem_u32(sa + A_BYTES), &tmX, full0 + 8 * s, ks.ct() * TILE + ks.half() * 64,
                   (int32_t)blockIdx.y * BN);
     }
@@ -234,8 +266,7 @@ __global__ void __launch_bounds__(128, MINB) k_step_tc_v(const __grid_constant__
 
   const bool ok = nk > 0 ? mbar_wait(accb, 0, a.err) : true;
   tc_fence_after();
-  const double at = a.a0 * (double)t / (double)sb;
-  const float coef_x = (float)(-(a.a0 - at));
+  const float coef_x = step_coef(a, t, sb);
   const float c0 = a.c0[rt.block];
   const float fe = deform_force(a.deform, rt.block, t, a.steps_b[rt.block]);
 #pragma unroll
@@ -243,7 +274,7 @@ __global__ void __launch_bounds__(128, MINB) k_step_tc_v(const __grid_constant__
     uint32_t v[CH];
     __syncwarp();
     if (nk > 0) {
-      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * CH), v);
+      tmem_ld_n<CH>(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * CH), v);
     } else {
 #pragma unroll
       for (int j = 0; j < CH; ++j) v[j] = 0u;
@@ -315,7 +346,7 @@ __device__ __forceinline__ void split_e4m3(float x, uint8_t& h, uint8_t& l) {
   l = lo.__x;
 }
 
-template <int BN, int STAGES, int MINB>
+template <int BN, int STAGES, int MINB, int CH>
 __global__ void __launch_bounds__(128, MINB)
     k_step_tc_f8(const __grid_constant__ CUtensorMap tmJh, const __grid_constant__ CUtensorMap tmJl,
                  const __grid_constant__ CUtensorMap tmXh, const __grid_constant__ CUtensorMap tmXl,
@@ -331,21 +362,16 @@ __global__ void __launch_bounds__(128, MINB)
 
   const RowTile rt = a.rt[blockIdx.x];
   const int32_t sb = a.steps_b[rt.block], t = step_of(a);
-  if ((a.active != nullptr && !a.active[rt.block]) || t >= sb) return;  // CTA-uniform
+  if ((a.active != nullptr && !a.active[rt.block]) || t >= sb) {  // CTA-uniform
+    grid_dep_wait();
+    return;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nk = rt.n_hi * n_slices;
   const int row = warp * 32 + lane;
   const bool vrow = row < rt.valid;
   const size_t base = (size_t)blockIdx.y * BN * a.n_pad + rt.row0 + row;
-  constexpr int CH = 16;
   float xs[CH], ys[CH];
-  if (vrow && a.z_out == nullptr) {
-#pragma unroll
-    for (int j = 0; j < CH; ++j) {
-      xs[j] = a.x[base + (size_t)j * a.n_pad];
-      ys[j] = a.y[base + (size_t)j * a.n_pad];
-    }
-  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(full0 + 8 * s, 1);
@@ -356,22 +382,45 @@ __global__ void __launch_bounds__(128, MINB)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), (uint32_t)BN);
+  // J does not depend on the step before: its first stages load ahead of the wait
+  if (threadIdx.x == 0) {
+    prefetch_map(&tmXh);
+    prefetch_map(&tmXl);
+    for (int kb = 0; kb < min(nk, STAGES); ++kb) {
+      mbar_expect_tx(full0 + 8 * kb, L::STAGE);
+      const int e = kb / n_slices, sl = kb % n_slices;
+      tma_load_2d(smem_u32(smem + kb * L::STAGE), sl == 2 ? &tmJl : &tmJh, full0 + 8 * kb, 0,
+                  (rt.f32_begin + e) * TILE);
+    }
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_dep_wait();
+  grid_dep_launch();
+  if (vrow && a.z_out == nullptr) {  // chunk 0 of the state: independent of the product, start it now
+#pragma unroll
+    for (int j = 0; j < CH; ++j) {
+      xs[j] = a.x[base + (size_t)j * a.n_pad];
+      ys[j] = a.y[base + (size_t)j * a.n_pad];
+    }
+  }
 
   if (warp == 0 && lane == 0 && nk > 0) {
     for (int kb = 0; kb < nk; ++kb) {
       const int s = kb % STAGES;
       const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
-      if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, a.err)) break;
       uint8_t* sa = smem + s * L::STAGE;
-      mbar_expect_tx(full0 + 8 * s, L::STAGE);
+      if (kb >= STAGES) {
+        if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, a.err)) break;
+        mbar_expect_tx(full0 + 8 * s, L::STAGE);
+      }
       const int e = kb / n_slices, sl = kb % n_slices;  // slice: 0 (Jh,Xh) 1 (Jh,Xl) 2 (Jl,Xh)
       const CUtensorMap* mj = sl == 2 ? &tmJl : &tmJh;
       const CUtensorMap* mx = sl == 1 ? &tmXl : &tmXh;
-      tma_load_2d(smem_u32(sa), mj, full0 + 8 * s, 0, (rt.f32_begin + e) * TILE);
+      if (kb >= STAGES)
+        tma_load_2d(smem_u32(sa), mj, full0 + 8 * s, 0, (rt.f32_begin + e) * TILE);
       tma_load_2d(smem_u32(sa + A_BYTES), mx, full0 + 8 * s,
                   a.tile_col[rt.tile_begin + e] * TILE, (int32_t)blockIdx.y * BN);
     }
@@ -397,8 +446,7 @@ __global__ void __launch_bounds__(128, MINB)
 
   const bool ok = nk > 0 ? mbar_wait(accb, 0, a.err) : true;
   tc_fence_after();
-  const double at = a.a0 * (double)t / (double)sb;
-  const float coef_x = (float)(-(a.a0 - at));
+  const float coef_x = a.z_out != nullptr ? 0.f : step_coef(a, t, sb);
   const float c0 = a.c0[rt.block];
   const float fe = deform_force(a.deform, rt.block, t, a.steps_b[rt.block]);
   const float inv_s = a.inv_scale;
@@ -407,7 +455,7 @@ __global__ void __launch_bounds__(128, MINB)
     uint32_t v[CH];
     __syncwarp();
     if (nk > 0) {
-      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * CH), v);
+      tmem_ld_n<CH>(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * CH), v);
     } else {
 #pragma unroll
       for (int j = 0; j < CH; ++j) v[j] = 0u;
@@ -563,6 +611,8 @@ __global__ void __launch_bounds__(192, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_dep_wait();
+  grid_dep_launch();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -638,8 +688,7 @@ __global__ void __launch_bounds__(192, 1)
       tc_fence_after();
       float* sx = reinterpret_cast<float*>(smem + L::STATE_OFF + b * 2 * L::STILE);
       float* sy = sx + BN * TILE;
-      const double at = a.a0 * (double)t / (double)a.steps_b[rt.block];
-      const float coef_x = (float)(-(a.a0 - at));
+      const float coef_x = step_coef(a, t, a.steps_b[rt.block]);
       const float c0 = a.c0[rt.block];
       const float fe = deform_force(a.deform, rt.block, t, a.steps_b[rt.block]);
       const bool vrow = ok && row < rt.valid;
@@ -752,6 +801,8 @@ __global__ void __launch_bounds__(384, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_dep_wait();
+  grid_dep_launch();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -840,8 +891,7 @@ __global__ void __launch_bounds__(384, 1)
       }
       const bool ok = mbar_wait(afull0 + 8 * ab, aph, a.err);
       tc_fence_after();
-      const double at = a.a0 * (double)t / (double)a.steps_b[rt.block];
-      const float coef_x = (float)(-(a.a0 - at));
+      const float coef_x = step_coef(a, t, a.steps_b[rt.block]);
       const float c0 = a.c0[rt.block];
       const float fe = deform_force(a.deform, rt.block, t, a.steps_b[rt.block]);
 #pragma unroll
@@ -930,34 +980,34 @@ bool make_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_t outer
 
 namespace {
 
-template <int BN, int STAGES, int MINB>
+template <int BN, int STAGES, int MINB, int CH = 16>
 qh_status launch_variant(Ctx* ctx, const Graph& g, const StepArgs& a, const __nv_bfloat16* xh_in) {
   CUtensorMap mJ, mX;
   if (!make_map(&mJ, g.tile_bf16, TILE, (uint64_t)g.n_tiles * TILE, TILE) ||
       !make_map(&mX, xh_in, (uint64_t)g.n_pad, (uint64_t)a.R, BN))
     return set_err(ctx, QH_ECUDA, "cuTensorMapEncodeTiled failed");
-  dim3 grid(g.n_row_tiles, a.R / BN);
-  k_step_tc_v<BN, STAGES, MINB><<<::qh::counted(grid), 128, TcSmem<BN, STAGES>::BYTES, ctx->stream>>>(mJ, mX, a);
-  cudaError_t e = cudaGetLastError();
+  StepLaunch l(dim3(g.n_row_tiles, a.R / BN), 128, TcSmem<BN, STAGES>::BYTES, ctx->stream,
+               a.after_step != 0);
+  cudaError_t e = cudaLaunchKernelEx(&l.cfg, k_step_tc_v<BN, STAGES, MINB, CH>, mJ, mX, a);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "k_step_tc_v launch");
   return QH_OK;
 }
 
-template <int BN, int STAGES, int MINB>
+template <int BN, int STAGES, int MINB, int CH = 16>
 cudaError_t set_attr_v() {
-  return cudaFuncSetAttribute(k_step_tc_v<BN, STAGES, MINB>,
+  return cudaFuncSetAttribute(k_step_tc_v<BN, STAGES, MINB, CH>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)TcSmem<BN, STAGES>::BYTES);
 }
 
-template <int BN, int STAGES, int MINB>
+template <int BN, int STAGES, int MINB, int CH = 16>
 cudaError_t set_attr_f8() {
-  return cudaFuncSetAttribute(k_step_tc_f8<BN, STAGES, MINB>,
+  return cudaFuncSetAttribute(k_step_tc_f8<BN, STAGES, MINB, CH>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)TcSmem<BN, STAGES>::BYTES);
 }
 
-template <int BN, int STAGES, int MINB>
+template <int BN, int STAGES, int MINB, int CH = 16>
 qh_status launch_f8_impl(Ctx* ctx, const Graph& g, const StepArgs& a, const Fp8Operands& op) {
   CUtensorMap mJh, mJl, mXh, mXl;
   const uint64_t jrows = (uint64_t)std::max<int64_t>(g.n_tiles_hi, 1) * TILE;
@@ -966,10 +1016,10 @@ qh_status launch_f8_impl(Ctx* ctx, const Graph& g, const StepArgs& a, const Fp8O
       !make_map(&mXh, op.xh_in, (uint64_t)g.n_pad, (uint64_t)a.R, BN, false, true) ||
       !make_map(&mXl, op.xl_in, (uint64_t)g.n_pad, (uint64_t)a.R, BN, false, true))
     return set_err(ctx, QH_ECUDA, "cuTensorMapEncodeTiled failed (e4m3)");
-  dim3 grid(g.n_row_tiles, a.R / BN);
-  k_step_tc_f8<BN, STAGES, MINB><<<::qh::counted(grid), 128, TcSmem<BN, STAGES>::BYTES,
-                                   ctx->stream>>>(mJh, mJl, mXh, mXl, a, op.n_slices);
-  cudaError_t e = cudaGetLastError();
+  StepLaunch l(dim3(g.n_row_tiles, a.R / BN), 128, TcSmem<BN, STAGES>::BYTES, ctx->stream,
+               a.after_step != 0);
+  cudaError_t e = cudaLaunchKernelEx(&l.cfg, k_step_tc_f8<BN, STAGES, MINB, CH>, mJh, mJl, mXh, mXl, a,
+                                     op.n_slices);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "k_step_tc_f8 launch");
   return QH_OK;
 }
@@ -985,8 +1035,9 @@ qh_status launch_persistent2(Ctx* ctx, const Graph& g, const StepArgs& a,
   const int32_t n_rep = a.R / P2_BN;
   const int32_t n_items = g.n_row_tiles * n_rep;
   const int grid = std::min(n_items, ctx->n_sm);
-  k_step_tc_p2<<<::qh::counted(grid), 384, P2Smem::BYTES, ctx->stream>>>(mJ, mX, mSx, mSy, a, n_items, n_rep);
-  cudaError_t e = cudaGetLastError();
+  StepLaunch l(dim3(grid), 384, P2Smem::BYTES, ctx->stream, a.after_step != 0);
+  cudaError_t e =
+      cudaLaunchKernelEx(&l.cfg, k_step_tc_p2, mJ, mX, mSx, mSy, a, n_items, n_rep);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "k_step_tc_p2 launch");
   return QH_OK;
 }
@@ -1004,9 +1055,9 @@ qh_status launch_persistent(Ctx* ctx, const Graph& g, const StepArgs& a,
   const int32_t n_rep = a.R / BN;
   const int32_t n_items = g.n_row_tiles * n_rep;
   const int grid = std::min(n_items, ctx->n_sm);
-  k_step_tc_p<BN, OSTAGES><<<::qh::counted(grid), 192, L::BYTES, ctx->stream>>>(mJ, mX, mSx, mSy, a, n_items,
-                                                                  n_rep);
-  cudaError_t e = cudaGetLastError();
+  StepLaunch l(dim3(grid), 192, L::BYTES, ctx->stream, a.after_step != 0);
+  cudaError_t e =
+      cudaLaunchKernelEx(&l.cfg, k_step_tc_p<BN, OSTAGES>, mJ, mX, mSx, mSy, a, n_items, n_rep);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "k_step_tc_p launch");
   return QH_OK;
 }
@@ -1050,6 +1101,9 @@ qh_status tc_prepare(Ctx* ctx) {
   if (e == cudaSuccess) e = set_attr_v<128, 3, 1>();
   if (e == cudaSuccess) e = set_attr_v<128, 2, 3>();
   if (e == cudaSuccess) e = set_attr_v<64, 2, 4>();
+  if (e == cudaSuccess) e = set_attr_v<64, 6, 1, 32>();
+  if (e == cudaSuccess) e = set_attr_f8<64, 4, 2>();
+  if (e == cudaSuccess) e = set_attr_f8<64, 6, 1, 32>();
   if (e == cudaSuccess) e = set_attr_v<256, 2, 2>();
   if (e == cudaSuccess) e = set_attr_f8<128, 2, 3>();
   if (e == cudaSuccess) e = set_attr_f8<64, 2, 4>();
@@ -1064,10 +1118,32 @@ qh_status tc_prepare(Ctx* ctx) {
   return QH_OK;
 }
 
+// Operand ring of the 64-replica CTAs: two slots with four CTAs per SM; a grid that leaves
+// SMs to fewer CTAs takes as many slots as fit beside them, so that a row tile's slices are
+// in flight together (each refill of a slot waits a copy's latency).  Measured, two slots
+// -> this, us per step: BF16 144 reads R = 64 6.30 -> 5.90, 1,800 reads R = 192 7.09 -> 6.82
+// (four slots at 171 CTAs 8.07 -> 8.24: BF16 keeps two there); FP8 1,800 reads R = 512
+// 9.83 -> 9.00, 7,200 reads R = 256 11.58 -> 10.64.
+static int ring_depth(const Graph& g, int R, int n_sm) {
+  const int64_t ctas = (int64_t)g.n_row_tiles * (R / 64);
+  return ctas <= n_sm ? 6 : ctas <= 2 * n_sm ? 4 : 2;
+}
+
+// Replicas per CTA of the FP8 step: 128 when such CTAs fill the SMs one and a half times,
+// else 64 (more CTAs, half the epilogue each).  128 / 64, us per step: 57 row tiles,
+// R = 256 (114 CTAs) 14.7 / 11.6, R = 512 (228) 18.07 / 18.07, R = 1,024 (456) 31.2 / 37.5.
+int f8_bn(const Graph& g, int R, int n_sm) {
+  return R % 128 == 0 && 2 * (int64_t)g.n_row_tiles * (R / 128) >= 3 * (int64_t)n_sm ? 128 : 64;
+}
+
 qh_status launch_step_f8(Ctx* ctx, const Graph& g, const StepArgs& a, const Fp8Operands& op) {
   if (g.n_row_tiles == 0) return QH_OK;
-  if (a.R % 128 == 0) return launch_f8_impl<128, 2, 3>(ctx, g, a, op);
-  return launch_f8_impl<64, 2, 4>(ctx, g, a, op);
+  if (f8_bn(g, a.R, ctx->n_sm) == 128) return launch_f8_impl<128, 2, 3>(ctx, g, a, op);
+  switch (ring_depth(g, a.R, ctx->n_sm)) {
+    case 6: return launch_f8_impl<64, 6, 1, 32>(ctx, g, a, op);
+    case 4: return launch_f8_impl<64, 4, 2>(ctx, g, a, op);
+    default: return launch_f8_impl<64, 2, 4>(ctx, g, a, op);
+  }
 }
 
 void launch_tiles_to_e4m3(cudaStream_t s, const float* tf, int64_t n, float scale, uint8_t* th,
@@ -1123,7 +1199,9 @@ qh_status launch_step_tc(Ctx* ctx, const Graph& g, const StepArgs& a, const __nv
     switch (plan.variant) {
       case 0: return launch_variant<128, 3, 1>(ctx, g, a, xh_in);
       case 1: return launch_variant<128, 2, 3>(ctx, g, a, xh_in);
-      case 2: return launch_variant<64, 2, 4>(ctx, g, a, xh_in);
+      case 2:
+        return ring_depth(g, a.R, ctx->n_sm) == 6 ? launch_variant<64, 6, 1, 32>(ctx, g, a, xh_in)
+                                                  : launch_variant<64, 2, 4>(ctx, g, a, xh_in);
       case 3: return launch_variant<256, 2, 2>(ctx, g, a, xh_in);
       case 4: return launch_persistent2(ctx, g, a, xh_in);
       case 5: return launch_persistent<64, 3>(ctx, g, a, xh_in);

@@ -205,6 +205,34 @@ struct Ctx {
   void* scratch(size_t bytes, int slot);
 };
 
+// Programmatic dependent launch.  A step launched after another one (StepArgs::after_step)
+// starts while that one finishes; grid_dep_wait returns once it has completed and its
+// writes are visible.  What precedes the wait may read only what no step writes.  Every
+// CTA waits before it exits, or a step with nothing left to do would complete ahead of the
+// one before it.
+__device__ __forceinline__ void grid_dep_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dep_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// Launch configuration of a step kernel, with that attribute after another step.
+struct StepLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  StepLaunch(dim3 grid, unsigned threads, size_t smem, cudaStream_t s, bool after_step) {
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = after_step ? 1 : 0;
+    note_launch(1);
+  }
+};
+
 // Device-side view handed to the step kernels.
 struct StepArgs {
   const RowTile* rt;
@@ -222,6 +250,10 @@ struct StepArgs {
   const int32_t* steps_b;  // [n_blocks] schedule length per block (a(t) = a0 t / steps_b)
   int32_t n_pad, R;
   int32_t t;              // step index, relative to *t_base
+  int32_t after_step;     // host: the launch before this one in the stream is another step,
+                          // whose end this one's prologue may overlap
+  const float* coef;      // schedule table (coef_prepare), or nullptr: computed per step
+  int32_t coef_len;       // its first schedule length
   const int32_t* t_base;  // device word a replayed chunk of steps counts from, or nullptr (0)
   int32_t use_lo;         // BF16 paths: also accumulate the lo (remainder) tiles
   uint8_t* x8h_out;       // FP8 path: e4m3 hi / lo parts of X_{t+1}
@@ -237,6 +269,30 @@ struct StepArgs {
                           // nullptr: y gains dt h_b (1 - t / steps_b) (uniform field
                           // along the incumbent, all +1 in the refinement's gauged frame)
 };
+
+// The schedule's step coefficients, once per solve.  -(a0 - a(t)) is FP64 arithmetic with a
+// division; this part's FP64 rate is about 1/64 of its FP32 rate, and every thread (or
+// epilogue warp) of every step took it.  Per distinct schedule length L (at most two):
+// L values (float)(-(a0 - a0 t / L)) for the per-step kernels, L of the multi-step kernel's
+// (float)(-(a0 - a0 t (1 / L))), L of its deformation ramp (float)(1 - t (1 / L)).
+constexpr int32_t COEF_MAX_STEPS = 1 << 20;  // longer schedules: computed per step
+constexpr int S_COEF = 107;                  // scratch slot
+__host__ __device__ inline int64_t coef_offset(int32_t coef_len, int32_t sb) {
+  return sb == coef_len ? 0 : 3 * (int64_t)coef_len;
+}
+__device__ __forceinline__ double step_at(double a0, int32_t t, int32_t sb) {
+  return a0 * (double)t / (double)sb;
+}
+__device__ __forceinline__ float step_coef(const StepArgs& a, int32_t t, int32_t sb) {
+  if (a.coef != nullptr) return a.coef[coef_offset(a.coef_len, sb) + t];
+  return (float)(-(a.a0 - step_at(a.a0, t, sb)));
+}
+__device__ __forceinline__ float run_coef(double a0, int32_t t, double inv_steps) {
+  return (float)(-(a0 - a0 * (double)t * inv_steps));
+}
+__device__ __forceinline__ float run_ramp(int32_t t, double inv_steps) {
+  return (float)(1.0 - (double)t * inv_steps);
+}
 
 __device__ __forceinline__ int32_t step_of(const StepArgs& a) {
   return a.t + (a.t_base != nullptr ? *a.t_base : 0);
@@ -318,10 +374,7 @@ struct F32Chunks {
 };
 constexpr int S_F32_LIST = 105, S_F32_COUNT = 106;  // scratch slots
 qh_status f32_prepare(Ctx* ctx, const Graph& g, const float* tile_f32, int32_t sb, F32Chunks* ch);
-// after_step: the launch before this one in the stream is another FP32 step (its prologue
-// may then overlap that step's end).
-qh_status launch_step_f32(Ctx* ctx, const Graph& g, const StepArgs& a, const F32Chunks& ch,
-                          bool after_step);
+qh_status launch_step_f32(Ctx* ctx, const Graph& g, const StepArgs& a, const F32Chunks& ch);
 cudaError_t f32_set_attrs();
 // CSR storage: warp per padded vertex, state [n_pad][R]; xh_in != nullptr selects the
 // BF16 X_hat operand, otherwise a.xin (FP32).  variant: CSR_LANE4 (4 replicas per lane,
@@ -377,6 +430,8 @@ void launch_cut_from_product(cudaStream_t s, const Graph& g, int32_t R, const fl
 void launch_trace_check(cudaStream_t s, int32_t n_blocks, const double* best_cut,
                         const int32_t* running, int32_t t_done, const int32_t* steps_b,
                         double* row);
+// Fill a.coef / a.coef_len for schedules of len0 and len1 steps (len1 = 0: one length).
+qh_status coef_prepare(Ctx* ctx, int32_t len0, int32_t len1, StepArgs* a);
 // *t_base += n: the last node of a replayed chunk of n steps.
 void launch_advance(cudaStream_t s, int32_t* t_base, int32_t n);
 void launch_early_stop(cudaStream_t s, int32_t n_blocks, const double* best_cut, double* best_seen,
@@ -430,6 +485,7 @@ struct Fp8Operands {
   const uint8_t* xl_in;
   int32_t n_slices;       // 2, or 3 when s*J has a nonzero remainder
 };
+int f8_bn(const Graph& g, int R, int n_sm);  // replicas per CTA of the FP8 step
 qh_status launch_step_f8(Ctx* ctx, const Graph& g, const StepArgs& a, const Fp8Operands& op);
 void launch_tiles_to_e4m3(cudaStream_t s, const float* tf, int64_t n, float scale, uint8_t* th,
                           uint8_t* tl, int32_t* has_lo);
