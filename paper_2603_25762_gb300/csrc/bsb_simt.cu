@@ -70,7 +70,10 @@ constexpr int F_STAGES = 3;
 constexpr int F_QUADS = F_KC / 4;      // 16-byte pieces of a staged row
 // Position of piece q of a staged row: row groups (J) and replicas (x) that a warp reads
 // at once fall into distinct banks.
-__device__ __forceinline__ int f32_jpos(int row, int q) { return (q ^ ((row >> 3) & 3)) * 4; }
+template <int TR>
+__device__ __forceinline__ int f32_jpos(int row, int q) {
+  return (q ^ ((row / TR) & 3)) * 4;
+}
 __device__ __forceinline__ int f32_xpos(int rep, int q) { return (q ^ (rep & 7)) * 4; }
 
 // Chunk lists: CTA per row tile.  Group g's list starts at entry f32_begin * 64 +
@@ -130,26 +133,28 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
-// One FP32 step of a 32-row group for 8 RPT NW replicas.  A warp covers the 32 rows x
-// 8 RPT replicas, a thread 8 rows x RPT replicas: per 4 columns it reads 8 + RPT 16-byte
-// operands from shared memory for 32 RPT FMAs.  J and x chunks come through a three-stage
+// One FP32 step of a 32-row group for 8 RPT NW replicas.  A warp covers 4 TR rows x 8 RPT
+// replicas, a thread TR rows x RPT replicas: per 4 columns it reads TR + RPT 16-byte
+// operands from shared memory for 4 TR RPT FMAs.  J and x chunks come through a three-stage
 // cp.async ring, both with their columns contiguous (no transpose); the XOR swizzles put
 // the 4 row groups (8 replicas) that a warp reads at once into distinct banks.  Every
 // output sums its columns in ascending order with one FMA each.  The rows' list and J do
 // not depend on the step before: they are fetched ahead of the grid dependency.
-// Bound by the latency of the operand copies at 12 warps per SM (ncu on hifi-region,
-// R = 1,024: issue slots 51 % busy, FMA pipe 34 %, DRAM under 25 %).  Stages of 2 chunks
-// (more CTAs per SM, twice the barriers) measured slower: 66 against 61 us per step there
-// with four of them, 85 against 69 on ont-like 3,000 SNPs at R = 512.  Microseconds per
-// step, the dense 128 x 64 tile product before -> now: 300 SNPs / 80 reads, R = 32:
-// 20.4 -> 2.9; 720 reads, R = 256: 49.7 -> 7.4; 7,200 reads, R = 256: 64.7 -> 17.9 and
-// R = 1,024: 192 -> 61; 12,000-SNP graph (468 neighbours), R = 128: 146 -> 63 and
-// R = 512: 349 -> 179.
-template <int RPT, int NW, bool DISC>
-__global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __restrict__ list,
+// Large graphs are bound by the latency of the operand copies at 12 warps per SM (ncu on
+// hifi-region, R = 1,024: issue slots 51 % busy, FMA pipe 34 %, DRAM under 25 %), small ones
+// by the chain launch - x copies - column loop - update.  Stages of 2 chunks (more CTAs per
+// SM, twice the barriers) measured slower: 66 against 61 us per step on hifi-region, 85
+// against 69 on ont-like 3,000 SNPs at R = 512; so did x and y prefetched into registers
+// ahead of the loop (hifi-region R = 256 21.8 against 17.9: fewer CTAs per SM).
+// Microseconds per step, the dense 128 x 64 tile product before -> now: 300 SNPs / 80
+// reads, R = 32: 20.4 -> 2.4; 720 reads, R = 256: 49.7 -> 6.6; 7,200 reads, R = 256: 64.7 ->
+// 17.9 and R = 1,024: 192 -> 61; 12,000-SNP graph (468 neighbours), R = 128: 146 -> 63 and
+// R = 512: 349 -> 178.
+template <int RPT, int NW, int TR, bool DISC>
+__global__ void __launch_bounds__(32 * NW * 8 / TR) k_step_f32(StepArgs a, const int2* __restrict__ list,
                                                       const int32_t* __restrict__ count,
                                                       int vec4) {
-  constexpr int RC = 8 * RPT * NW, NT = 32 * NW;
+  constexpr int RC = 8 * RPT * NW, NT = 32 * NW * 8 / TR;
   extern __shared__ __align__(128) float f32_smem[];
   float* const js = f32_smem;                               // [F_STAGES][32 rows][32]
   float* const xs = f32_smem + F_STAGES * F_ROWS * F_KC;    // [F_STAGES][RC][32]
@@ -157,7 +162,8 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
   const int32_t rti = blockIdx.x / F_GROUPS, grp = blockIdx.x % F_GROUPS;
   const RowTile rt = a.rt[rti];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int rl = lane & 3, pl = lane >> 2;
+  const int rl = (lane & 3) + 4 * (warp / NW), pl = lane >> 2;  // rows TR rl .. TR rl + TR-1
+  const int rp0 = (warp % NW) * 8 * RPT + pl;                   // replicas rp0 + 8 j
   const int32_t r0 = blockIdx.y * RC;
   const int32_t vrows = rt.valid - grp * F_ROWS;  // real rows of this group
   if (vrows <= 0) return;
@@ -182,7 +188,7 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
 #pragma unroll
     for (int i = 0; i < F_ROWS * F_QUADS / NT; ++i) {
       const int row = qr + i * (NT / F_QUADS);
-      cp_async16(dst + row * F_KC + f32_jpos(row, q), src + row * TILE);
+      cp_async16(dst + row * F_KC + f32_jpos<TR>(row, q), src + row * TILE);
     }
   };
   auto load_x = [&](int32_t st, int2 en) {
@@ -190,8 +196,9 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
     float* dst = xs + (st % F_STAGES) * (RC * F_KC);
     const float* src = a.xin + en.y + c_in;
 #pragma unroll
-    for (int i = 0; i < RC * F_QUADS / NT; ++i) {
+    for (int i = 0; i < (RC * F_QUADS + NT - 1) / NT; ++i) {
       const int rep = qr + i * (NT / F_QUADS);
+      if (RC * F_QUADS < NT && rep >= RC) return;
       const int32_t r = min(r0 + rep, a.R - 1);  // past the last replica: any valid row
       cp_async16(dst + rep * F_KC + f32_xpos(rep, q), src + (int64_t)r * a.n_pad);
     }
@@ -221,11 +228,11 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
     cp_async_commit();
   }
   int2 nxt = en[F_STAGES - 1];
-  float acc[RPT][8];
+  float acc[RPT][TR];
 #pragma unroll
   for (int j = 0; j < RPT; ++j)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) acc[j][i] = 0.f;
+    for (int i = 0; i < TR; ++i) acc[j][i] = 0.f;
   for (int32_t st = 0; st < ns; ++st) {
     cp_async_wait<F_STAGES - 2>();
     __syncthreads();  // stage st has landed; stage st - 1's buffers are free
@@ -233,15 +240,15 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
     load_x(st + F_STAGES - 1, nxt);
     cp_async_commit();
     nxt = entry(st + F_STAGES);
-    const float* jb = js + (st % F_STAGES) * (F_ROWS * F_KC) + rl * 8 * F_KC;
-    const float* xb = xs + (st % F_STAGES) * (RC * F_KC) + (warp * 8 * RPT + pl) * F_KC;
+    const float* jb = js + (st % F_STAGES) * (F_ROWS * F_KC) + rl * TR * F_KC;
+    const float* xb = xs + (st % F_STAGES) * (RC * F_KC) + rp0 * F_KC;
     const int nq = 2 * min(F_STAGE_CHUNKS, nc - st * F_STAGE_CHUNKS);
 #pragma unroll 2
     for (int k = 0; k < nq; ++k) {
-      float4 jv[8];
+      float4 jv[TR];
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
-        jv[i] = *reinterpret_cast<const float4*>(jb + i * F_KC + f32_jpos(rl * 8, k));
+      for (int i = 0; i < TR; ++i)
+        jv[i] = *reinterpret_cast<const float4*>(jb + i * F_KC + f32_jpos<TR>(rl * TR, k));
 #pragma unroll
       for (int j = 0; j < RPT; ++j) {
         float4 v = *reinterpret_cast<const float4*>(xb + j * 8 * F_KC + f32_xpos(pl, k));
@@ -249,13 +256,13 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
           v = make_float4(sb_operand(QH_SB_DISCRETE, v.x), sb_operand(QH_SB_DISCRETE, v.y),
                           sb_operand(QH_SB_DISCRETE, v.z), sb_operand(QH_SB_DISCRETE, v.w));
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[j][i] = fmaf(jv[i].x, v.x, acc[j][i]);
+        for (int i = 0; i < TR; ++i) acc[j][i] = fmaf(jv[i].x, v.x, acc[j][i]);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[j][i] = fmaf(jv[i].y, v.y, acc[j][i]);
+        for (int i = 0; i < TR; ++i) acc[j][i] = fmaf(jv[i].y, v.y, acc[j][i]);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[j][i] = fmaf(jv[i].z, v.z, acc[j][i]);
+        for (int i = 0; i < TR; ++i) acc[j][i] = fmaf(jv[i].z, v.z, acc[j][i]);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[j][i] = fmaf(jv[i].w, v.w, acc[j][i]);
+        for (int i = 0; i < TR; ++i) acc[j][i] = fmaf(jv[i].w, v.w, acc[j][i]);
       }
     }
   }
@@ -265,54 +272,58 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
   const float c0 = a.c0[rt.block];
   const float fe = deform_force(a.deform, rt.block, t, sb);
   auto index = [&](int j) -> size_t {
-    return (size_t)(r0 + warp * 8 * RPT + pl + 8 * j) * a.n_pad + row0 + rl * 8;
+    return (size_t)(r0 + rp0 + 8 * j) * a.n_pad + row0 + rl * TR;
   };
   if (vec4 && a.z_out == nullptr) {
     // rows past the block keep what they hold (zeros); x and y of the next replica load
     // while this one's are updated
-    float4 xn[2], yn[2];
+    using V = typename std::conditional<TR == 2, float2, float4>::type;
+    constexpr int VW = TR == 2 ? 2 : 4, NV = TR / VW;
+    union Rows {
+      V v[NV];
+      float f[TR];
+    };
+    Rows xn, yn;
     auto fetch = [&](int j) {
-      if (r0 + warp * 8 * RPT + pl + 8 * j >= a.R) return;
+      if (r0 + rp0 + 8 * j >= a.R) return;
       const size_t idx = index(j);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        xn[h] = *reinterpret_cast<const float4*>(a.xin + idx + 4 * h);
-        yn[h] = *reinterpret_cast<const float4*>(a.y + idx + 4 * h);
+      for (int h = 0; h < NV; ++h) {
+        xn.v[h] = *reinterpret_cast<const V*>(a.xin + idx + VW * h);
+        yn.v[h] = *reinterpret_cast<const V*>(a.y + idx + VW * h);
       }
     };
     fetch(0);
 #pragma unroll
     for (int j = 0; j < RPT; ++j) {
-      const float4 x4[2] = {xn[0], xn[1]}, y4[2] = {yn[0], yn[1]};
+      Rows xr = xn, yr = yn;
       if (j + 1 < RPT) fetch(j + 1);
-      if (r0 + warp * 8 * RPT + pl + 8 * j >= a.R) continue;
+      if (r0 + rp0 + 8 * j >= a.R) continue;
       const size_t idx = index(j);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float xv[4] = {x4[h].x, x4[h].y, x4[h].z, x4[h].w};
-        float yv[4] = {y4[h].x, y4[h].y, y4[h].z, y4[h].w};
+      for (int i = 0; i < TR; ++i) {
+        float x = xr.f[i], y = yr.f[i];
+        sb_update(a.sb, acc[j][i], x, y, a.dt, coef_x, a.dta0, c0, fe);
+        const bool real = rl * TR + i < vrows;
+        xr.f[i] = real ? x : xr.f[i];
+        yr.f[i] = real ? y : yr.f[i];
+      }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          float x = xv[i], y = yv[i];
-          sb_update(a.sb, acc[j][4 * h + i], x, y, a.dt, coef_x, a.dta0, c0, fe);
-          const bool real = rl * 8 + 4 * h + i < vrows;
-          xv[i] = real ? x : xv[i];
-          yv[i] = real ? y : yv[i];
-        }
-        *reinterpret_cast<float4*>(a.xout + idx + 4 * h) = make_float4(xv[0], xv[1], xv[2], xv[3]);
-        *reinterpret_cast<float4*>(a.y + idx + 4 * h) = make_float4(yv[0], yv[1], yv[2], yv[3]);
+      for (int h = 0; h < NV; ++h) {
+        *reinterpret_cast<V*>(a.xout + idx + VW * h) = xr.v[h];
+        *reinterpret_cast<V*>(a.y + idx + VW * h) = yr.v[h];
       }
     }
     return;
   }
 #pragma unroll 1
-  for (int i = 0; i < 8 * RPT; ++i) {  // the product alone (z_out), or unaligned buffers
-    const int j = i >> 3;
+  for (int i = 0; i < TR * RPT; ++i) {  // the product alone (z_out), or unaligned buffers
+    const int j = i / TR;
     float z = 0.f;
 #pragma unroll
-    for (int m = 0; m < 8 * RPT; ++m) z = m == i ? acc[m >> 3][m & 7] : z;
-    if (rl * 8 + (i & 7) >= vrows || r0 + warp * 8 * RPT + pl + 8 * j >= a.R) continue;
-    const size_t idx = index(j) + (i & 7);
+    for (int m = 0; m < TR * RPT; ++m) z = m == i ? acc[m / TR][m % TR] : z;
+    if (rl * TR + i % TR >= vrows || r0 + rp0 + 8 * j >= a.R) continue;
+    const size_t idx = index(j) + i % TR;
     if (a.z_out != nullptr) {
       a.z_out[idx] = z;
       continue;
@@ -324,23 +335,24 @@ __global__ void __launch_bounds__(32 * NW) k_step_f32(StepArgs a, const int2* __
   }
 }
 
-template <int RPT, int NW, bool DISC>
+template <int RPT, int NW, int TR, bool DISC>
 cudaError_t launch_f32_impl(cudaStream_t s, const Graph& g, const StepArgs& a,
                             const F32Chunks& ch, int vec4) {
   constexpr int RC = 8 * RPT * NW;
   constexpr size_t SMEM = sizeof(float) * F_STAGES * F_KC * (F_ROWS + RC);
-  StepLaunch l(dim3((unsigned)g.n_row_tiles * F_GROUPS, (unsigned)((a.R + RC - 1) / RC)), 32 * NW,
+  StepLaunch l(dim3((unsigned)g.n_row_tiles * F_GROUPS, (unsigned)((a.R + RC - 1) / RC)),
+               32 * NW * 8 / TR,
                SMEM, s, a.after_step != 0);
-  return cudaLaunchKernelEx(&l.cfg, k_step_f32<RPT, NW, DISC>, a, ch.list, ch.count, vec4);
+  return cudaLaunchKernelEx(&l.cfg, k_step_f32<RPT, NW, TR, DISC>, a, ch.list, ch.count, vec4);
 }
 
-template <int RPT, int NW>
+template <int RPT, int NW, int TR>
 cudaError_t f32_attr() {
   constexpr int SMEM = (int)sizeof(float) * F_STAGES * F_KC * (F_ROWS + 8 * RPT * NW);
-  cudaError_t e = cudaFuncSetAttribute(k_step_f32<RPT, NW, false>,
+  cudaError_t e = cudaFuncSetAttribute(k_step_f32<RPT, NW, TR, false>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_step_f32<RPT, NW, true>,
+    e = cudaFuncSetAttribute(k_step_f32<RPT, NW, TR, true>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
   return e;
 }
@@ -1383,9 +1395,9 @@ qh_status f32_prepare(Ctx* ctx, const Graph& g, const float* tile_f32, int32_t s
 }
 
 cudaError_t f32_set_attrs() {
-  cudaError_t e = f32_attr<4, 2>();
-  if (e == cudaSuccess) e = f32_attr<2, 2>();
-  if (e == cudaSuccess) e = f32_attr<1, 2>();
+  cudaError_t e = f32_attr<4, 2, 8>();
+  if (e == cudaSuccess) e = f32_attr<2, 2, 4>();
+  if (e == cudaSuccess) e = f32_attr<1, 1, 2>();
   return e;
 }
 
@@ -1395,24 +1407,26 @@ qh_status launch_step_f32(Ctx* ctx, const Graph& g, const StepArgs& a, const F32
   const uintptr_t bits = (uintptr_t)a.y | (uintptr_t)a.xout | (uintptr_t)a.z_out;
   const int vec4 = (bits & 15) == 0;
   const bool disc = a.sb == QH_SB_DISCRETE;
-  // Replicas per thread: few warps hide no latency, so a small graph takes fewer replicas
-  // per thread (more warps), a large one more (fewer shared-memory reads per FMA).
-  // Measured, us per step at 1 / 2 / 4 replicas a thread: 720 reads, R = 64 (192 warps
-  // at 1): 5.4 / 6.6 / 8.8; 720 reads, R = 256 (768): 8.6 / 7.4 / 8.9; 1,800 reads,
-  // R = 256 (960 warps at 2): 15.7 / 9.9 / 11.8; 720 reads, R = 1,024 (1,536): 17 / 16 /
-  // 13.9; 7,200 reads, R = 256 (3,648): 32.9 / 25.2 / 17.9.  And no thread for replicas
-  // past R: 32 blocks, R = 16: 17.4 / 16.5 / 27.1.
-  auto warps = [&](int rpt) -> int64_t {
-    return (int64_t)g.n_row_tiles * F_GROUPS * ((a.R + 16 * rpt - 1) / (16 * rpt)) * 2;
-  };
-  const int rpt = a.R <= 16 || warps(1) <= 3 * ctx->n_sm     ? 1
-                  : a.R <= 32 || warps(2) <= 10 * ctx->n_sm ? 2
-                                                            : 4;
+  // Outputs per thread.  A small graph's step is the latency of its column loop, so it takes
+  // 2 rows x 1 replica a thread (a quarter of the operand reads and FMAs per column in each
+  // warp, four times the warps); a large one 8 x 4 (fewest shared-memory reads per FMA); in
+  // between 4 x 2.  u = 32-row groups x 8-replica columns.  Measured, us per step at
+  // 2x1 / 4x2 / 8x4: 144 reads R = 64 (u = 64) 3.4 / 4.5 / 7.8; 720 reads R = 256 (768)
+  // 8.1 / 6.6 / 9.2; 7,200 reads R = 64 (1,824) 12.7 / 7.7 / 9.5; 1,200 SNPs R = 512 (2,560)
+  // 49.8 / 32.9 / 41.9; 720 reads R = 1,024 (3,072) 18.5 / 15.4 / 14.1; 7,200 reads R = 256
+  // (7,296) 39 / 23 / 17.9.  And no thread for replicas past R: 8 x 4 takes 64 a CTA, 4 x 2
+  // 32, 2 x 1 8 (12,000 SNPs R = 16: 21.3 / 30.4 / 45).
+  const int64_t u = (int64_t)g.n_row_tiles * F_GROUPS * ((a.R + 7) / 8);
   cudaError_t e;
-#define QH_F32(RPT)                                                               \
-  (disc ? launch_f32_impl<RPT, 2, true>(ctx->stream, g, a, ch, vec4)  \
-        : launch_f32_impl<RPT, 2, false>(ctx->stream, g, a, ch, vec4))
-  e = rpt == 1 ? QH_F32(1) : rpt == 2 ? QH_F32(2) : QH_F32(4);
+#define QH_F32(RPT, NW, TR)                                                \
+  (disc ? launch_f32_impl<RPT, NW, TR, true>(ctx->stream, g, a, ch, vec4)  \
+        : launch_f32_impl<RPT, NW, TR, false>(ctx->stream, g, a, ch, vec4))
+  if (a.R <= 16 || u <= 3 * ctx->n_sm)
+    e = QH_F32(1, 1, 2);
+  else if (a.R <= 32 || u <= 18 * ctx->n_sm)
+    e = QH_F32(2, 2, 4);
+  else
+    e = QH_F32(4, 2, 8);
 #undef QH_F32
   return e == cudaSuccess ? QH_OK : cuda_fail(ctx, e, "k_step_f32 launch");
 }

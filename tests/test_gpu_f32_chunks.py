@@ -28,10 +28,10 @@ def _dense(g, n_pad, pidx):
     return J
 
 
-# row counts around the 32-row groups and the 128-row tiles; replicas around the 16, 32 and
-# 64 a CTA takes at one, two and four per thread (400 reads x 400 replicas reach four)
-@pytest.mark.parametrize("reads,R", [(2, 1), (31, 15), (32, 16), (33, 17), (64, 33), (127, 64),
-                                     (129, 65), (257, 300), (400, 1600), (700, 100)])
+# row counts around the 32-row groups and the 128-row tiles; replicas around the 8, 32 and
+# 64 a CTA takes (400 reads x 1,600 replicas reach the last)
+@pytest.mark.parametrize("reads,R", [(2, 1), (33, 8), (96, 9), (31, 15), (32, 16), (33, 17), (64, 33), (127, 64),
+                                     (129, 65), (257, 300), (400, 1600), (400, 1633), (700, 100)])
 def test_product_exact_at_edges(reads, R):
     import torch
 
@@ -56,7 +56,7 @@ def test_product_exact_at_edges(reads, R):
 
 
 @pytest.mark.parametrize("variant,reads,R", [("ballistic", 129, 17), ("discrete", 161, 40),
-                                             ("adiabatic", 97, 9)])
+                                             ("adiabatic", 97, 9), ("ballistic", 400, 1633)])
 def test_unaligned_momentum_equals_aligned(variant, reads, R):
     """y from a buffer that is only 4-byte aligned takes scalar accesses: the same bits."""
     import torch
