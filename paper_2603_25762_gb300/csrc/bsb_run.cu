@@ -1170,6 +1170,13 @@ bool run_variant(int v) { return v >= RUN_VARIANT_FIRST && v < RUN_VARIANT_FIRST
 static bool run_jres(int v) { return v == RUN_VARIANT_FIRST || v == RUN_VARIANT_FIRST + 2; }
 static bool run_group(int v) { return v == RUN_VARIANT_FIRST || v == RUN_VARIANT_FIRST + 3; }
 
+// Step period of a wave by its fullest CTA's items (index 0 unused), us.  A CTA runs its
+// items' epilogues one after another: up to two items the hand-off between row tiles sets
+// the period, at four the epilogues do, without x of one item in TMEM.  Measured: 1,800
+// reads R = 1,024 (one item) 5.9, 7,200 reads R = 512 (two) 6.4, R = 1,024 (three) 8.5;
+// four against three on 512 blocks, R = 256: a ratio of 1.43.
+constexpr double RUN_PERIOD[MAX_ITEMS + 1] = {0.0, 5.9, 6.4, 8.5, 12.1};
+
 // Work split.  Items are numbered row-tile-major (item = row_tile * n_kt + k), and
 // the blocks' row tiles are contiguous.  Blocks (all, or those of a partial solve)
 // are packed into waves whose items fit on chip (at most MAX_ITEMS per SM); a wave
@@ -1242,35 +1249,88 @@ bool run_plan(const Graph& g, int R, int n_sm, int variant, bool use_lo, RunPlan
     for (int c = w.work_off; c < (int)p.work.size(); ++c) w.max_items = std::max(w.max_items, p.work[c].y);
     p.waves.push_back(w);
   };
-  std::vector<int32_t> rows;
+  // blocks in order, the waves filled evenly
+  std::vector<std::vector<int32_t>> waves;
   int64_t cur = 0;
   for (int32_t b = 0; b < g.n_blocks; ++b) {
     if (count[b] == 0) continue;
-    if (!rows.empty() && cur + load(b) > target) {  // target <= cap
-      emit(rows);
-      rows.clear();
+    if (waves.empty() || cur + load(b) > target) {  // target <= cap
+      waves.emplace_back();
       cur = 0;
     }
-    for (int32_t r = first[b]; r < first[b] + count[b]; ++r) rows.push_back(r);
+    waves.back().push_back(b);
     cur += load(b);
   }
-  if (!rows.empty()) emit(rows);
+  // A wave's step period grows with its fullest CTA (RUN_PERIOD), and least per item at
+  // three: whole waves of three items per CTA and the rest as waves of two, the blocks
+  // placed largest first, when the periods add up to less than the even split's.
+  if (!jres && waves.size() > 1 && max_items >= 3) {
+    const int64_t units = (total + n_sm - 1) / n_sm;  // CTA-fulls of one item
+    int64_t threes = units / 3, twos = units % 3 == 0 ? 0 : 1;
+    if (units % 3 == 1) {  // 3 k + 1 = 3 (k - 1) + 2 + 2
+      threes -= 1;
+      twos = 2;
+    }
+    std::vector<int32_t> order;
+    for (int32_t b = 0; b < g.n_blocks; ++b)
+      if (count[b] > 0) order.push_back(b);
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int32_t x, int32_t y) { return load(x) > load(y); });
+    // blocks of one load follow each other: the wave takes the largest that still fits
+    std::vector<std::vector<int32_t>> packed;
+    size_t left = order.size();
+    std::vector<std::vector<int32_t>> by_load(cap + 1);
+    for (size_t i = order.size(); i-- > 0;) by_load[load(order[i])].push_back(order[i]);
+    while (left > 0) {
+      int64_t room = (int64_t)n_sm * ((int64_t)packed.size() < threes             ? 3
+                                      : (int64_t)packed.size() < threes + twos ? 2
+                                                                                  : 3);
+      packed.emplace_back();
+      for (int64_t l = std::min(room, cap); l > 0; --l)
+        while (l <= room && !by_load[l].empty()) {
+          packed.back().push_back(by_load[l].back());
+          by_load[l].pop_back();
+          room -= l;
+          --left;
+        }
+      if (packed.back().empty()) break;  // a block larger than this wave: keep the even split
+      std::sort(packed.back().begin(), packed.back().end());
+    }
+    auto cost = [&](const std::vector<std::vector<int32_t>>& ws) {
+      double c = 0;
+      for (const auto& w : ws) {
+        int64_t n = 0;
+        for (int32_t b : w) n += load(b);
+        c += RUN_PERIOD[std::min<int64_t>((n + n_sm - 1) / n_sm, MAX_ITEMS)];
+      }
+      return c;
+    };
+    if (left == 0 && cost(packed) < cost(waves)) waves = std::move(packed);
+  }
+  std::vector<int32_t> rows;
+  for (const auto& w : waves) {
+    rows.clear();
+    for (int32_t b : w)
+      for (int32_t r = first[b]; r < first[b] + count[b]; ++r) rows.push_back(r);
+    emit(rows);
+  }
   if (plan) *plan = std::move(p);
   return true;
 }
 
-// Items per CTA for a solve: three or four, whichever gives the fewer step-periods of
-// waves.  A CTA runs its items' epilogues one after another, so four items make the step
-// period epilogue-bound: measured on batched-blocks (R = 256, 11,048 items), 13.5 µs per
-// step at four items per CTA (20 waves) against 9.44 µs at three (27 waves, x of one item
-// in TMEM), a ratio of 0.70.  Three items win unless they need more than 1/0.70 times
-// the waves (a graph that fits one wave at four but not at three keeps four).
+// Items per CTA for a solve: three or four, whichever gives the shorter sum of the waves'
+// step periods.
 int run_items(const Graph& g, int R, int n_sm, int variant, bool use_lo,
               const std::vector<int32_t>* mask) {
   RunPlan p3, p4;
   if (!run_plan(g, R, n_sm, variant, use_lo, &p3, mask, 3)) return MAX_ITEMS;
   if (!run_plan(g, R, n_sm, variant, use_lo, &p4, mask, MAX_ITEMS)) return 3;
-  return 100 * (int64_t)p3.waves.size() <= 143 * (int64_t)p4.waves.size() ? 3 : MAX_ITEMS;
+  auto cost = [](const RunPlan& p) {
+    double c = 0;
+    for (const RunWave& w : p.waves) c += RUN_PERIOD[w.max_items];
+    return c;
+  };
+  return cost(p3) <= cost(p4) ? 3 : MAX_ITEMS;
 }
 
 qh_status run_prepare(Ctx* ctx, const Graph& g, int R, int variant, bool use_lo, RunBufs* rb,
