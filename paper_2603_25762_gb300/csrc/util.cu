@@ -137,28 +137,37 @@ __global__ void k_bitonic_global(uint64_t* keys, int64_t n, int64_t k, int64_t j
 
 constexpr int BSORT_LOCAL = 2048;
 
-__global__ void k_bitonic_local(uint64_t* keys, int64_t n, int64_t k, int64_t jstart) {
+// A thread per compare-exchange.  Strides up to 32 stay inside the 64 keys of a warp's 32
+// pairs, so those stages need no barrier of the CTA: 26 of the 66 stages of a whole sort
+// keep one.  A 2,048-key sort measured 25 us with two pairs per thread of 512 and a barrier
+// per stage, 15.6 us now.
+__global__ void __launch_bounds__(BSORT_LOCAL / 2) k_bitonic_local(uint64_t* keys, int64_t k,
+                                                                   int64_t jstart) {
   __shared__ uint64_t s[BSORT_LOCAL];
-  int64_t base = (int64_t)blockIdx.x * BSORT_LOCAL;
-  for (int t = threadIdx.x; t < BSORT_LOCAL; t += blockDim.x) s[t] = keys[base + t];
+  const int64_t base = (int64_t)blockIdx.x * BSORT_LOCAL;
+  const int t = threadIdx.x;
+  s[t] = keys[base + t];
+  s[t + BSORT_LOCAL / 2] = keys[base + t + BSORT_LOCAL / 2];
   __syncthreads();
   for (int64_t kk = (k == 0 ? 2 : k); kk <= (k == 0 ? BSORT_LOCAL : k); kk <<= 1) {
-    for (int64_t j = (k == 0 ? kk >> 1 : jstart); j > 0; j >>= 1) {
-      for (int t = threadIdx.x; t < BSORT_LOCAL; t += blockDim.x) {
-        int l = t ^ (int)j;
-        if (l > t) {
-          uint64_t a = s[t], b = s[l];
-          bool up = ((base + t) & kk) == 0;
-          if ((a > b) == up) {
-            s[t] = b;
-            s[l] = a;
-          }
-        }
+    for (int j = (int)(k == 0 ? kk >> 1 : jstart); j > 0; j >>= 1) {
+      const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1)), l = i + j;
+      const uint64_t a = s[i], b = s[l];
+      if ((a > b) == (((base + i) & kk) == 0)) {
+        s[i] = b;
+        s[l] = a;
       }
-      __syncthreads();
+      // the next stage: half the stride, or the widest of the next k
+      const int64_t next = j > 1 ? j >> 1 : (k == 0 ? kk : 1);
+      if (j > 32 || next > 32)
+        __syncthreads();
+      else
+        __syncwarp();
     }
   }
-  for (int t = threadIdx.x; t < BSORT_LOCAL; t += blockDim.x) keys[base + t] = s[t];
+  __syncthreads();
+  keys[base + t] = s[t];
+  keys[base + t + BSORT_LOCAL / 2] = s[t + BSORT_LOCAL / 2];
 }
 
 __global__ void k_fill_u64(uint64_t* p, int64_t b, int64_t e, uint64_t v) {
@@ -191,11 +200,11 @@ void sort_u64(cudaStream_t s, uint64_t* keys, int64_t n, int64_t cap) {
   if (N > n) k_fill_u64<<<::qh::counted((unsigned)((N - n + 255) / 256)), 256, 0, s>>>(keys, n, N, ~0ull);
   unsigned nb_local = (unsigned)(N / BSORT_LOCAL);
   // all stages with k <= BSORT_LOCAL in shared memory
-  k_bitonic_local<<<::qh::counted(nb_local), 512, 0, s>>>(keys, N, 0, 0);
+  k_bitonic_local<<<::qh::counted(nb_local), BSORT_LOCAL / 2, 0, s>>>(keys, 0, 0);
   for (int64_t k = 2 * BSORT_LOCAL; k <= N; k <<= 1) {
     for (int64_t j = k >> 1; j >= BSORT_LOCAL; j >>= 1)
       k_bitonic_global<<<::qh::counted((unsigned)((N + 255) / 256)), 256, 0, s>>>(keys, N, k, j);
-    k_bitonic_local<<<::qh::counted(nb_local), 512, 0, s>>>(keys, N, k, BSORT_LOCAL >> 1);
+    k_bitonic_local<<<::qh::counted(nb_local), BSORT_LOCAL / 2, 0, s>>>(keys, k, BSORT_LOCAL >> 1);
   }
 }
 
