@@ -167,9 +167,9 @@ void clear_foreign_error(Ctx* ctx) {
 }
 
 qh_status check_err_word(Ctx* ctx) {
-  int32_t herr = 0;
-  QH_CUDA_TRY(cudaMemcpyAsync(&herr, ctx->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+  QH_CUDA_TRY(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
   QH_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+  const int32_t herr = *ctx->h_err;
   if (herr & ERR_TIMEOUT) {
     cudaMemsetAsync(ctx->d_err, 0, sizeof(int32_t), ctx->stream);
     return set_err(ctx, QH_ETIMEOUT, "a bounded device wait expired in the bSB step kernel");
@@ -334,6 +334,7 @@ qh_status qh_create(qh_ctx** out, int device, void* stream) {
     ctx->mem.fail_after = std::make_shared<int64_t>(-1);
   }
   if (cudaMalloc(&ctx->d_err, sizeof(int32_t)) != cudaSuccess ||
+      cudaHostAlloc((void**)&ctx->h_err, sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess ||
       cudaMemsetAsync(ctx->d_err, 0, sizeof(int32_t), ctx->stream) != cudaSuccess) {
     delete h;
     return QH_ECUDA;
@@ -357,6 +358,7 @@ void qh_destroy(qh_ctx* h) {
   for (void* p : ctx->slots)
     if (p) cudaFree(p);
   if (ctx->d_err) cudaFree(ctx->d_err);
+  if (ctx->h_err) cudaFreeHost(ctx->h_err);
   for (auto& e : ctx->ev)
     if (e) cudaEventDestroy(e);
   if (ctx->mem.alive) *ctx->mem.alive = false;  // graphs and solutions left behind free synchronously

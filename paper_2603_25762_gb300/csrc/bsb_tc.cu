@@ -128,13 +128,15 @@ __global__ void __launch_bounds__(128) k_step_tc(const __grid_constant__ CUtenso
 #pragma unroll
       for (int j = 0; j < 32; ++j) v[j] = 0u;
     }
-    if (!vrow) continue;
     const size_t b0 = base + (size_t)(c * 32) * a.n_pad;
-    if (a.z_out != nullptr) {
+    if (a.z_out != nullptr) {  // z is zero at padding vertices
+      if (ok)
 #pragma unroll
-      for (int j = 0; j < 32; ++j) a.z_out[b0 + (size_t)j * a.n_pad] = __uint_as_float(v[j]);
+        for (int j = 0; j < 32; ++j)
+          a.z_out[b0 + (size_t)j * a.n_pad] = vrow ? __uint_as_float(v[j]) : 0.f;
       continue;
     }
+    if (!vrow) continue;
     float xs[32], ys[32];
 #pragma unroll
     for (int j = 0; j < 32; ++j) {

@@ -192,6 +192,7 @@ struct Ctx {
   int n_sm = 148;
   std::string err;
   int32_t* d_err = nullptr;
+  int32_t* h_err = nullptr;         // pinned host word d_err is read back into
   std::vector<void*> slots;         // grow-only scratch buffers
   std::vector<size_t> slot_bytes;
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
