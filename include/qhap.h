@@ -223,7 +223,8 @@ typedef struct {
                            patience > 0): 0 = inside the multi-step launch when it
                            applies (a multi-step step kernel, integer weights, at
                            most three items per SM fit every block) and pays
-                           (check_every <= 128), else between launches; 1 = always
+                           (check_every <= 22 to 128, by the items per SM), else
+                           between launches; 1 = always
                            between launches, with the separate cut kernels.  Both
                            give the same steps_run, cuts and spins.  Other values
                            -> QH_EINVAL */

@@ -889,19 +889,27 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
   // Early-stop checks inside the multi-step launch: integer weights, so that the tensor
   // cores give the energies exactly (every row sum of |J| below 2^24), and every block
   // in one wave at three items per SM (the fourth item's TMEM holds the check product).
-  // The kernel with checks runs its steps about 20% slower than the one without, and a
-  // check between launches costs about 30 step times (hifi-region, 1,024 replicas), so
-  // the checks move inside the launch when they come at least every FUSED_CHECK_MAX
-  // steps.
-  constexpr int32_t FUSED_CHECK_MAX = 128;
+  // The kernel with checks keeps no x in TMEM and runs its steps slower (hifi-region, three
+  // items per SM: 11.4 against 8.5 us; one item 6.4 against 6.2), and a check between
+  // launches costs about 80 us.  Measured, us per step inside / between at check_every = 20,
+  // 25, 32, 50: three items 12.8 / 13.0, 12.4 / 12.0, 12.2 / 11.3, 11.7 / 10.1; two items
+  // 9.0 / 9.6, 8.8 / 9.0, 8.6 / 8.5, 8.3 / 7.8; one item 6.9 / 8.4, 6.8 / 8.0, 6.7 / 7.6, 6.6 /
+  // 7.0, and equal from 100 on.  So the checks move inside the launch up to this period.
+  constexpr int32_t FUSED_CHECK_MAX[4] = {0, 128, 30, 22};
   bool fused = multistep && early && !track && o->check_mode == 0 && W.integer_weights &&
-               o->check_every <= FUSED_CHECK_MAX;
+               o->check_every <= FUSED_CHECK_MAX[1];
   if (fused) {
     int32_t max_n = 0;
     for (int32_t b = 0; b < nb; ++b) max_n = std::max(max_n, W.h_block_size[b]);
+    RunPlan fp;
     fused = W.max_abs_w * (double)max_n < 16777216.0 &&
-            run_plan(W, R, ctx->n_sm, tplan.variant, a.use_lo != 0, nullptr,
+            run_plan(W, R, ctx->n_sm, tplan.variant, a.use_lo != 0, &fp,
                      sel ? &sel_mask : nullptr, 3);
+    if (fused) {
+      int items = 1;
+      for (const RunWave& w : fp.waves) items = std::max(items, w.max_items);
+      fused = o->check_every <= FUSED_CHECK_MAX[items];
+    }
   }
   RunCheck chk;
   if (multistep) {
@@ -927,9 +935,11 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
     chk.decided = chk.e_cnt + 2 * nb;
     chk.stop_t = reinterpret_cast<int32_t*>(chk.e_cnt + 3 * nb);
   }
-  // every replica's cut of the state x (signs into B.signs for the picks and spins)
+  // every replica's cut of the state x.  The transposed signs (B.signs) are for the gathered
+  // cuts and for the spins that track_best keeps; otherwise the spins come from x.
+  const bool need_signs = !tc_cut || track;
   auto replica_cuts = [&](const float* xc, const int32_t* act) -> qh_status {
-    launch_signs(s, W, R, xc, B.signs);
+    if (need_signs) launch_signs(s, W, R, xc, B.signs);
     if (!tc_cut) {
       launch_cut(s, W, R, B.signs, W.w, sum_w_work, B.node_val, B.cuts, act);
       return QH_OK;
@@ -1084,7 +1094,10 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
       if (st != QH_OK) return st;
     }
     launch_pick_best(s, nb, R, B.cuts, B.best_r, B.best_cut, B.active);
-    launch_extract_spins(s, W, R, B.signs, B.best_r, B.spins, B.active);
+    if (need_signs)
+      launch_extract_spins(s, W, R, B.signs, B.best_r, B.spins, B.active);
+    else
+      launch_extract_spins_x(s, W, x_final, B.best_r, B.spins, B.active);
     if (track)  // the best result during the run, unless the final one is strictly better
       launch_track_final(s, W, B.best_cut, B.best_r, B.active, B.kept_cut, B.kept_r, B.kept_flag,
                          B.kept_spins, B.spins);

@@ -450,6 +450,9 @@ void launch_track_final(cudaStream_t s, const Graph& g, double* best_cut, int32_
                         int32_t* flag, const int8_t* kept_spins, int8_t* spins);
 void launch_extract_spins(cudaStream_t s, const Graph& g, int32_t R, const int8_t* signs_t,
                           const int32_t* best_r, int8_t* spins, const int32_t* active);
+// the same from the state x, [R][n_pad]
+void launch_extract_spins_x(cudaStream_t s, const Graph& g, const float* x, const int32_t* best_r,
+                            int8_t* spins, const int32_t* active);
 void launch_block_sums(cudaStream_t s, const Graph& g, const double* w, double* sum_w,
                        double* sum_j2, double* node_tmp /* 2 * n_nodes */);
 // Refill the band tiles and the remainder CSR values of a CSR-mode graph from weights
