@@ -334,7 +334,7 @@ qh_status qh_create(qh_ctx** out, int device, void* stream) {
     ctx->mem.fail_after = std::make_shared<int64_t>(-1);
   }
   if (cudaMalloc(&ctx->d_err, sizeof(int32_t)) != cudaSuccess ||
-      cudaHostAlloc((void**)&ctx->h_err, sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess ||
+      cudaHostAlloc((void**)&ctx->h_err, 3 * sizeof(int32_t), cudaHostAllocDefault) != cudaSuccess ||
       cudaMemsetAsync(ctx->d_err, 0, sizeof(int32_t), ctx->stream) != cudaSuccess) {
     delete h;
     return QH_ECUDA;
@@ -1057,9 +1057,17 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
       if (st != QH_OK) return st;
       launch_stop_fixup(s, W, R, chk, B.x, B.steps_run);
     } else if (multistep) {
+      // A launch over stopped blocks still costs its checks (about 50 us), so the host keeps
+      // one period ahead of the device and ends the loop when no block runs any more.
       const int32_t chunk = checking ? o->check_every : max_steps;
-      for (int32_t t0 = 0; t0 < max_steps; t0 += chunk) {
+      volatile int32_t* some_run = ctx->h_err + 1;
+      for (int32_t t0 = 0, k = 0; t0 < max_steps; t0 += chunk, ++k) {
         const int32_t t1 = std::min(max_steps, t0 + chunk);
+        if (checking && early && k >= 2) {
+          QH_CUDA_TRY(cudaEventSynchronize(ctx->ev[4 + (k & 1)]));
+          if (!some_run[k & 1]) break;
+        }
+        launches += (int64_t)rb.waves.size();
         qh_status st = launch_run(ctx, W, a, rb, B.xh0, B.xh1, t0, t1);
         if (st != QH_OK) return st;
         if (checking && t1 < max_steps) {
@@ -1071,9 +1079,12 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
           if (track)
             launch_track_check(s, W, R, B.signs, B.best_cut, B.best_r, B.running, t1, B.steps_b,
                                B.kept_cut, B.kept_r, B.kept_flag, B.kept_spins);
-          if (early)
+          if (early) {
             launch_early_stop(s, nb, B.best_cut, B.seen, B.stall, B.running, B.steps_run,
                               o->patience, t1, B.steps_b);
+            launch_any_running(s, nb, B.running, t1, B.steps_b, ctx->h_err + 1 + (k & 1));
+            QH_CUDA_TRY(cudaEventRecord(ctx->ev[4 + (k & 1)], s));
+          }
         }
       }
     } else {
@@ -1123,10 +1134,10 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ctx->ev[2], ctx->ev[3]);
     step_ms_total += ms;
-    launches += fused ? (int64_t)rb.waves.size()
-                : multistep ? (int64_t)rb.waves.size() *
-                                  (checking ? (max_steps + o->check_every - 1) / o->check_every : 1)
-                            : max_steps;
+    if (fused)
+      launches += (int64_t)rb.waves.size();
+    else if (!multistep)
+      launches += max_steps;
     for (int32_t b = 0; b < nb; ++b)
       if (h_active[b]) {
         spin_updates += (double)G.h_block_size[b] * R * h_steps_run[b];

@@ -1128,6 +1128,14 @@ __global__ void k_early_stop(int32_t nb, const double* __restrict__ best_cut, do
   }
 }
 
+__global__ void k_any_running(int32_t nb, const int32_t* __restrict__ active, int32_t t_done,
+                              const int32_t* __restrict__ steps_b, int32_t* out) {
+  int any = 0;
+  for (int32_t b = threadIdx.x; b < nb; b += blockDim.x) any |= active[b] && t_done < steps_b[b];
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) *out = any;
+}
+
 // Best during the run (track_best): after a check's pick, a running block whose best cut
 // beats the kept one keeps it (cut, replica; flag = 1 to copy its spins); at the end the
 // kept result replaces the final one unless the final is strictly better.
@@ -1672,6 +1680,11 @@ void launch_early_stop(cudaStream_t s, int32_t n_blocks, const double* best_cut,
   if (n_blocks > 0)
     k_early_stop<<<::qh::counted(nblk(n_blocks)), 256, 0, s>>>(n_blocks, best_cut, best_seen, stall, active,
                                                steps_run, patience, t_done, steps_b);
+}
+
+void launch_any_running(cudaStream_t s, int32_t n_blocks, const int32_t* active, int32_t t_done,
+                        const int32_t* steps_b, int32_t* out) {
+  k_any_running<<<::qh::counted(1), 256, 0, s>>>(n_blocks, active, t_done, steps_b, out);
 }
 
 void launch_track_check(cudaStream_t s, const Graph& g, int32_t R, const int8_t* signs_t,

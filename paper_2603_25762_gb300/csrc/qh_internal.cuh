@@ -192,10 +192,11 @@ struct Ctx {
   int n_sm = 148;
   std::string err;
   int32_t* d_err = nullptr;
-  int32_t* h_err = nullptr;         // pinned host word d_err is read back into
+  int32_t* h_err = nullptr;         // pinned host word d_err is read back into, and after it
+                                    // the last two checks' "some block still runs" words
   std::vector<void*> slots;         // grow-only scratch buffers
   std::vector<size_t> slot_bytes;
-  cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
+  cudaEvent_t ev[6] = {};           // solve and step loop begin / end; the last two checks
   // one captured step loop, replayed while its shape is unchanged
   cudaGraphExec_t loop_exec = nullptr;
   std::string loop_key;
@@ -438,6 +439,9 @@ void launch_advance(cudaStream_t s, int32_t* t_base, int32_t n);
 void launch_early_stop(cudaStream_t s, int32_t n_blocks, const double* best_cut, double* best_seen,
                        int32_t* stall, int32_t* active, int32_t* steps_run, int32_t patience,
                        int32_t t_done, const int32_t* steps_b);
+// *out (pinned host memory) = does a block still have steps to run after t_done?
+void launch_any_running(cudaStream_t s, int32_t n_blocks, const int32_t* active, int32_t t_done,
+                        const int32_t* steps_b, int32_t* out);
 // Best during the run (track_best): after a check (signs, cut and pick of that state)
 // keep each running block's better result; at the end let the kept result replace the
 // final one unless the final is strictly better.

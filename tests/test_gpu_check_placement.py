@@ -44,3 +44,24 @@ def test_check_placement(R, check_every, inside):
         s.free()
     g.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [1, 10])
+def test_launches_end_with_the_last_block(n):
+    """Checks between launches: the host is one period ahead of the device, so one period
+    follows the one in which the last block stopped."""
+    ctx = qhap.Context(0)
+    fr = synth.tiny_reads(1001) if n == 1 else synth.batched_blocks(1004, n_blocks=n, n_min=20,
+                                                                    n_max=400)
+    g = ctx.build_graph(fr, mode=qhap.MODE_READ)
+    sol = ctx.solve(g, replicas=128, steps=3000, precision=qhap.PREC_BF16, seed=2, check_every=40,
+                    patience=3, check_mode=1, step_kernel="multistep-stream-tile")
+    run = max(sol.block(b)["steps_run"] for b in range(g.n_blocks))
+    assert run < 3000 - 80
+    assert sol.timing()["n_step_launches"] == run // 40 + 1
+    _, trace = sol.check_trace()
+    assert np.isfinite(trace[: run // 40]).any(axis=1).all()
+    assert np.isnan(trace[run // 40:]).all()
+    sol.free()
+    g.free()
+    ctx.close()
