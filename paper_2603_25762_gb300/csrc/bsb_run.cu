@@ -42,9 +42,10 @@
 // separate instantiation (CHECK = true): the kernel without them carries none of their
 // code.
 //
-// Roles (384 threads): warp 0 = TMA producer (six lanes for X_hat, six for J), warp 1 = MMA issuer (one
-// thread), warps 2-9 = epilogue (TMEM lane quarter = warp % 4 = 32 vertices, two warps
-// per quarter split the 128 replicas), warp 10 = signal, warp 11 = J producer.  With JRES
+// Roles (384 threads): warp 0 = TMA producer (a lane per copy: one for X_hat and one for J
+// of each ring slot), warp 1 = MMA issuer (one thread), warps 2-9 = epilogue (TMEM lane
+// quarter = warp % 4 = 32 vertices, two warps per quarter split the 128 replicas), warp
+// 10 = signal, warp 11 = J producer.  With JRES
 // the J tiles of the CTA's single row tile stay in shared memory for the whole launch and
 // only X_hat streams.  Otherwise J and X_hat K-slices stream through the ring: copied
 // together by warp 0, or (jsplit: the kernel without checks, rows wider than the ring)
