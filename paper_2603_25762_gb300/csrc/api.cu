@@ -1647,6 +1647,20 @@ qh_status qh_debug_run_trace(qh_ctx* h, const qh_graph* gh, int32_t R, int32_t s
   return check_err_word(ctx);
 }
 
+// Do the caller's arrays hold a NaN, an infinity or a value near the overflow?  The products
+// leave out the parts of J without a nonzero; 0 * x is not 0 for such an x, so they then
+// walk every stored tile.  (A solve's own x stays in [-1, 1].)
+static qh_status find_overflow(Ctx* ctx, std::initializer_list<const float*> arrays, size_t n,
+                               bool* found) {
+  volatile int32_t* word = ctx->h_err + 1;
+  *word = 0;
+  for (const float* v : arrays) launch_find_overflow(ctx->stream, v, (int64_t)n, ctx->h_err + 1);
+  QH_STAGE_CHECK("debug: range of the state");
+  QH_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+  *found = *word != 0;
+  return QH_OK;
+}
+
 qh_status qh_debug_matvec(qh_ctx* h, const qh_graph* gh, int32_t precision, int32_t R, const float* x,
                           float* z) {
   if (!h || !gh || !x || !z) return QH_EINVAL;
@@ -1708,7 +1722,10 @@ qh_status qh_debug_matvec(qh_ctx* h, const qh_graph* gh, int32_t precision, int3
     a.xin = x;
     a.xout = nullptr;
     F32Chunks ch;
-    st = f32_prepare(ctx, g, g.tile_f32, QH_SB_BALLISTIC, &ch);
+    bool wild = false;
+    st = find_overflow(ctx, {x}, (size_t)R * g.n_pad, &wild);
+    if (st == QH_OK)
+      st = f32_prepare(ctx, g, g.tile_f32, wild ? QH_SB_ADIABATIC : QH_SB_BALLISTIC, &ch);
     if (st == QH_OK) st = launch_step_f32(ctx, g, a, ch);
     if (st) return st;
   } else {
@@ -1776,6 +1793,10 @@ qh_status qh_debug_steps_v(qh_ctx* h, const qh_graph* gh, int32_t precision, int
   if (st) return st;
   const size_t NS = (size_t)R * g.n_pad;
   cudaStream_t s = ctx->stream;
+  bool wild = false;
+  if (nsteps > 0) st = find_overflow(ctx, {x, y}, NS, &wild);
+  if (st) return st;
+  if (wild) a.kslice = nullptr;
   float* xu = x;  // user buffers in [R][n_pad]
   float* yu = y;
   const int csr_v = step_kernel >= 0 ? step_kernel : csr_default_variant(g, precision, R);
@@ -1794,7 +1815,8 @@ qh_status qh_debug_steps_v(qh_ctx* h, const qh_graph* gh, int32_t precision, int
     if (!x1) return set_err(ctx, QH_ENOMEM, "allocation failed (debug)");
     QH_CUDA_TRY(cudaMemcpyAsync(x1, x, NS * 4, cudaMemcpyDeviceToDevice, s));
     F32Chunks ch;
-    if (!g.csr_mode) st = f32_prepare(ctx, g, g.tile_f32, sb_variant, &ch);
+    if (!g.csr_mode)
+      st = f32_prepare(ctx, g, g.tile_f32, wild ? QH_SB_ADIABATIC : sb_variant, &ch);
     if (st) return st;
     for (int32_t k = 0; k < nsteps; ++k) {
       a.t = t0 + k;

@@ -1128,6 +1128,14 @@ __global__ void k_early_stop(int32_t nb, const double* __restrict__ best_cut, do
   }
 }
 
+__global__ void k_find_overflow(const float* __restrict__ v, int64_t n, int32_t* out) {
+  int bad = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    bad |= !(fabsf(v[i]) <= 1e38f);
+  if (__syncthreads_or(bad) && threadIdx.x == 0) *out = 1;
+}
+
 __global__ void k_any_running(int32_t nb, const int32_t* __restrict__ active, int32_t t_done,
                               const int32_t* __restrict__ steps_b, int32_t* out) {
   int any = 0;
@@ -1680,6 +1688,12 @@ void launch_early_stop(cudaStream_t s, int32_t n_blocks, const double* best_cut,
   if (n_blocks > 0)
     k_early_stop<<<::qh::counted(nblk(n_blocks)), 256, 0, s>>>(n_blocks, best_cut, best_seen, stall, active,
                                                steps_run, patience, t_done, steps_b);
+}
+
+void launch_find_overflow(cudaStream_t s, const float* v, int64_t n, int32_t* out) {
+  if (n > 0)
+    k_find_overflow<<<::qh::counted((unsigned)std::min<int64_t>((n + 255) / 256, 1024)), 256, 0, s>>>(
+        v, n, out);
 }
 
 void launch_any_running(cudaStream_t s, int32_t n_blocks, const int32_t* active, int32_t t_done,

@@ -439,6 +439,8 @@ void launch_advance(cudaStream_t s, int32_t* t_base, int32_t n);
 void launch_early_stop(cudaStream_t s, int32_t n_blocks, const double* best_cut, double* best_seen,
                        int32_t* stall, int32_t* active, int32_t* steps_run, int32_t patience,
                        int32_t t_done, const int32_t* steps_b);
+// *out (pinned host memory, zeroed before) becomes 1 if an entry of v is NaN or above 1e38
+void launch_find_overflow(cudaStream_t s, const float* v, int64_t n, int32_t* out);
 // *out (pinned host memory) = does a block still have steps to run after t_done?
 void launch_any_running(cudaStream_t s, int32_t n_blocks, const int32_t* active, int32_t t_done,
                         const int32_t* steps_b, int32_t* out);
