@@ -182,7 +182,7 @@ qh_status check_err_word(Ctx* ctx) {
 }
 
 // Time every valid step-kernel variant on the live state for a few steps and keep
-// the fastest for this graph shape.  The state is re-initialised afterwards.
+// the fastest for this graph shape (the multi-step family first, below).  The state is re-initialised afterwards.
 std::string tune_key(const Graph& g, int R, int use_lo, int sb) {
   char kb[160];
   snprintf(kb, sizeof kb, "%d|%d|%lld|%d|%d|%d|%d", R, g.n_row_tiles, (long long)g.n_tiles,
@@ -215,8 +215,15 @@ qh_status autotune(Ctx* ctx, const Graph& g, StepArgs a, const SolveBufs& B, int
                    bool allow_run) {
   const std::string kb = tune_key(g, R, 0, a.sb);
   cudaStream_t s = ctx->stream;
-  float best = 1e30f;
-  int best_v = -1;
+  // The per-step and the multi-step kernels round y differently, so which family runs must
+  // not hang on a close race: a per-step kernel is taken only where it is FAMILY_EDGE times
+  // faster.  Six steps also charge the multi-step launch's fixed cost (about 10 us) to few
+  // steps.  Measured over whole solves, us per step multi / per-step, at the per-step
+  // kernels' best: 4,000 SNPs R = 128 BF16X2 12.3 / 10.3, 903 reads R = 256 6.0 / 6.0;
+  // elsewhere the multi-step kernel leads, to 17.5 / 57.6 on 40 blocks at R = 256.
+  constexpr float FAMILY_EDGE = 1.6f;
+  float best[2] = {1e30f, 1e30f};  // per-step, multi-step
+  int best_v[2] = {-1, -1};
   std::string rep;
   for (int v = 0; v < tc_n_variants(); ++v) {
     if (!tc_variant_ok(v, g, R, ctx->n_sm, a.use_lo != 0)) continue;
@@ -250,15 +257,16 @@ qh_status autotune(Ctx* ctx, const Graph& g, StepArgs a, const SolveBufs& B, int
     char line[96];
     snprintf(line, sizeof line, "%s%s=%.2fus", rep.empty() ? "" : ";", tc_variant_name(v), ms * 1e3f);
     rep += line;
-    if (ms < best) {
-      best = ms;
-      best_v = v;
+    const int fam = run_variant(v) ? 1 : 0;
+    if (ms < best[fam]) {
+      best[fam] = ms;
+      best_v[fam] = v;
     }
   }
   qh_status st = check_err_word(ctx);
   if (st != QH_OK) return st;
-  plan->variant = best_v;
-  ctx->tuned.emplace_back(kb, best_v);
+  plan->variant = best_v[best_v[1] >= 0 && best[1] <= FAMILY_EDGE * best[0] ? 1 : 0];
+  ctx->tuned.emplace_back(kb, plan->variant);
   ctx->tune_report = rep;
   return QH_OK;
 }
