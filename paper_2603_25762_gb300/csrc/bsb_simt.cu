@@ -6,6 +6,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "chunk.cuh"
 #include "qh_internal.cuh"
 #include "util.cuh"
 
@@ -83,8 +84,7 @@ __global__ void __launch_bounds__(256) k_x_to_sign4(const float* __restrict__ x,
 // out changes no bit; adiabatic SB has no walls, its x may overflow, and it walks every
 // chunk (F32Chunks::all).
 constexpr int F_ROWS = 32;             // rows of a group
-constexpr int F_COLS = 8;              // columns of a chunk: one 32-byte sector of x
-constexpr int F_TILE_CHUNKS = TILE / F_COLS;
+static_assert(TILE == F32_TILE, "chunk records");
 constexpr int F_GROUPS = TILE / F_ROWS;
 constexpr int F_STAGE_CHUNKS = 4;      // chunks per pipeline stage
 constexpr int F_KC = F_COLS * F_STAGE_CHUNKS;
@@ -99,8 +99,7 @@ __device__ __forceinline__ int f32_jpos(int row, int q) {
 __device__ __forceinline__ int f32_xpos(int rep, int q) { return (q ^ (rep & 7)) * 4; }
 
 // Chunk lists: CTA per row tile.  Group g's list starts at entry f32_begin * 64 +
-// g * 16 * n_hi, columns ascending: .x = offset of the chunk's first column in the FP32
-// tiles (in units of 8 floats), .y = its first padded column.
+// g * 16 * n_hi, columns ascending: .x = the chunk (f32_chunk), .y = its first padded column.
 __global__ void __launch_bounds__(256) k_f32_chunks(const RowTile* __restrict__ rts,
                                                     const int32_t* __restrict__ tile_col,
                                                     const float* __restrict__ tile_f32, int all,
@@ -115,7 +114,7 @@ __global__ void __launch_bounds__(256) k_f32_chunks(const RowTile* __restrict__ 
   for (int32_t e = 0; e < rt.n_hi; ++e) {
     // warp w looks at rows 16 w .. 16 w + 15, lane l at columns 4 l .. 4 l + 3
     const float4* src = reinterpret_cast<const float4*>(
-        tile_f32 + (int64_t)(rt.f32_begin + e) * (TILE * TILE) + warp * 16 * TILE) + lane;
+        tile_f32 + ((int64_t)rt.f32_begin + e) * (TILE * TILE) + warp * 16 * TILE) + lane;
     bool nz = false;
     if (!all) {
 #pragma unroll
@@ -133,8 +132,7 @@ __global__ void __launch_bounds__(256) k_f32_chunks(const RowTile* __restrict__ 
       const uint32_t mask = __ballot_sync(0xffffffffu, on);
       if (on)
         out[n + __popc(mask & ((1u << lane) - 1u))] =
-            make_int2((rt.f32_begin + e) * (TILE * TILE / F_COLS) + lane,
-                      tile_col[rt.tile_begin + e] * TILE + lane * F_COLS);
+            make_int2(f32_chunk(e, lane), tile_col[rt.tile_begin + e] * TILE + lane * F_COLS);
       n += __popc(mask);
     }
     __syncthreads();
@@ -199,6 +197,7 @@ __global__ void __launch_bounds__(32 * NW * 8 / TR) k_step_f32(StepArgs a, const
                     (int64_t)grp * F_TILE_CHUNKS * rt.n_hi;
   // this thread copies quad q (4 of the stage's 32 columns) of some rows and replicas
   const int q = tid % F_QUADS, qr = tid / F_QUADS, c_of = q >> 1, c_in = (q & 1) * 4;
+  const float* const jrow = a.tile_f32 + f32_row_offset(rt.f32_begin) + (grp * F_ROWS) * TILE + c_in;
   auto entry = [&](int32_t st) -> int2 {
     const int32_t c = st * F_STAGE_CHUNKS + c_of;
     return c < nc ? lst[c] : make_int2(-1, 0);
@@ -206,7 +205,7 @@ __global__ void __launch_bounds__(32 * NW * 8 / TR) k_step_f32(StepArgs a, const
   auto load_j = [&](int32_t st, int2 en) {
     if (en.x < 0) return;
     float* dst = js + (st % F_STAGES) * (F_ROWS * F_KC);
-    const float* src = a.tile_f32 + (int64_t)en.x * F_COLS + (grp * F_ROWS) * TILE + c_in;
+    const float* src = jrow + f32_chunk_offset(en.x);
 #pragma unroll
     for (int i = 0; i < F_ROWS * F_QUADS / NT; ++i) {
       const int row = qr + i * (NT / F_QUADS);
