@@ -834,29 +834,37 @@ __global__ void k_cut_nodes_few(int32_t n, const int64_t* __restrict__ rp,
   }
 }
 
-// Real weights over many replicas: the same per-vertex sums in fixed point.  A weight is
-// the integer W = rn(w scale), |W| <= 2^CUT_BITS (scale a power of two from the largest
-// |w|), as three signed base-2^16 digits held as FP32 values.  One FMA per digit adds a
-// sign's term; up to CUT_FOLD edges the digit sums stay below 2^24, where FP32 holds every
-// integer, and are then folded into a 64-bit integer: the vertex's sum is exact, and the
-// only rounding is that of the weights, 2^-47 of the largest.  Relative error of the cuts
-// against FP64 (exact summation), largest over 8 solves: 12,000 SNPs 3.8e-16, 3,000 SNPs
-// 3.8e-16 (compensated FP32 sums, which this replaces: 4.8e-15 and 9.6e-15).
+// Real weights over many replicas: the same per-vertex sums in fixed point, scaled row by
+// row.  A weight is the integer W = rn(w 2^ex), |W| <= 2^bits, with the power of two from the
+// row's own largest |w|: blocks and rows of unlike weights each keep their bits (one scale
+// for the whole graph held a block of weights 1e-8 of the largest to 1.3e-7).  bits is 53,
+// the whole significand of the row's largest weight, up to 512 edges; a longer row gives up
+// the bits that its sum needs in 64 (49 at 8,192 edges).  So a row's sum is off by at most
+// 2^-bits max|w| an edge, whatever else the graph holds.
+// W is three signed base-2^18 digits held as FP32 values.  One FMA per digit adds a sign's
+// term; up to CUT_FOLD edges the digit sums stay below 2^24, where FP32 holds every integer,
+// and are then folded into a 64-bit integer: the sum of the W is exact.
 // Warp per vertex, 32 edges at a time: each lane turns one weight into digits (shared
-// memory) and holds its column; a lane owns PER replicas, their signs one byte each.  us
-// per call, compensated FP32 -> now: 12,000 SNPs (5.6M entries), R = 512: 2,163 -> 815;
-// 50,000 SNPs (7.6M entries), R = 128: 1,190 -> 558.  Six base-256 digits with a DP4A
-// per four edges measured 1,127 and 624: this part's DP4A rate is low.
+// memory) and holds its column; a lane owns PER replicas, their signs one byte each.
+// Relative error of the cuts against extended precision, compensated FP32 (before fixed
+// point) / one 46-bit scale / now: 12,000 SNPs 5.4e-15 / 4.0e-16 / 2.5e-16; 200 SNPs 5.1e-15 /
+// 2.5e-16 / 4.5e-16; a block of weights 1e-8 of the other block's 4.7e-16 / 3.3e-7 / 6.7e-16.  A
+// solve's time outside its steps, ms: 12,000 SNPs (5.6M entries) R = 512: 2.64 / 1.29 / 1.27;
+// 50,000 SNPs (7.6M entries) R = 128: 3.08 / 1.58 / 1.56.  Six base-256 digits with a DP4A per
+// four edges measured slower: this part's DP4A rate is low.
 constexpr int CUT_DIGITS = 3;
-constexpr int CUT_BITS = 46;
-constexpr int CUT_FOLD = 256;
+constexpr int CUT_DIGIT_BITS = 18;
+constexpr int CUT_BITS = 53;
+constexpr int CUT_FOLD = 64;
+static_assert(CUT_FOLD << (CUT_DIGIT_BITS - 1) < 1 << 24, "exact digit sums in FP32");
+static_assert(CUT_DIGITS * CUT_DIGIT_BITS > CUT_BITS, "the digits hold a weight");
 
 template <int PER, bool VEC>
 __global__ void __launch_bounds__(256) k_cut_nodes_fx(
     int32_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
     const double* __restrict__ w, const int32_t* __restrict__ block_of,
-    const int32_t* __restrict__ pad_index, const int8_t* __restrict__ st, int32_t R, double scale,
-    double inv_scale, double* node_val, const int32_t* __restrict__ active) {
+    const int32_t* __restrict__ pad_index, const int8_t* __restrict__ st, int32_t R,
+    double* node_val, const int32_t* __restrict__ active) {
   static_assert(PER == 4 || PER == 8, "one or two sign words per lane");
   constexpr int Q = PER / 4;
   __shared__ __align__(16) float dig_all[256 / 32][CUT_DIGITS][32];
@@ -868,6 +876,19 @@ __global__ void __launch_bounds__(256) k_cut_nodes_fx(
   float(*dig)[32] = dig_all[threadIdx.x >> 5];
   const int32_t pa = pad_index[a];
   const int64_t e0 = rp[a], e1 = rp[a + 1];
+  // the row's scale, from the exponent of its largest |w| (taken as 2^-900 below that, so that
+  // both factors are normal)
+  double scale, inv_scale;
+  {
+    uint32_t top = 0;
+    for (int64_t e = e0 + lane; e < e1; e += 32)
+      top = max(top, (uint32_t)__double2hiint(w[e]) & 0x7fffffffu);
+    const int ew = max((int)(__reduce_max_sync(0xffffffffu, top) >> 20), 123);
+    const int lg = 64 - __clzll(max(e1 - e0, (int64_t)1) - 1);  // the row's edges <= 2^lg
+    const int ex = min(CUT_BITS, 62 - lg) - 1 - (ew - 1023);
+    scale = __hiloint2double((1023 + ex) << 20, 0);
+    inv_scale = __hiloint2double((1023 - ex) << 20, 0);
+  }
   for (int32_t r0 = 0; r0 < R; r0 += 32 * PER) {
     const int32_t r = r0 + PER * lane;
     // the signs of PER replicas of one vertex, as Q words (bytes past R: +1, unused)
@@ -911,9 +932,11 @@ __global__ void __launch_bounds__(256) k_cut_nodes_fx(
         __syncwarp();  // the group before has been read
 #pragma unroll
         for (int d = 0; d < CUT_DIGITS; ++d) {
-          const int16_t v = (int16_t)(W & 0xffff);
+          const int32_t v = d + 1 < CUT_DIGITS  // the last digit may be 2^17
+                                ? (int32_t)((uint32_t)W << (32 - CUT_DIGIT_BITS)) >> (32 - CUT_DIGIT_BITS)
+                                : (int32_t)W;
           dig[d][lane] = (float)v;
-          W = (W - v) >> 16;
+          W = (W - v) >> CUT_DIGIT_BITS;
         }
         __syncwarp();
         const int ng = (int)(e1 - eg < 32 ? (e1 - eg + 3) / 4 : 8);  // groups of four edges
@@ -956,7 +979,7 @@ __global__ void __launch_bounds__(256) k_cut_nodes_fx(
         long long v = 0;
 #pragma unroll
         for (int d = CUT_DIGITS - 1; d >= 0; --d)
-          v = v * 65536 + __float2int_rn(k & 1 ? acc[k / 2][d].y : acc[k / 2][d].x);
+          v = v * (1 << CUT_DIGIT_BITS) + __float2int_rn(k & 1 ? acc[k / 2][d].y : acc[k / 2][d].x);
         tot[k] += v;
       }
     }
@@ -1586,17 +1609,10 @@ void launch_cut(cudaStream_t s, const Graph& g, int32_t R, const int8_t* signs_t
     k_cut_nodes_few<<<::qh::counted(grid), 256, 0, s>>>(
         g.n_nodes, g.row_ptr, g.col, w, g.block_of, g.pad_index, signs_t, R, node_val, active);
   } else {
-    // |w| scale < 2^bits, and a row of the largest block stays below 2^62
-    int bits = CUT_BITS, lg = 0;
-    while ((1 << lg) < max_n && lg < 30) ++lg;
-    bits = std::min(bits, 62 - lg);
-    const int ex = bits - 1 - std::ilogb(m);
-    const double sc = std::ldexp(1.0, ex), inv = std::ldexp(1.0, -ex);
 #define QH_CUT_FX(PER, VEC)                                                                    \
   k_cut_nodes_fx<PER, VEC><<<::qh::counted(warps), 256, 0, s>>>(g.n_nodes, g.row_ptr, g.col, w, \
                                                                 g.block_of, g.pad_index,       \
-                                                                signs_t, R, sc, inv, node_val, \
-                                                                active)
+                                                                signs_t, R, node_val, active)
     // eight replicas a lane when they fill the warp
     if (R % 8 == 0 && R >= 256)
       QH_CUT_FX(8, true);
