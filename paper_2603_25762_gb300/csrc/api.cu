@@ -183,19 +183,24 @@ qh_status check_err_word(Ctx* ctx) {
 
 // Time every valid step-kernel variant on the live state for a few steps and keep
 // the fastest for this graph shape (the multi-step family first, below).  The state is re-initialised afterwards.
-std::string tune_key(const Graph& g, int R, int use_lo, int sb) {
+// All of what the choice hangs on is in the key: BF16 and BF16X2 solves of one graph walk
+// different entries, and some c0 rule the multi-step kernels out.
+std::string tune_key(const Graph& g, int R, int use_lo, int sb, bool allow_run) {
   char kb[160];
-  snprintf(kb, sizeof kb, "%d|%d|%lld|%d|%d|%d|%d", R, g.n_row_tiles, (long long)g.n_tiles,
-           g.max_tiles_per_row, g.n_pad, use_lo, sb);
+  snprintf(kb, sizeof kb, "%d|%d|%lld|%d|%d|%d|%d|%d", R, g.n_row_tiles, (long long)g.n_tiles,
+           g.max_tiles_per_row, g.n_pad, use_lo, sb, allow_run ? 1 : 0);
   return kb;
 }
 
-
-bool tuned_variant(Ctx* ctx, const Graph& g, int R, int sb, TcPlan* plan) {
-  const std::string kb = tune_key(g, R, 0, sb);
-  for (auto& kv : ctx->tuned)
-    if (kv.first == kb) {
-      plan->variant = kv.second;
+// The kept choice for this shape.  Two graphs of one key may still differ (in which of their
+// entries are remainders), so the choice must fit this one.
+bool tuned_variant(Ctx* ctx, const Graph& g, int R, int use_lo, int sb, bool allow_run,
+                   TcPlan* plan) {
+  const std::string kb = tune_key(g, R, use_lo, sb, allow_run);
+  for (auto kv = ctx->tuned.rbegin(); kv != ctx->tuned.rend(); ++kv)
+    if (kv->first == kb) {
+      if (!tc_variant_ok(kv->second, g, R, ctx->n_sm, use_lo != 0)) return false;
+      plan->variant = kv->second;
       return true;
     }
   return false;
@@ -213,7 +218,7 @@ bool run_c0_ok(const float* c0, int32_t nb, float dt) {
 
 qh_status autotune(Ctx* ctx, const Graph& g, StepArgs a, const SolveBufs& B, int R, TcPlan* plan,
                    bool allow_run) {
-  const std::string kb = tune_key(g, R, 0, a.sb);
+  const std::string kb = tune_key(g, R, a.use_lo, a.sb, allow_run);
   cudaStream_t s = ctx->stream;
   // The per-step and the multi-step kernels round y differently, so which family runs must
   // not hang on a close race: a per-step kernel is taken only where it is FAMILY_EDGE times
@@ -872,12 +877,14 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
     if (o->step_kernel >= 0 && !G.csr_mode) {
       tplan.variant = o->step_kernel;
     } else if (!G.csr_mode) {
-      if (!tuned_variant(ctx, G, R, o->sb_variant, &tplan)) {  // first solve of this shape: time the variants
+      const bool allow_run = run_c0_ok(h_c0.data(), nb, a.dt);
+      if (!tuned_variant(ctx, G, R, a.use_lo, o->sb_variant, allow_run, &tplan)) {
+        // first solve of this shape: time the variants
         QH_CUDA_TRY(cudaMemcpyAsync(B.running, B.active, nb * 4, cudaMemcpyDeviceToDevice, s));
         launch_init_state(s, W, R, o->replica_base, o->seed, 0, B.x, B.y, B.xh0, B.active,
                           o->sb_variant);
         QH_STAGE_CHECK("solve: state init (tuning)");
-        st = autotune(ctx, W, a, B, R, &tplan, run_c0_ok(h_c0.data(), nb, a.dt));
+        st = autotune(ctx, W, a, B, R, &tplan, allow_run);
       }
     }
     if (st != QH_OK) return st;

@@ -1222,6 +1222,7 @@ bool run_plan(const Graph& g, int R, int n_sm, int variant, bool use_lo, RunPlan
     if (load(b) > cap) return false;
     total += load(b);
   }
+  if (plan == nullptr) return true;
   const int64_t n_waves = (total + cap - 1) / cap;
   const int64_t target = (total + n_waves - 1) / n_waves;
   RunPlan p;
@@ -1315,7 +1316,7 @@ bool run_plan(const Graph& g, int R, int n_sm, int variant, bool use_lo, RunPlan
       for (int32_t r = first[b]; r < first[b] + count[b]; ++r) rows.push_back(r);
     emit(rows);
   }
-  if (plan) *plan = std::move(p);
+  *plan = std::move(p);
   return true;
 }
 
