@@ -79,8 +79,11 @@ __global__ void k_cov_fill(int32_t m, const int64_t* __restrict__ fp, const int3
 
 // Sort each SNP's covering list by fragment index, each entry with its allele or (cov_pos
 // != nullptr) its position.  Warp per SNP: lists of up to 256 entries are sorted in the
-// warp's shared-memory slice (bitonic, keys fragment << 32 | payload); longer ones (rare)
-// by lane 0 in place.
+// warp's shared-memory slice (bitonic, keys fragment << 32 | payload); longer ones (deep
+// coverage) in place, by the same network over any length: every comparison ascends (the
+// first of a merge against the mirrored half), so a partner past the end, taken as
+// infinite, never moves.  An insertion sort by one lane took most of a deep graph build: 50
+// SNPs under 5,000 reads 189 ms with the alleles alone, 293 with the positions, 11.6 now.
 constexpr int COV_SORT_MAX = 256;
 
 __global__ void __launch_bounds__(256) k_cov_sort(int32_t n, const int64_t* __restrict__ cov_ptr,
@@ -128,25 +131,32 @@ __global__ void __launch_bounds__(256) k_cov_sort(int32_t n, const int64_t* __re
     }
     return;
   }
-  if (lane != 0) return;
-  for (int64_t i = b + 1; i < e; ++i) {
-    const int32_t f = cov_frag[i];
-    const int32_t v = cov_pos != nullptr ? cov_pos[i] : cov_allele[i];
-    int64_t j = i - 1;
-    while (j >= b && cov_frag[j] > f) {
-      cov_frag[j + 1] = cov_frag[j];
-      if (cov_pos != nullptr)
-        cov_pos[j + 1] = cov_pos[j];
-      else
-        cov_allele[j + 1] = cov_allele[j];
-      --j;
+  auto exchange = [&](int32_t i, int32_t l) {
+    const int32_t fi = cov_frag[b + i], fl = cov_frag[b + l];
+    if (fi <= fl) return;
+    cov_frag[b + i] = fl;
+    cov_frag[b + l] = fi;
+    if (cov_pos != nullptr) {
+      const int32_t v = cov_pos[b + i];
+      cov_pos[b + i] = cov_pos[b + l];
+      cov_pos[b + l] = v;
+    } else {
+      const int8_t v = cov_allele[b + i];
+      cov_allele[b + i] = cov_allele[b + l];
+      cov_allele[b + l] = v;
     }
-    cov_frag[j + 1] = f;
-    if (cov_pos != nullptr)
-      cov_pos[j + 1] = v;
-    else
-      cov_allele[j + 1] = (int8_t)v;
-  }
+  };
+  for (int64_t k = 2; k < 2 * (int64_t)len; k <<= 1)
+    for (int64_t j = k >> 1; j > 0; j >>= 1) {
+      // pair t: i in the lower half of its group of 2 j, l its mirror (first) or i + j
+      for (int64_t t = lane;; t += 32) {
+        const int64_t i = 2 * (t & ~(j - 1)) + (t & (j - 1));
+        if (i >= len) break;
+        const int64_t l = 2 * j == k ? (i & ~(k - 1)) + (k - 1 - (i & (k - 1))) : i + j;
+        if (l < len) exchange((int32_t)i, (int32_t)l);
+      }
+      __syncwarp();
+    }
 }
 
 // ------------------------------------------------------------------ read graph
@@ -339,8 +349,12 @@ struct SnpRowSmem {
 //  * Partners within SNP_NEAR / 2 of u sum into a dense window in shared memory.  The
 //    others (long-range contacts) go into a list of SNP_FAR terms, sorted by (partner,
 //    fragment) at the end; a partner is always on one side of that line.
-//  * A row with more far terms, or with more terms than the CTA kernel's sort path takes
-//    (which alone says whether its window is small enough), is deferred to the CTA kernel.
+//  * A row with more far terms is deferred to the CTA kernel, in PASS 0 as soon as it shows;
+//    so is one with more terms than that kernel's sort path takes (SNP_ROW_CAP) in a window
+//    wider than its dense path's (SNP_DENSE_CAP), which it refuses.  PASS 0 marks them in
+//    `late` for PASS 1.  Rows of more than SNP_ROW_CAP terms were once all deferred; graph
+//    builds of ONT-like reads at 100x, a CTA per row with a search / that / now: 600 SNPs
+//    1.26 / 2.35 / 1.14 ms, 3,000 SNPs 2.77 / 8.36 / 1.81, 12,000 SNPs 8.29 / 29.6 / 4.07.
 // Bound by FP64 and by the latency of the terms' loads.  GB300's FP64 rate makes a division
 // per term the largest cost of the fill: the divisor is a fragment's, so the quotient is
 // taken from its correctly rounded reciprocal (snp_quotient, the same bits).  Measured,
@@ -378,7 +392,7 @@ __global__ void __launch_bounds__(32 * SNP_WARPS) k_snp_rows_warp(
     const uint8_t* __restrict__ is_porec, const int64_t* __restrict__ cov_ptr,
     const int32_t* __restrict__ cov_frag, const int32_t* __restrict__ cov_pos,
     const double* __restrict__ L, double alpha, int linkage_k, int64_t* cnt,
-    const int64_t* __restrict__ row_ptr, int32_t* col, double* w, int32_t* defer,
+    const int64_t* __restrict__ row_ptr, int32_t* col, double* w, uint8_t* late, int32_t* defer,
     int32_t* n_defer) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SnpWarpSmem& sm = reinterpret_cast<SnpWarpSmem*>(smem_raw)[threadIdx.x >> 5];
@@ -386,6 +400,7 @@ __global__ void __launch_bounds__(32 * SNP_WARPS) k_snp_rows_warp(
   const int64_t u64 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   if (u64 >= n) return;
   const int32_t u = (int32_t)u64;
+  if (PASS == 1 && late[u]) return;
   const bool plain = !(alpha == 0.0 || (alpha >= 1e-200 && alpha <= 1e200));
   for (int t = lane; t < SNP_NEAR; t += 32) {
     if (PASS == 1) sm.acc[t] = 0.0;
@@ -396,7 +411,7 @@ __global__ void __launch_bounds__(32 * SNP_WARPS) k_snp_rows_warp(
   const int32_t near0 = u - SNP_NEAR / 2;
   int32_t n_far = 0;
   int64_t terms = 0;
-  for (int64_t c0 = cb; c0 < ce; c0 += 32) {
+  for (int64_t c0 = cb; c0 < ce && n_far <= SNP_FAR; c0 += 32) {
     const int cn = (int)(ce - c0 < 32 ? ce - c0 : 32);
     // lane c: covering fragment c0 + c
     int64_t fb = 0;
@@ -467,11 +482,27 @@ __global__ void __launch_bounds__(32 * SNP_WARPS) k_snp_rows_warp(
       __syncwarp();  // the next fragment's terms go on top of this one's
     }
   }
+  if (PASS == 0) {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) terms += __shfl_xor_sync(0xffffffffu, terms, off);
-  if (n_far > SNP_FAR || terms > SNP_ROW_CAP) {  // the CTA kernel's row
-    if (PASS == 0 && lane == 0) defer[atomicAdd(n_defer, 1)] = u;
-    return;
+    for (int off = 16; off > 0; off >>= 1) terms += __shfl_xor_sync(0xffffffffu, terms, off);
+    bool wide = false;
+    if (n_far <= SNP_FAR && terms > SNP_ROW_CAP) {
+      int32_t w0 = INT32_MAX, w1 = -1;
+      for (int64_t c = cb + lane; c < ce; c += 32) {
+        const int32_t i = cov_frag[c];
+        w0 = min(w0, snp[fp[i]]);
+        w1 = max(w1, snp[fp[i + 1] - 1]);
+      }
+      w0 = __reduce_min_sync(0xffffffffu, w0);
+      w1 = __reduce_max_sync(0xffffffffu, w1);
+      wide = w1 - w0 + 1 > SNP_DENSE_CAP;
+    }
+    const bool defers = n_far > SNP_FAR || wide;  // the CTA kernel's row
+    if (lane == 0) {
+      late[u] = defers;
+      if (defers) defer[atomicAdd(n_defer, 1)] = u;
+    }
+    if (defers) return;
   }
   // sort the far terms by (partner, fragment)
   int32_t N = 1;
@@ -1275,13 +1306,15 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
     int32_t* defer = (int32_t*)ctx->scratch(sizeof(int32_t) * (n + 1), 23);
     g->row_ptr = (int64_t*)dalloc(*g, sizeof(int64_t) * (n + 1));
     if (!g->row_ptr || !defer) return set_err(ctx, QH_ENOMEM, "allocation failed (edges)");
+    uint8_t* late = (uint8_t*)ctx->scratch((size_t)n + 1, 29);
+    if (!late) return set_err(ctx, QH_ENOMEM, "allocation failed (edges)");
     int32_t* n_defer = defer + n;
     QH_CUDA_TRY(cudaMemsetAsync(n_defer, 0, sizeof(int32_t), s));
     if (n > 0) {
       k_snp_rows_warp<0><<<::qh::counted(grid_w), 32 * SNP_WARPS, smem_w, s>>>(
           n, g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag,
-          cov_pos, L, o->porec_alpha, o->linkage_k, cnt, nullptr, nullptr, nullptr, defer,
-          n_defer);
+          cov_pos, L, o->porec_alpha, o->linkage_k, cnt, nullptr, nullptr, nullptr, late,
+          defer, n_defer);
       k_snp_rows<0><<<::qh::counted(grid), 512, smem, s>>>(
           g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, L,
           o->porec_alpha, o->linkage_k, cnt, nullptr, nullptr, nullptr, ctx->d_err, defer,
@@ -1299,8 +1332,8 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
     if (n > 0 && g->nnz > 0) {
       k_snp_rows_warp<1><<<::qh::counted(grid_w), 32 * SNP_WARPS, smem_w, s>>>(
           n, g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag,
-          cov_pos, L, o->porec_alpha, o->linkage_k, nullptr, g->row_ptr, g->col, g->w, nullptr,
-          nullptr);
+          cov_pos, L, o->porec_alpha, o->linkage_k, nullptr, g->row_ptr, g->col, g->w, late,
+          nullptr, nullptr);
       k_snp_rows<1><<<::qh::counted(grid), 512, smem, s>>>(
           g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, L,
           o->porec_alpha, o->linkage_k, nullptr, g->row_ptr, g->col, g->w, ctx->d_err, defer,
