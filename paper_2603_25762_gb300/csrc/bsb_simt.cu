@@ -991,27 +991,30 @@ __global__ void __launch_bounds__(256) k_cut_nodes_fx(
   }
 }
 
-// CTA per (32 replicas, CUT_ROWS vertices, block): 32 vertex slices per replica summed in
-// a fixed order, then the 32 slice sums in order.  A block of one chunk gets its cuts =
-// (sum_w - s^T W s) / 4 here; a larger one leaves the chunk's sum in the chunk's first row
-// of node_val (read by this CTA alone, before the barrier) for k_cut_chunks.  One CTA per
-// 32 replicas walked all vertices before: 469 us for 50,000 vertices at R = 128, 44 us
-// now with k_cut_chunks.
-constexpr int CUT_ROWS = 512;
-
-__global__ void __launch_bounds__(1024) k_cut_reduce(const int32_t* __restrict__ pad_off,
+// CTA per (32 replicas, CUT_ROWS vertices of a block: Graph::cut_rt): 32 vertex slices per
+// replica summed in a fixed order, then the 32 slice sums in order.  A block of one chunk
+// gets its cuts = (sum_w - s^T W s) / 4 here; a larger one leaves the chunk's sum in the
+// chunk's first row of node_val (read by this CTA alone, before the barrier) for
+// k_cut_chunks.  One CTA per 32 replicas walked all vertices before: 469 us for 50,000
+// vertices at R = 128, 44 us now with k_cut_chunks.  A grid of blocks x the largest block's
+// chunks was mostly empty CTAs beside one large block: a solve of two steps on 100,000
+// vertices and 20,000 small blocks, R = 128, took 34.4 ms, 8.0 now.
+__global__ void __launch_bounds__(1024) k_cut_reduce(const RowTile* __restrict__ rts,
+                                                     const int32_t* __restrict__ cut_rt,
+                                                     const int32_t* __restrict__ pad_off,
                                                      const int64_t* __restrict__ block_ptr, int32_t R,
                                                      double* node_val,
                                                      const double* __restrict__ sum_w, double* cuts,
                                                      const int32_t* __restrict__ active) {
   __shared__ double part[32][33];
-  const int32_t b = blockIdx.z;
+  const int32_t groups = (R + 31) / 32;
+  const RowTile rt = rts[cut_rt[blockIdx.x / groups]];
+  const int32_t b = rt.block;
   if (active != nullptr && !active[b]) return;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int32_t r = blockIdx.x * 32 + tx;
+  const int32_t r = (int32_t)(blockIdx.x % groups) * 32 + tx;
   const int32_t sz = (int32_t)(block_ptr[b + 1] - block_ptr[b]);
-  const int32_t c0 = blockIdx.y * CUT_ROWS, c1 = min(sz, c0 + CUT_ROWS);
-  if (c0 >= sz) return;
+  const int32_t c0 = rt.row0 - pad_off[b], c1 = min(sz, c0 + CUT_ROWS);
   double* nv = node_val + (size_t)pad_off[b] * R;
   double s = 0.0;
   if (r < R)
@@ -1622,9 +1625,8 @@ void launch_cut(cudaStream_t s, const Graph& g, int32_t R, const int8_t* signs_t
       QH_CUT_FX(4, false);
 #undef QH_CUT_FX
   }
-  const dim3 grid((R + 31) / 32, (max_n + CUT_ROWS - 1) / CUT_ROWS, g.n_blocks);
-  k_cut_reduce<<<::qh::counted(grid), 1024, 0, s>>>(g.pad_off, g.block_ptr, R, node_val, sum_w,
-                                                    cuts, active);
+  k_cut_reduce<<<::qh::counted((unsigned)g.n_cut_chunks * (unsigned)((R + 31) / 32)), 1024, 0, s>>>(
+      g.rt, g.cut_rt, g.pad_off, g.block_ptr, R, node_val, sum_w, cuts, active);
   if (max_n > CUT_ROWS)
     k_cut_chunks<<<::qh::counted(nblk((int64_t)g.n_blocks * R)), 256, 0, s>>>(
         g.n_blocks, g.pad_off, g.block_ptr, R, node_val, sum_w, cuts, active);

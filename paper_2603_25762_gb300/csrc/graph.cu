@@ -1495,12 +1495,14 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
   std::vector<int32_t> h_rt_of_block(std::max(nb, 1), 0);
   std::vector<int32_t> h_tile_col;
   std::vector<KSlice> h_kslice;
+  std::vector<int32_t> h_cut_rt;
   int64_t entry = 0;
   for (int32_t b = 0; b < nb; ++b) {
     h_rt_of_block[b] = (int32_t)g->h_rt.size();
     int32_t T = h_T[b];
     for (int32_t r = 0; r < T; ++r) {
       int64_t s0 = h_slot_off[b] + (int64_t)r * T;
+      if (r % (CUT_ROWS / TILE) == 0) h_cut_rt.push_back((int32_t)g->h_rt.size());
       RowTile rt;
       rt.block = b;
       rt.row0 = g->h_pad_off[b] + r * TILE;
@@ -1541,10 +1543,12 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
   g->tile_bf16 = (__nv_bfloat16*)dalloc(*g, sizeof(__nv_bfloat16) * TILE * TILE * std::max<int64_t>(g->n_tiles, 1));
   g->tile_f32 = (float*)dalloc(*g, sizeof(float) * TILE * TILE * std::max<int64_t>(g->n_tiles_hi, 1));
   g->rt_of_block = (int32_t*)dalloc(*g, sizeof(int32_t) * std::max(nb, 1));
+  g->n_cut_chunks = (int32_t)h_cut_rt.size();
+  g->cut_rt = (int32_t*)dalloc(*g, sizeof(int32_t) * std::max(g->n_cut_chunks, 1));
   g->slot_off = (int64_t*)dalloc(*g, sizeof(int64_t) * (nb + 1));
   g->tiles_per_block = (int32_t*)dalloc(*g, sizeof(int32_t) * std::max(nb, 1));
   g->slot_tile = (int64_t*)dalloc(*g, sizeof(int64_t) * (n_slots + 1));
-  if (!g->rt || !g->tile_col || !g->kslice || !g->tile_bf16 || !g->tile_f32 || !g->rt_of_block || !g->slot_off ||
+  if (!g->rt || !g->tile_col || !g->kslice || !g->tile_bf16 || !g->tile_f32 || !g->rt_of_block || !g->cut_rt || !g->slot_off ||
       !g->tiles_per_block || !g->slot_tile)
     return set_err(ctx, QH_ENOMEM, "allocation failed (tiles)");
   if (g->n_row_tiles > 0)
@@ -1552,6 +1556,9 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
                                 cudaMemcpyHostToDevice, s));
   if (g->n_tiles > 0)
     QH_CUDA_TRY(cudaMemcpyAsync(g->tile_col, h_tile_col.data(), sizeof(int32_t) * g->n_tiles,
+                                cudaMemcpyHostToDevice, s));
+  if (g->n_cut_chunks > 0)
+    QH_CUDA_TRY(cudaMemcpyAsync(g->cut_rt, h_cut_rt.data(), sizeof(int32_t) * g->n_cut_chunks,
                                 cudaMemcpyHostToDevice, s));
   if (!h_kslice.empty())
     QH_CUDA_TRY(cudaMemcpyAsync(g->kslice, h_kslice.data(), sizeof(KSlice) * h_kslice.size(),

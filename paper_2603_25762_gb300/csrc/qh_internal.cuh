@@ -38,6 +38,8 @@ enum : int32_t {
   ERR_CONFIG = 16,      // a kernel refused the launch's arguments (host-side slip)
 };
 
+constexpr int CUT_ROWS = 512;  // vertices of a block that one CTA of the cut reduction sums
+
 struct RowTile {           // one 128-row slab of a block in the padded layout
   int32_t block;           // phase block
   int32_t row0;            // first padded row (multiple of 128)
@@ -118,6 +120,8 @@ struct Graph {
   int32_t max_tiles_per_row = 0;  // largest n_all over row tiles
   RowTile* rt = nullptr;          // [n_row_tiles]
   int32_t* rt_of_block = nullptr; // [n_blocks] first row tile of the block
+  int32_t* cut_rt = nullptr;      // [n_cut_chunks] first row tile of every CUT_ROWS rows of a
+  int32_t n_cut_chunks = 0;       // block
   int32_t* tile_col = nullptr;    // [n_tiles] column tile (padded col / 128)
   KSlice* kslice = nullptr;       // per row tile: its K-slices that hold a nonzero
   int64_t* slot_off = nullptr;    // [n_blocks+1] tile-slot offsets (T_b^2 slots per block)
