@@ -567,21 +567,31 @@ __global__ void __launch_bounds__(32 * SNP_WARPS) k_snp_rows_warp(
   if (PASS == 0 && lane == 0) cnt[u] = total;
 }
 
-// The rows k_snp_rows_warp deferred (`rows`, *n_list of them), a CTA each.  PASS 0: count
-// distinct partners; PASS 1: write (v, w_uv).  A row whose covered window is at most
-// SNP_DENSE_CAP sums into a dense window; otherwise its fragment terms are gathered and
-// sorted by (partner, fragment), at most SNP_ROW_CAP of them.  Both sum a partner's terms
-// in fragment order.
-template <int PASS>
-__global__ void __launch_bounds__(512) k_snp_rows(
+// The rows k_snp_rows_warp deferred, a CTA each (`rows`, *n_list of them).  PASS 0: count
+// distinct partners; PASS 1: write (v, w_uv).  A row whose covered window is at most DCAP
+// SNPs sums into a dense window; otherwise its fragment terms are gathered and sorted by
+// (partner, fragment), at most TCAP of them.  Both sum a partner's terms in fragment order.
+// SMALL: SNP_SMALL_CAP of either in 32 KB of shared memory, so that seven CTAs share an SM;
+// a row over both goes to `defer` (PASS 0) and is the large kernel's, with SNP_DENSE_CAP
+// and SNP_ROW_CAP.  Without the small tier rows of many long-range contacts took turns in
+// one CTA per SM.  Graph build, ms, small tier for all rows / large tier alone / now: 8,000
+// SNPs with 200,000 contacts 1.81 / 9.5 / 1.98, 2,000 with 200,000 3.84 / 13.2 / 3.12 (what is
+// left over the first at 8,000 is the warp's count of the row up to its 257th far term).
+constexpr int SNP_SMALL_CAP = 2048;
+constexpr size_t SNP_SMALL_SMEM = (size_t)SNP_SMALL_CAP * 16;
+
+template <int PASS, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? 256 : 512) k_snp_rows(
     const int64_t* __restrict__ fp, const int32_t* __restrict__ snp,
     const int8_t* __restrict__ allele, const uint8_t* __restrict__ qual,
     const uint8_t* __restrict__ is_porec, const int64_t* __restrict__ cov_ptr,
-    const int32_t* __restrict__ cov_frag, const double* __restrict__ L, double alpha,
-    int linkage_k, int64_t* cnt, const int64_t* __restrict__ row_ptr, int32_t* col, double* w,
-    int32_t* err, const int32_t* __restrict__ rows, const int32_t* __restrict__ n_list) {
-  constexpr int DCAP = SNP_DENSE_CAP;
-  constexpr int TCAP = SNP_ROW_CAP;
+    const int32_t* __restrict__ cov_frag, const int32_t* __restrict__ cov_pos,
+    const double* __restrict__ L, double alpha, int linkage_k, int64_t* cnt,
+    const int64_t* __restrict__ row_ptr, int32_t* col, double* w, int32_t* err,
+    const int32_t* __restrict__ rows, const int32_t* __restrict__ n_list, int32_t* defer,
+    int32_t* n_defer) {
+  constexpr int DCAP = SMALL ? SNP_SMALL_CAP : SNP_DENSE_CAP;
+  constexpr int TCAP = SMALL ? SNP_SMALL_CAP : SNP_ROW_CAP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int32_t s_total;
   __shared__ int32_t s_runs[32];
@@ -631,12 +641,7 @@ __global__ void __launch_bounds__(512) k_snp_rows(
         const int64_t fb = fp[i], fe = fp[i + 1];
         const int32_t S = (int32_t)(fe - fb);
         const int32_t depth = (int32_t)(((int64_t)linkage_k * (S - 1)) / 10);
-        int64_t l = fb, h = fe;
-        while (l < h) {
-          int64_t mid = (l + h) >> 1;
-          if (snp[mid] < u) l = mid + 1; else h = mid;
-        }
-        const int32_t p = (int32_t)(l - fb);
+        const int32_t p = cov_pos[cb + c];
         const int32_t lo = max(0, p - depth), hi = min(S - 1, p + depth);
         const int64_t eu = fb + p;
         const double a = (is_porec != nullptr && is_porec[i]) ? alpha : 1.0;
@@ -694,13 +699,7 @@ __global__ void __launch_bounds__(512) k_snp_rows(
         int64_t fb = fp[i], fe = fp[i + 1];
         int32_t S = (int32_t)(fe - fb);
         int32_t depth = (int32_t)(((int64_t)linkage_k * (S - 1)) / 10);
-        // position of u inside fragment i (binary search, SNPs ascending)
-        int64_t l = fb, h = fe;
-        while (l < h) {
-          int64_t mid = (l + h) >> 1;
-          if (snp[mid] < u) l = mid + 1; else h = mid;
-        }
-        int32_t p = (int32_t)(l - fb);
+        int32_t p = cov_pos[cb + c0 + c];  // u inside fragment i
         int32_t lo = max(0, p - depth), hi = min(S - 1, p + depth);
         s_off[c + 1] = hi - lo;  // partners (window minus u itself)
       }
@@ -711,8 +710,8 @@ __global__ void __launch_bounds__(512) k_snp_rows(
       }
       __syncthreads();
       int32_t tot = s_off[cn];
-      if (base + tot > TCAP) {
-        if (threadIdx.x == 0) atomicOr(err, ERR_ROWCAP);
+      if (base + tot > TCAP) {  // small kernel: the large kernel's row; large: error
+        if (!SMALL && threadIdx.x == 0) atomicOr(err, ERR_ROWCAP);
         base = TCAP + 1;
         __syncthreads();
         break;
@@ -729,12 +728,7 @@ __global__ void __launch_bounds__(512) k_snp_rows(
         int64_t fb = fp[i], fe = fp[i + 1];
         int32_t S = (int32_t)(fe - fb);
         int32_t depth = (int32_t)(((int64_t)linkage_k * (S - 1)) / 10);
-        int64_t l = fb, h = fe;
-        while (l < h) {
-          int64_t mid = (l + h) >> 1;
-          if (snp[mid] < u) l = mid + 1; else h = mid;
-        }
-        int32_t p = (int32_t)(l - fb);
+        int32_t p = cov_pos[cb + c0 + c];
         int32_t wlo = max(0, p - depth);
         int32_t pp = wlo + k;
         if (pp >= p) ++pp;  // skip u itself
@@ -751,7 +745,12 @@ __global__ void __launch_bounds__(512) k_snp_rows(
       __syncthreads();
     }
     if (base > TCAP) {
-      if (PASS == 0 && threadIdx.x == 0) cnt[u] = 0;
+      if (PASS == 0 && threadIdx.x == 0) {
+        if (SMALL)
+          defer[atomicAdd(n_defer, 1)] = u;
+        else
+          cnt[u] = 0;
+      }
       __syncthreads();
       continue;
     }
@@ -1299,26 +1298,36 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
     const size_t smem_w = sizeof(SnpWarpSmem) * SNP_WARPS;
     QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows_warp<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w));
     QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows_warp<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w));
-    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SNP_SMALL_SMEM));
+    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SNP_SMALL_SMEM));
+    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QH_CUDA_TRY(cudaFuncSetAttribute(k_snp_rows<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const unsigned grid = (unsigned)std::max(1, std::min(n, ctx->n_sm));
+    const unsigned grid_s = (unsigned)std::max(1, std::min(n, ctx->n_sm * 16));  // for balance
     const unsigned grid_w = (unsigned)((n + SNP_WARPS - 1) / SNP_WARPS);
     int32_t* defer = (int32_t*)ctx->scratch(sizeof(int32_t) * (n + 1), 23);
     g->row_ptr = (int64_t*)dalloc(*g, sizeof(int64_t) * (n + 1));
     if (!g->row_ptr || !defer) return set_err(ctx, QH_ENOMEM, "allocation failed (edges)");
     uint8_t* late = (uint8_t*)ctx->scratch((size_t)n + 1, 29);
-    if (!late) return set_err(ctx, QH_ENOMEM, "allocation failed (edges)");
+    int32_t* defer2 = (int32_t*)ctx->scratch(sizeof(int32_t) * (n + 1), 30);
+    if (!late || !defer2) return set_err(ctx, QH_ENOMEM, "allocation failed (edges)");
     int32_t* n_defer = defer + n;
+    int32_t* n_defer2 = defer2 + n;
     QH_CUDA_TRY(cudaMemsetAsync(n_defer, 0, sizeof(int32_t), s));
+    QH_CUDA_TRY(cudaMemsetAsync(n_defer2, 0, sizeof(int32_t), s));
     if (n > 0) {
       k_snp_rows_warp<0><<<::qh::counted(grid_w), 32 * SNP_WARPS, smem_w, s>>>(
           n, g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag,
           cov_pos, L, o->porec_alpha, o->linkage_k, cnt, nullptr, nullptr, nullptr, late,
           defer, n_defer);
-      k_snp_rows<0><<<::qh::counted(grid), 512, smem, s>>>(
-          g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, L,
-          o->porec_alpha, o->linkage_k, cnt, nullptr, nullptr, nullptr, ctx->d_err, defer,
-          n_defer);
+      k_snp_rows<0, true><<<::qh::counted(grid_s), 256, SNP_SMALL_SMEM, s>>>(
+          g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, cov_pos, L,
+          o->porec_alpha, o->linkage_k, cnt, nullptr, nullptr, nullptr, ctx->d_err, defer, n_defer,
+          defer2, n_defer2);
+      k_snp_rows<0, false><<<::qh::counted(grid), 512, smem, s>>>(
+          g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, cov_pos, L,
+          o->porec_alpha, o->linkage_k, cnt, nullptr, nullptr, nullptr, ctx->d_err, defer2,
+          n_defer2, nullptr, nullptr);
     }
     if (!scan_i64(ctx, s, cnt, g->row_ptr, n)) return set_err(ctx, QH_ENOMEM, "allocation failed (scan)");
     QH_CUDA_TRY(cudaMemcpyAsync(&g->nnz, g->row_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
@@ -1334,10 +1343,14 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
           n, g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag,
           cov_pos, L, o->porec_alpha, o->linkage_k, nullptr, g->row_ptr, g->col, g->w, late,
           nullptr, nullptr);
-      k_snp_rows<1><<<::qh::counted(grid), 512, smem, s>>>(
-          g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, L,
+      k_snp_rows<1, true><<<::qh::counted(grid_s), 256, SNP_SMALL_SMEM, s>>>(
+          g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, cov_pos, L,
           o->porec_alpha, o->linkage_k, nullptr, g->row_ptr, g->col, g->w, ctx->d_err, defer,
-          n_defer);
+          n_defer, nullptr, nullptr);
+      k_snp_rows<1, false><<<::qh::counted(grid), 512, smem, s>>>(
+          g->frag_ptr, g->snp, g->allele, g->qual, g->is_porec, g->cov_ptr, g->cov_frag, cov_pos, L,
+          o->porec_alpha, o->linkage_k, nullptr, g->row_ptr, g->col, g->w, ctx->d_err, defer2,
+          n_defer2, nullptr, nullptr);
     }
   }
   const int32_t N = g->n_nodes;
