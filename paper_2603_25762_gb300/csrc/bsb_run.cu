@@ -54,6 +54,7 @@
 #include <vector>
 
 #include "qh_internal.cuh"
+#include "ring.cuh"
 #include "tc_ptx.cuh"
 
 namespace qh {
@@ -605,7 +606,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
     // measured slower: its lookup sits in the issuing thread (12,000 SNPs: 18.0).
     if (n_items > 0) {
       const bool lead = lane == 0;
-      uint32_t q = 0;
+      uint32_t q = 0, part = 0;  // part: once the waits gave up, copies issued from use q on
       bool jissued = false;
       if (JRES && lead) {  // all items of the CTA share one row tile
         const ItemInfo& it = info[0];
@@ -685,6 +686,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
                                          a.err, abort_flag);
                 if (lok && lead && kb0 == 0) trace_at(a, u, i, TR_OWN);
                 if (!__all_sync(0xffffffffu, lok)) {
+                  q += (uint32_t)kb0;
                   ok = false;
                   break;
                 }
@@ -705,7 +707,23 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
                               mine ? it.k * RB : ks.jrow());
                 }
               }
-              if (!__all_sync(0xffffffffu, lok)) ok = false;
+              if (__builtin_expect(!__all_sync(0xffffffffu, lok), 0)) {
+                // Given up part-way: lane l's X_hat copy and lane 8 + l's J copy share a slot
+                // and its barrier.  Where one was issued and the other not, the barrier is
+                // set to complete with the one.
+                const bool issued = lok && (mine || minej);
+                const uint32_t got = __ballot_sync(0xffffffffu, issued);
+                q += (uint32_t)kb0;
+                if (!JRES && !jsplit && lane < 16 && !issued && ((got >> (lane ^ 8)) & 1u)) {
+                  const uint32_t bar = full0 + 8 * ((q + (uint32_t)(lane & 7)) % ST);
+                  if (lane < 8)
+                    mbar_expect_tx(bar, SLICE);
+                  else
+                    mbar_complete_tx(bar, SLICE);
+                }
+                part = (got | got >> 8) & 0xffu;
+                ok = false;
+              }
             }
             if (!ok) break;
             q += (uint32_t)it.nk;
@@ -717,8 +735,10 @@ __global__ void __launch_bounds__(RUN_THREADS, 1)
       // copies still in flight must land before the CTA exits: the last load of
       // every ring slot, and the resident J tiles
       if (lead) {
-        for (uint32_t jq = q > (uint32_t)ST ? q - ST : 0u; jq < q; ++jq)
-          mbar_wait(full0 + 8 * (jq % ST), (jq / ST) & 1u, a.err);
+        uint32_t use;
+        for (uint32_t l = 0; l < (uint32_t)ST; ++l)
+          if (ring_last_use(q, part, l, ST, &use))
+            mbar_wait(full0 + 8 * (use % ST), (use / ST) & 1u, a.err);
         if (jissued) mbar_wait(jbar, 0, a.err);
       }
     }
