@@ -234,6 +234,7 @@ __global__ void __launch_bounds__(32 * NW * 8 / TR) k_step_f32(StepArgs a, const
   const bool live = (a.active == nullptr || a.active[rt.block]) && t < sb;
   const int32_t row0 = rt.row0 + grp * F_ROWS;
   if (!live) {
+    cp_async_commit();  // the J copies above belong to no group yet, and the wait is for groups
     cp_async_wait<0>();
     if (a.z_out == nullptr && a.xout != a.xin)  // carry a frozen block to the next buffer
       for (int i = tid; i < RC * F_ROWS; i += NT) {
