@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(32 * NW * 8 / TR) k_step_f32(StepArgs a, const
                     (int64_t)grp * F_TILE_CHUNKS * rt.n_hi;
   // this thread copies quad q (4 of the stage's 32 columns) of some rows and replicas
   const int q = tid % F_QUADS, qr = tid / F_QUADS, c_of = q >> 1, c_in = (q & 1) * 4;
-  const float* const jrow = a.tile_f32 + f32_row_offset(rt.f32_begin) + (grp * F_ROWS) * TILE + c_in;
+  const int64_t row_chunk = f32_row_chunk(rt.f32_begin);
   auto entry = [&](int32_t st) -> int2 {
     const int32_t c = st * F_STAGE_CHUNKS + c_of;
     return c < nc ? lst[c] : make_int2(-1, 0);
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(32 * NW * 8 / TR) k_step_f32(StepArgs a, const
   auto load_j = [&](int32_t st, int2 en) {
     if (en.x < 0) return;
     float* dst = js + (st % F_STAGES) * (F_ROWS * F_KC);
-    const float* src = jrow + f32_chunk_offset(en.x);
+    const float* src = f32_chunk_at(a.tile_f32, row_chunk, en.x) + (grp * F_ROWS) * TILE + c_in;
 #pragma unroll
     for (int i = 0; i < F_ROWS * F_QUADS / NT; ++i) {
       const int row = qr + i * (NT / F_QUADS);

@@ -25,11 +25,15 @@ QH_CHUNK_FN int32_t f32_chunk(int32_t e, int32_t c) {
   return e * (F32_TILE * F32_TILE / F_COLS) + c;
 }
 
-// Offset of row tile f32_begin (its first tile) in the FP32 tiles, in floats, and of a
-// record's first column from there.
-QH_CHUNK_FN int64_t f32_row_offset(int32_t f32_begin) {
-  return (int64_t)f32_begin * (F32_TILE * F32_TILE);
+// The first chunk of a row tile whose first tile is f32_begin, and the address of a record's
+// first column.  The form matters to the compiler: 80 reads at R = 32 / hifi-region at
+// R = 1,024 take 2.09 / 59.4 us a step with this one, 2.13 / 59.1 with a pointer to the row
+// tile, 2.17 / 62.0 with an offset from here added to the tiles' address by the caller.
+QH_CHUNK_FN int64_t f32_row_chunk(int32_t f32_begin) {
+  return (int64_t)f32_begin * (F32_TILE * F32_TILE / F_COLS);
 }
-QH_CHUNK_FN int64_t f32_chunk_offset(int32_t rec) { return (int64_t)rec * F_COLS; }
+QH_CHUNK_FN const float* f32_chunk_at(const float* tiles, int64_t row_chunk, int32_t rec) {
+  return tiles + (row_chunk + rec) * F_COLS;
+}
 
 }  // namespace qh

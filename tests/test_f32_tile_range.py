@@ -23,7 +23,8 @@ int main(void) {
       for (int32_t c = 0; c < 16; ++c) {
         const int32_t rec = qh::f32_chunk(e, c);
         const int64_t want = (b + e) * 16384 + 8 * c;  /* tiles of 128 x 128, chunks of 8 columns */
-        if (rec < 0 || qh::f32_row_offset((int32_t)b) + qh::f32_chunk_offset(rec) != want) ++bad;
+        const float* at = qh::f32_chunk_at((const float*)64, qh::f32_row_chunk((int32_t)b), rec);
+        if (rec < 0 || (int64_t)(uintptr_t)at != 64 + 4 * want) ++bad;
       }
   printf("bad %ld\n", bad);
   return bad != 0;
