@@ -1233,12 +1233,14 @@ qh_status build_graph_device(Ctx* ctx, const qh_fragments* f, const qh_graph_opt
     if (nnz_f > 0) k_cov_count<<<::qh::counted(nblk(nnz_f)), 256, 0, s>>>(nnz_f, g->snp, cnt);
     g->cov_ptr = (int64_t*)dalloc(*g, sizeof(int64_t) * (n + 1));
     g->cov_frag = (int32_t*)dalloc(*g, sizeof(int32_t) * std::max<int64_t>(nnz_f, 1));
-    g->cov_allele = (int8_t*)dalloc(*g, std::max<int64_t>(nnz_f, 1));
-    if (o->mode == QH_MODE_SNP) {
+    if (o->mode == QH_MODE_READ) {
+      g->cov_allele = (int8_t*)dalloc(*g, std::max<int64_t>(nnz_f, 1));
+      if (!g->cov_allele) return set_err(ctx, QH_ENOMEM, "allocation failed (coverage)");
+    } else {
       cov_pos = (int32_t*)ctx->scratch(sizeof(int32_t) * (size_t)std::max<int64_t>(nnz_f, 1), 26);
       if (!cov_pos) return set_err(ctx, QH_ENOMEM, "allocation failed (coverage)");
     }
-    if (!g->cov_ptr || !g->cov_frag || !g->cov_allele) return set_err(ctx, QH_ENOMEM, "allocation failed (coverage)");
+    if (!g->cov_ptr || !g->cov_frag) return set_err(ctx, QH_ENOMEM, "allocation failed (coverage)");
     if (!scan_i32_to_i64(ctx, s, cnt, g->cov_ptr, n)) return set_err(ctx, QH_ENOMEM, "allocation failed (scan)");
     QH_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (n + 1), s));
     if (m > 0)

@@ -92,7 +92,7 @@ struct Graph {
   // SNP -> covering fragments (device), fragments ascending per SNP
   int64_t* cov_ptr = nullptr;
   int32_t* cov_frag = nullptr;
-  int8_t* cov_allele = nullptr;
+  int8_t* cov_allele = nullptr;  // READ mode (the votes); SNP graphs have none
   // edges (device), both directions
   int64_t nnz = 0;
   int64_t* row_ptr = nullptr;
