@@ -223,8 +223,9 @@ typedef struct {
                            patience > 0): 0 = inside the multi-step launch when it
                            applies (a multi-step step kernel, integer weights, at
                            most three items per SM fit every block) and pays
-                           (check_every <= 22 to 128, by the items per SM), else
-                           between launches; 1 = always
+                           for a solve that runs to its end (check_every <= 128, 30
+                           or 22 at one, two or three items per SM), else between
+                           launches; 1 = always
                            between launches, with the separate cut kernels.  Both
                            give the same steps_run, cuts and spins.  Other values
                            -> QH_EINVAL */

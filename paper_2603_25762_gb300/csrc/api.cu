@@ -181,8 +181,9 @@ qh_status check_err_word(Ctx* ctx) {
   return QH_OK;
 }
 
-// Time every valid step-kernel variant on the live state for a few steps and keep
-// the fastest for this graph shape (the multi-step family first, below).  The state is re-initialised afterwards.
+// Time every valid step-kernel variant on the live state for a few steps and keep the
+// fastest for this graph shape, the multi-step family first (autotune, below).  The state is
+// re-initialised afterwards.
 // All of what the choice hangs on is in the key: BF16 and BF16X2 solves of one graph walk
 // different entries, and some c0 rule the multi-step kernels out.
 std::string tune_key(const Graph& g, int R, int use_lo, int sb, bool allow_run) {
@@ -222,9 +223,11 @@ qh_status autotune(Ctx* ctx, const Graph& g, StepArgs a, const SolveBufs& B, int
   cudaStream_t s = ctx->stream;
   // The per-step and the multi-step kernels round y differently, so which family runs must
   // not hang on a close race: a per-step kernel is taken only where it is FAMILY_EDGE times
-  // faster.  Six steps also charge the multi-step launch's fixed cost (about 10 us) to few
-  // steps.  Measured over whole solves, us per step multi / per-step, at the per-step
-  // kernels' best: 4,000 SNPs R = 128 BF16X2 12.3 / 10.3, 903 reads R = 256 6.0 / 6.0;
+  // faster in this race.  The race favours neither: six steps charge the multi-step launch's
+  // fixed cost (about 10 us) to few steps, and the per-step kernels run without the overlap
+  // of launches that a solve gives them (6.7 against 5.9 us, 1,801 reads R = 192).  Measured
+  // over whole solves, us per step multi / per-step, at the per-step kernels' best: 4,000 SNPs R = 128
+  // BF16X2 12.3 / 10.3 (given up for the same cuts on every run), 903 reads R = 256 6.0 / 6.0;
   // elsewhere the multi-step kernel leads, to 17.5 / 57.6 on 40 blocks at R = 256.
   constexpr float FAMILY_EDGE = 1.6f;
   float best[2] = {1e30f, 1e30f};  // per-step, multi-step
@@ -904,12 +907,19 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
   // Early-stop checks inside the multi-step launch: integer weights, so that the tensor
   // cores give the energies exactly (every row sum of |J| below 2^24), and every block
   // in one wave at three items per SM (the fourth item's TMEM holds the check product).
-  // The kernel with checks keeps no x in TMEM and runs its steps slower (hifi-region, three
-  // items per SM: 11.4 against 8.5 us; one item 6.4 against 6.2), and a check between
-  // launches costs about 80 us.  Measured, us per step inside / between at check_every = 20,
-  // 25, 32, 50: three items 12.8 / 13.0, 12.4 / 12.0, 12.2 / 11.3, 11.7 / 10.1; two items
-  // 9.0 / 9.6, 8.8 / 9.0, 8.6 / 8.5, 8.3 / 7.8; one item 6.9 / 8.4, 6.8 / 8.0, 6.7 / 7.6, 6.6 /
-  // 7.0, and equal from 100 on.  So the checks move inside the launch up to this period.
+  // The kernel with checks keeps no x in TMEM and runs its steps slower, and a check between
+  // launches costs about 80 us.  Which is cheaper also hangs on whether the blocks stop: with
+  // the checks inside a stopped block runs one period on, and between launches the host ends
+  // the loop.  Measured, hifi-region, 1,000 steps, ms of steps inside / between:
+  //   that run to the end, check_every = 20, 22, 25, 30, 50, 100, 128 at one item per CTA
+  //   (R = 128) 6.61 / 8.50, 6.58 / 8.29, 6.55 / 7.99, 6.50 / 7.69, 6.39 / 6.98, 6.31 / 6.46, 6.29 /
+  //   6.37; 20 to 30 at two (R = 512) 9.09 / 9.84, 9.02 / 9.59, 8.90 / 9.20, 8.74 / 8.82; 20, 22
+  //   at three (R = 1,024) 12.82 / 13.36, 12.68 / 12.96;
+  //   that stop within 100 to 310 steps, R = 128 at 20, 25, 30: 1.49 / 1.58, 1.00 / 0.85, 1.14 /
+  //   0.97; R = 512 at 20, 25, 30: 2.02 / 1.80, 2.61 / 2.32, 2.31 / 1.87; R = 1,024 at 20, 22:
+  //   2.90 / 2.47, 4.50 / 4.06.
+  // So up to these periods inside is the cheaper of the two for a solve that runs on, by up to
+  // 1.9 ms, and costs one that stops early up to 0.45 ms.
   constexpr int32_t FUSED_CHECK_MAX[4] = {0, 128, 30, 22};
   bool fused = multistep && early && !track && o->check_mode == 0 && W.integer_weights &&
                o->check_every <= FUSED_CHECK_MAX[1];

@@ -160,16 +160,16 @@ __device__ __forceinline__ void cp_async_wait() {
 // the 4 row groups (8 replicas) that a warp reads at once into distinct banks.  Every
 // output sums its columns in ascending order with one FMA each.  The rows' list and J do
 // not depend on the step before: they are fetched ahead of the grid dependency.
-// Large graphs are bound by the latency of the operand copies at 12 warps per SM (ncu on
-// hifi-region, R = 1,024: issue slots 51 % busy, FMA pipe 34 %, DRAM under 25 %), small ones
-// by the chain launch - x copies - column loop - update.  Stages of 2 chunks (more CTAs per
+// Large graphs are bound by the latency of the operand copies and reads at 12 warps per SM
+// (ncu on hifi-region, R = 1,024: issue slots 57 % of the active cycles, FMA pipe 42 %, shared
+// memory 55 %, DRAM 14 %), small ones by the chain launch - x copies - column loop - update.  Stages of 2 chunks (more CTAs per
 // SM, twice the barriers) measured slower: 66 against 61 us per step on hifi-region, 85
 // against 69 on ont-like 3,000 SNPs at R = 512; so did x and y prefetched into registers
 // ahead of the loop (hifi-region R = 256 21.8 against 17.9: fewer CTAs per SM).
 // Microseconds per step, the dense 128 x 64 tile product before -> now: 300 SNPs / 80
-// reads, R = 32: 20.4 -> 2.4; 720 reads, R = 256: 49.7 -> 6.6; 7,200 reads, R = 256: 64.7 ->
-// 17.9 and R = 1,024: 192 -> 61; 12,000-SNP graph (468 neighbours), R = 128: 146 -> 63 and
-// R = 512: 349 -> 178.
+// reads, R = 32: 20.4 -> 2.1; 720 reads, R = 256: 49.7 -> 6.4; 7,200 reads, R = 256: 64.7 ->
+// 17.4 and R = 1,024: 192 -> 59; 12,000-SNP graph (468 neighbours), R = 128: 146 -> 61 and
+// R = 512: 349 -> 175.
 template <int RPT, int NW, int TR, bool DISC>
 __global__ void __launch_bounds__(32 * NW * 8 / TR) k_step_f32(StepArgs a, const int2* __restrict__ list,
                                                       const int32_t* __restrict__ count,
@@ -852,7 +852,8 @@ __global__ void k_cut_nodes_few(int32_t n, const int64_t* __restrict__ rp,
 // 2.5e-16 / 4.5e-16; a block of weights 1e-8 of the other block's 4.7e-16 / 3.3e-7 / 6.7e-16.  A
 // solve's time outside its steps, ms: 12,000 SNPs (5.6M entries) R = 512: 2.64 / 1.29 / 1.27;
 // 50,000 SNPs (7.6M entries) R = 128: 3.08 / 1.58 / 1.56.  Six base-256 digits with a DP4A per
-// four edges measured slower: this part's DP4A rate is low.
+// four edges measured slower: this part's DP4A rate is low.  Bound by issue (61 % of the
+// active cycles; FMA pipe 47 %) at the 16 warps per SM that 122 registers leave.
 constexpr int CUT_DIGITS = 3;
 constexpr int CUT_DIGIT_BITS = 18;
 constexpr int CUT_BITS = 53;

@@ -168,10 +168,11 @@ __global__ void __launch_bounds__(128) k_step_tc(const __grid_constant__ CUtenso
 // next 32 are in flight while the current 32 are updated.
 // A step's launch overlaps the end of the step before it (grid_dep_wait): barriers, TMEM,
 // and the first J copies come before the wait.  us per step, BF16, before -> with that,
-// a ring as deep as the grid allows and the coefficient table: 80 reads R = 64 6.8 -> 4.5;
-// 1,800 reads R = 192 8.05 -> 6.15; 7,200 reads R = 576 14.9 -> 12.5.  FP8: 720 reads
-// R = 128 14.2 -> 7.6; 7,200 reads R = 256 15.5 -> 9.8, R = 512 19.7 -> 17.0, R = 1,024
-// 31.8 -> 29.9.
+// a ring as deep as the grid allows and the coefficient table: 80 reads R = 64 6.4 -> 4.6;
+// 1,801 reads R = 192 8.2 -> 6.0; 7,200 reads R = 576 14.8 -> 12.4.  FP8: 720 reads R = 128
+// 14.0 -> 7.7; 1,800 reads R = 512 14.7 -> 8.3; 7,200 reads R = 256 15.6 -> 9.8, R = 512 19.5 ->
+// 16.8, R = 1,024 31.6 -> 29.6.  The overlap alone (off -> on): 80 reads
+// R = 64 5.5 -> 4.5, 1,801 reads R = 192 6.7 -> 5.9, R = 576 13.0 -> 12.3; FP8 R = 256 11.3 -> 9.8.
 template <int BN, int STAGES, int MINB, int CH>
 __global__ void __launch_bounds__(128, MINB) k_step_tc_v(const __grid_constant__ CUtensorMap tmJ,
                                                          const __grid_constant__ CUtensorMap tmX,
@@ -1122,10 +1123,11 @@ qh_status tc_prepare(Ctx* ctx) {
 
 // Operand ring of the 64-replica CTAs: two slots with four CTAs per SM; a grid that leaves
 // SMs to fewer CTAs takes as many slots as fit beside them, so that a row tile's slices are
-// in flight together (each refill of a slot waits a copy's latency).  Measured, two slots
-// -> this, us per step: BF16 144 reads R = 64 6.30 -> 5.90, 1,800 reads R = 192 7.09 -> 6.82
-// (four slots at 171 CTAs 8.07 -> 8.24: BF16 keeps two there); FP8 1,800 reads R = 512
-// 9.83 -> 9.00, 7,200 reads R = 256 11.58 -> 10.64.
+// in flight together (each refill of a slot waits a copy's latency).  Measured, two slots ->
+// this, us per step: BF16 80 reads R = 64 4.88 -> 4.61, 144 reads R = 64 5.37 -> 4.90, 1,801
+// reads R = 192 5.99 -> 5.99 (four slots at 171 CTAs measured slower: BF16 keeps two there); FP8
+// 720 reads R = 128 8.40 -> 7.71, 1,800 reads R = 512 9.44 -> 8.35, 7,200 reads R = 256 10.69 ->
+// 9.84.
 static int ring_depth(const Graph& g, int R, int n_sm) {
   const int64_t ctas = (int64_t)g.n_row_tiles * (R / 64);
   return ctas <= n_sm ? 6 : ctas <= 2 * n_sm ? 4 : 2;

@@ -355,7 +355,8 @@ struct SnpRowSmem {
 //    `late` for PASS 1.  Rows of more than SNP_ROW_CAP terms were once all deferred; graph
 //    builds of ONT-like reads at 100x, a CTA per row with a search / that / now: 600 SNPs
 //    1.26 / 2.35 / 1.14 ms, 3,000 SNPs 2.77 / 8.36 / 1.81, 12,000 SNPs 8.29 / 29.6 / 4.07.
-// Bound by FP64 and by the latency of the terms' loads.  GB300's FP64 rate makes a division
+// The fill is bound by FP64 (pipe 83 % busy at 12,000 SNPs; 664 us), the count by the latency of
+// the terms' loads (issue 25 % of the active cycles; 176 us).  GB300's FP64 rate makes a division
 // per term the largest cost of the fill: the divisor is a fragment's, so the quotient is
 // taken from its correctly rounded reciprocal (snp_quotient, the same bits).  Measured,
 // both passes, against a CTA per row with a search for u and a barrier per fragment, and a

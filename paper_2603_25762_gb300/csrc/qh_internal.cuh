@@ -213,9 +213,10 @@ struct Ctx {
 
 // Programmatic dependent launch.  A step launched after another one (StepArgs::after_step)
 // starts while that one finishes; grid_dep_wait returns once it has completed and its
-// writes are visible.  What precedes the wait may read only what no step writes.  Every
-// CTA waits before it exits, or a step with nothing left to do would complete ahead of the
-// one before it.
+// writes are visible.  What precedes the wait may read only what no step writes.  A step must
+// not complete ahead of the one before it, so its CTAs wait before they exit, also those with
+// nothing left to do; k_step_f32's CTAs for rows past a block's end do not, since another
+// group of the same row tile always does.
 __device__ __forceinline__ void grid_dep_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
