@@ -823,9 +823,14 @@ static qh_status solve_impl(qh_ctx* h, const qh_graph* gh, const qh_bsb_opts* o,
     addi(G.n_nodes); addi(G.n_pad); addi(G.n_blocks); addi(G.n_row_tiles); addi(G.n_tiles);
     addi(G.n_tiles_hi); addi(G.has_lo); addi(G.csr_mode); addi(G.integer_weights);
     addi(G.max_tiles_per_row); addi(G.pnnz); addi(G.nnz);
+    // the cuts of the checks: their grids go by the chunks and the largest block, the kernel of
+    // real weights by the range of the weights
+    addi(G.n_cut_chunks); addi(*std::max_element(G.h_block_size.begin(), G.h_block_size.end()));
+    addi(cut_fixed_point(G) ? 1 : 0);
     addi(f8.n_slices); add(f8_jh); add(f8_jl);
     skey += std::to_string(f8_s) + "|";
     for (const void* p : {(const void*)G.rt, (const void*)G.tile_col, (const void*)G.kslice,
+                          (const void*)G.cut_rt,
                           (const void*)W.tile_bf16,
                           (const void*)W.tile_f32, (const void*)G.prow_ptr, (const void*)G.pcol,
                           (const void*)W.pval, (const void*)W.band, (const void*)W.rval,

@@ -1605,11 +1605,10 @@ void launch_cut(cudaStream_t s, const Graph& g, int32_t R, const int8_t* signs_t
   int32_t max_n = 1;
   for (int32_t b = 0; b < g.n_blocks; ++b) max_n = std::max(max_n, g.h_block_size[b]);
   const unsigned warps = nblk((int64_t)g.n_nodes * 32);
-  const double m = g.max_abs_w;
   if (g.integer_weights) {
     k_cut_nodes<<<::qh::counted(warps), 256, 0, s>>>(
         g.n_nodes, g.row_ptr, g.col, w, g.block_of, g.pad_index, signs_t, R, per, node_val, active);
-  } else if (R <= 4 || !(m > 1e-250 && m < 1e250)) {
+  } else if (R <= 4 || !cut_fixed_point(g)) {
     const dim3 grid(warps, (unsigned)((R + 3) / 4));
     k_cut_nodes_few<<<::qh::counted(grid), 256, 0, s>>>(
         g.n_nodes, g.row_ptr, g.col, w, g.block_of, g.pad_index, signs_t, R, node_val, active);

@@ -422,6 +422,10 @@ qh_status launch_band_mma(Ctx* ctx, const Graph& g, const StepArgs& a, const __n
                           const __nv_bfloat16* xh_vm, float* z);
 void launch_transpose(cudaStream_t s, const float* in, float* out, int64_t rows, int64_t cols);
 void launch_signs(cudaStream_t s, const Graph& g, int32_t R, const float* x, int8_t* signs_t);
+// Can the cuts of real weights be summed in fixed point?
+inline bool cut_fixed_point(const Graph& g) {
+  return g.max_abs_w > 1e-250 && g.max_abs_w < 1e250;  // false for NaN
+}
 void launch_cut(cudaStream_t s, const Graph& g, int32_t R, const int8_t* signs_t, const double* w,
                 const double* sum_w, double* node_val, double* cuts, const int32_t* active);
 void launch_pick_best(cudaStream_t s, int32_t n_blocks, int32_t R, const double* cuts,
